@@ -12,14 +12,14 @@
 //   P   = exp2(S * scale*log2e - m)  -> bf16, written over S in tensor memory
 //   O  += P V_j                      A = P from tensor memory, B = V_j MN-major
 //
-// Three kernels.  tc_fwd_pair_kernel (d = 64, 128; no mask or causal, calls with enough tiles): two
-// query tiles per CTA, a softmax warpgroup each, a thread holds a whole row of scores.
-// tc_fwd_rows_kernel (d = 64, 128; every other call): one query tile, the two softmax warpgroups take
-// alternate key tiles, each with an S buffer and a partial accumulator of its own, and the two partial
-// softmaxes are merged in the epilogue.  tc_fwd_kernel (d = 256; key tiles of 64): both warpgroups
+// Four kernels.  tc_fwd_flow_kernel (d = 64, 128): a thread holds a whole row of scores, S has buffers of its own that
+// are free as soon as it has been copied out.  PAIR (no mask or causal, calls with enough tiles): two query tiles per CTA, a
+// softmax warpgroup each.  Otherwise one query tile, the two softmax warpgroups take alternate key tiles, each with a partial
+// accumulator of its own, and the two partial softmaxes are merged in the epilogue.  tc_fwd_pair_kernel and
+// tc_fwd_rows_kernel: the same two shapes for calls whose P must not be rounded to one bf16 term; its second term takes the
+// tensor memory that the S buffers would need.  tc_fwd_kernel (d = 256; key tiles of 64): both warpgroups
 // split the columns of every tile and exchange row maxima through shared memory, one accumulator of
-// 256 columns.  Each has one MMA-issuing thread and one TMA-producing thread; the roles and the
-// tensor-memory layout are described at each kernel.
+// 256 columns.  The roles and the tensor-memory layout are described at each kernel.
 #include <type_traits>
 
 #include "attn_internal.h"
@@ -388,36 +388,48 @@ __device__ __forceinline__ float row_max(const uint32_t (&v)[128])
         for (int e = 0; e < 8; ++e) m[e] = max3(m[e], __uint_as_float(v[c + e]), __uint_as_float(v[c + e + 8]));
     return fmaxf(max3(max3(m[0], m[1], m[2]), m[3], m[4]), max3(m[5], m[6], m[7]));
 }
-// P = exp2(v * sl2 + noff) as bf16 pairs over the first 64 columns of S (every thread overwrites only its own lane, whose
-// scores it already holds), SPLIT: what that loses over the other 64; returns the sum of the row of P before rounding
+// x = exp2(v * s + n) of two scores; both are added to `sum`
+__device__ __forceinline__ void exp_pair(uint32_t v0, uint32_t v1, uint64_t s2, uint64_t n2, uint64_t &sum, float &x0, float &x1)
+{
+    uint64_t x;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(v0), "r"(v1));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(x) : "l"(x), "l"(s2), "l"(n2));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(x1) : "l"(x));
+    x0 = ex2_fast_f(x0);
+    x1 = ex2_fast_f(x1);
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(x0), "f"(x1));
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(sum) : "l"(sum), "l"(x));
+}
+__device__ __forceinline__ float sum_of(const uint64_t (&sum)[4])
+{
+    float a[8];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) asm("mov.b64 {%0, %1}, %2;" : "=f"(a[2 * e]), "=f"(a[2 * e + 1]) : "l"(sum[e]));
+    return ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+}
+// P = exp2(v * sl2 + noff) as two bf16 terms: pairs of leading terms over the first 64 columns of S (every thread overwrites
+// only its own lane, whose scores it already holds), what they lose over the other 64; returns the sum of the row of P before
+// rounding.
 //
 // The first 96 keys of P are handed over (`early`, one arrival per warp) as soon as they are stored: the tensor core, idle by
 // then, forms their part of O += P V under the exponentials of the rest.
-template <bool SPLIT>
-__device__ __forceinline__ float exp_row(const uint32_t (&v)[128], float sl2, float noff, uint32_t to, uint64_t *early, uint64_t *last, int lane)
+__device__ __forceinline__ float exp_row_split(const uint32_t (&v)[128], float sl2, float noff, uint32_t to, uint64_t *early, uint64_t *last, int lane)
 {
     uint64_t s2, n2, sum[4] = {0ull, 0ull, 0ull, 0ull};
     asm("mov.b64 %0, {%1, %1};" : "=l"(s2) : "f"(sl2));
     asm("mov.b64 %0, {%1, %1};" : "=l"(n2) : "f"(noff));
 #pragma unroll
     for (int c = 0; c < 128; c += 32) {
-        uint32_t pp[16], pl[SPLIT ? 16 : 1];
+        uint32_t pp[16], pl[16];
 #pragma unroll
         for (int e = 0; e < 32; e += 2) {
-            uint64_t x;
             float x0, x1;
-            asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(v[c + e]), "r"(v[c + e + 1]));
-            asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(x) : "l"(x), "l"(s2), "l"(n2));
-            asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(x1) : "l"(x));
-            x0 = ex2_fast_f(x0);
-            x1 = ex2_fast_f(x1);
-            asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(x0), "f"(x1));
-            asm("add.rn.f32x2 %0, %1, %2;" : "=l"(sum[(e / 2) & 3]) : "l"(sum[(e / 2) & 3]), "l"(x));
+            exp_pair(v[c + e], v[c + e + 1], s2, n2, sum[(e / 2) & 3], x0, x1);
             pp[e / 2] = pack_bf16(x0, x1);
-            if constexpr (SPLIT) pl[e / 2] = pack_bf16_rest(x0, x1, pp[e / 2]);
+            pl[e / 2] = pack_bf16_rest(x0, x1, pp[e / 2]);
         }
         tmem_st16(to + c / 2, pp);
-        if constexpr (SPLIT) tmem_st16(to + 64 + c / 2, pl);
+        tmem_st16(to + 64 + c / 2, pl);
         if (c >= 64) {
             tmem_wait_st();
             tcgen05_fence_before();
@@ -425,14 +437,11 @@ __device__ __forceinline__ float exp_row(const uint32_t (&v)[128], float sl2, fl
             if (lane == 0) mbar_arrive(c == 64 ? early : last);
         }
     }
-    float a[8];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) asm("mov.b64 {%0, %1}, %2;" : "=f"(a[2 * e]), "=f"(a[2 * e + 1]) : "l"(sum[e]));
-    return ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+    return sum_of(sum);
 }
 
 // ---------------------------------------------------------------------------------------
-// d = 64 and 128: the two softmax warpgroups take ALTERNATE key tiles.  Warpgroup w owns the S buffer w and
+// d = 64 and 128, P as two bf16 terms: the two softmax warpgroups take ALTERNATE key tiles.  Warpgroup w owns the S buffer w and
 // an accumulator O_w of its own (tensor memory: S_0 128, S_1 128, O_0 d, O_1 d columns), and a thread owns a
 // whole row of its tile: the row maximum needs no exchange, and while one warpgroup is loading, taking the
 // maximum or storing P, the other one keeps the MUFU pipe busy with its exponentials.  Each warpgroup runs its
@@ -442,7 +451,6 @@ __device__ __forceinline__ float exp_row(const uint32_t (&v)[128], float sl2, fl
 // The issuing thread waits for P alone and commits S alone (why: tc_fwd_pair_kernel).  K(k+2) and V(k+2) report to the barrier of
 // P(k), which it waits for before S(k+2); the loading thread takes S(k) complete as the release of their stages: K(k+2) goes
 // where K(k) was, and O += P(k-2) V was issued before S(k), so V needs four stages.
-// Block-sparse forward, 32 heads, n = 32768, d = 128, 10 %: 2159 -> 2086 us; one head, n = 16384, causal: 138 -> 133.
 template <int HD>
 struct RowsCfg {
     static constexpr int NK = 2, NV = 4;
@@ -464,8 +472,8 @@ enum { F2_Q = 0, F2_K1 = 1, F2_V01 = 2, F2_S = 3, F2_PE = 5, F2_P = 7, F2_O = 9 
 // the softmax warpgroups take them (256 x 224 + 128 x 40 = 62,464 of the 384 x 168 = 64,512 the block holds), so
 // that a thread can keep its whole row of 128 scores.
 constexpr int kThreadsRows = kSoftmaxThreads + 128;
-// SPLIT: P enters its product as two bf16 terms (columns 0-63 and 64-127 of S), for calls whose P must not be rounded to one
-template <int HD, bool FINE, bool SPLIT>
+// P enters its product as two bf16 terms (columns 0-63 and 64-127 of S).
+template <int HD, bool FINE>
 __global__ void __launch_bounds__(kThreadsRows, 1)
 tc_fwd_rows_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CUtensorMap mK,
                    const __grid_constant__ CUtensorMap mV, const FwdArgs a)
@@ -590,7 +598,7 @@ tc_fwd_rows_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                         tcgen05_fence_after();
                     }
                     mma_ts_lo(tO, tP + kk * 8, mV_ + kk * 128, idesc_o, (k > 1) || (kk > 0));
-                    if constexpr (SPLIT) mma_ts_lo(tO, tP + 64 + kk * 8, mV_ + kk * 128, idesc_o, 1);
+                    mma_ts_lo(tO, tP + 64 + kk * 8, mV_ + kk * 128, idesc_o, 1);
                 }
                 // the products execute in issue order: S(k+2) overwrites buffer b after P(k) has been consumed, and
                 // its completion tells warpgroup b that O_b holds the product of tile k as well
@@ -675,7 +683,7 @@ tc_fwd_rows_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
             const float noff = m_ref == -INFINITY ? 0.f : -m_ref;
             // P = exp2(S * scale * log2e - m_ref) as bf16 pairs over the first 64 columns of S (every thread
             // overwrites only its own lane, whose scores it already holds)
-            l_run += exp_row<SPLIT>(v, sl2, noff, T_S + lane_addr, &bars[F2_PE + w], &bars[F2_P + w], lane);
+            l_run += exp_row_split(v, sl2, noff, T_S + lane_addr, &bars[F2_PE + w], &bars[F2_P + w], lane);
             ++cnt;
         }
         // ------------------------------------------------------------ epilogue: merge the two partial softmaxes
@@ -723,7 +731,7 @@ tc_fwd_rows_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
 }
 
 // ---------------------------------------------------------------------------------------
-// d = 64 and 128, masks without lists: 256 queries per CTA.  Warpgroup w owns the query tile w and walks every key tile.  Tensor
+// The same with 256 queries per CTA, for masks without lists.  Warpgroup w owns the query tile w and walks every key tile.  Tensor
 // memory as above (S_0, S_1, O_0, O_1); nothing is merged at the end.  Issue order: S_0(0), S_1(0), then per key tile k:
 // O_0 += P_0 V, S_0(k+1), O_1 += P_1 V, S_1(k+1).
 //
@@ -734,17 +742,6 @@ tc_fwd_rows_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
 // anyway before S_0(k+1); the loading thread takes S_0(k) complete as the release of the stages they go to: S_1(k-1) and
 // O_1 += P_1(k-2) V were issued before it, so two K stages and three V stages suffice.  S_0(k) is the newest completion its
 // barrier can have there, so the parity wait cannot be a phase behind.
-// 32 heads, n = 8192, d = 128, causal: 489 us (single tiles, same launch order: 555); 32 heads, n = 4096: 148 (171); 24 heads,
-// n = 3000, d = 64, no mask: 97 (109).  Bound now by the chain of one warpgroup: scores out of tensor memory, maximum,
-// exponentials (1,330 cycles, of which the MUFU needs 1,024), P back, its two products.
-//
-// A row's largest probabilities are what the rounding of P to bf16 costs most, and the one that the reference was taken from is
-// exactly 1.  Two partial softmaxes a row (above) have two such entries, one softmax has one, and its O is one per cent further
-// from 64 bits.  So the first kExactTiles tiles after the first one move the reference (up, by less than one unit beyond what the
-// maximum asks for) to where their largest entry is a power of two.  Error of O, 32 heads, n = 4096, d = 128, causal, against
-// the two partial softmaxes': 1.010 times without, 0.994 with two exact tiles (1.000 with one, emulated).  It costs
-// two rescalings of O per query tile (32 heads, n = 8192, d = 128, causal: 574 -> 584 us with 16 columns at a time, 573 with 32).
-constexpr unsigned kExactTiles = 2;
 template <int HD>
 struct PairCfg {
     static constexpr int NK = 2, NV = 3;                       // stages
@@ -760,7 +757,7 @@ struct PairCfg {
 };
 enum { F3_Q = 0, F3_V0 = 1, F3_S = 2, F3_PE = 4, F3_P = 6, F3_O = 8 };
 
-template <int HD, bool SPLIT>
+template <int HD>
 __global__ void __launch_bounds__(kThreadsRows, 1)
 tc_fwd_pair_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CUtensorMap mK,
                    const __grid_constant__ CUtensorMap mV, const FwdArgs a)
@@ -867,7 +864,7 @@ tc_fwd_pair_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                         tcgen05_fence_after();
                     }
                     mma_ts_lo(tO, tP + kk * 8, mV_ + kk * 128, idesc_o, (k > 0) || (kk > 0));
-                    if constexpr (SPLIT) mma_ts_lo(tO, tP + 64 + kk * 8, mV_ + kk * 128, idesc_o, 1);
+                    mma_ts_lo(tO, tP + 64 + kk * 8, mV_ + kk * 128, idesc_o, 1);
                 }
             };
             mbar_wait(&bars[F3_Q], 0, ab);
@@ -914,14 +911,8 @@ tc_fwd_pair_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                     if (e >= keep) v[e] = 0xff800000u;   // -inf
             }
             const float m_tile = row_max(v) * sl2;   // scale > 0: the maximum commutes with it
-            bool need = m_tile > m_ref + kRescaleThreshold || (m_ref == -INFINITY && m_tile != -INFINITY);
-            float m_new = need ? fmaxf(m_ref, m_tile) : m_ref;
-            if (!SPLIT && k - 1u < kExactTiles && m_ref != -INFINITY && m_tile != -INFINITY) {
-                // the next reference from which the tile's maximum is a whole number of powers of two away, by less than one
-                // unit up also where the sum is rounded (references of 2^24 and more)
-                m_new = m_tile > m_ref ? m_tile : fminf(fmaxf(m_tile + ceilf(m_ref - m_tile), m_ref), m_ref + 1.f);
-                need = true;
-            }
+            const bool need = m_tile > m_ref + kRescaleThreshold || (m_ref == -INFINITY && m_tile != -INFINITY);
+            const float m_new = need ? fmaxf(m_ref, m_tile) : m_ref;
             if (__any_sync(0xffffffffu, need)) {
                 const float alpha = (need && m_ref != -INFINITY) ? ex2_fast_f(m_ref - m_new) : 1.f;
                 if (k > 0) {   // O_w += P V of the previous tile was issued before this tile's S_w: it has landed
@@ -939,7 +930,7 @@ tc_fwd_pair_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                 m_ref = m_new;
             }
             const float noff = m_ref == -INFINITY ? 0.f : -m_ref;
-            l_run += exp_row<SPLIT>(v, sl2, noff, T_S + lane_addr, &bars[F3_PE + w], &bars[F3_P + w], lane);
+            l_run += exp_row_split(v, sl2, noff, T_S + lane_addr, &bars[F3_PE + w], &bars[F3_P + w], lane);
         }
         // ------------------------------------------------------------ epilogue
         if (mine > 0) {
@@ -965,6 +956,404 @@ tc_fwd_pair_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                 }
             }
             if (ig < n) a.LSE[(size_t)bh * n + ig] = row_lse(m_ref, l_run);
+        }
+    }
+    tcgen05_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tm, 512);
+}
+
+// ---------------------------------------------------------------------------------------
+// d = 64 and 128, P as one bf16 term.  PAIR: two query tiles, warpgroup w owns tile w and walks every key tile; otherwise one
+// query tile whose key tiles the warpgroups take in turn (as in tc_fwd_rows_kernel, merged at the end).
+//
+// S = Q K^T goes into a buffer X that no P is written to (tensor memory, d = 128: X 128 columns, P_0, P_1 64 each, O_0, O_1 128
+// each; d = 64: two buffers X).  The warpgroup copies its row into registers and gives X back, so that the next S is formed
+// under its exponentials, and P goes to columns of its own, free once the product before has read them.  With P over S (the
+// kernels above) S of the next tile waits for P and its product: a chain of 3,290 cycles a tile and warpgroup, period of
+// two tiles 3,800; here a warpgroup's chain is 2,100 (wait seen 130, copy and maximum 550, exponentials 1,420) and the
+// period 3,030.  Bound now, d = 128: the one X (S 690, seen and copied 400, given back and seen 150 to 300, for each of two
+// warpgroups); d = 64: the warpgroup's own chain, the MUFU pipe 70 % busy.
+// Two issuing threads: A forms S, B adds P V; nothing orders their products but the barriers of X and P.
+// 32 heads, n = 8192, d = 128, causal: 566 -> 525 us; block-sparse, 32 heads, n = 32768, 10 %: 1844 -> 1794 us; 24 heads,
+// n = 3000, d = 64, one query tile: 109 -> 105 us; 64 heads, n = 2048, d = 64: 127 us both.
+//
+// A row's largest probabilities are what the rounding of P to bf16 costs most, and the one that the reference was taken from is
+// exactly 1.  Two partial softmaxes a row (one query tile) have two such entries, one softmax has one, and its O is one per cent further
+// from 64 bits.  So the first kExactTiles tiles after the first one move the reference (up, by less than one unit beyond what the
+// maximum asks for) to where their largest entry is a power of two.  Error of O, 32 heads, n = 4096, d = 128, causal, against
+// the two partial softmaxes': 1.010 times without, 0.994 with two exact tiles (1.000 with one, emulated).  It costs
+// two rescalings of O per query tile (32 heads, n = 8192, d = 128, causal: 574 -> 584 us with 16 columns at a time, 573 with 32).
+constexpr unsigned kExactTiles = 2;   // PAIR
+template <int HD, bool PAIR>
+struct FlowCfg {
+    static constexpr int NQ = PAIR ? 2 : 1;                    // query tiles
+    static constexpr int NK = PAIR ? 2 : 3, NV = 3;            // stages
+    static constexpr int NX = HD == 64 ? 2 : 1;                // S buffers
+    static constexpr uint32_t kSlab = 128 * 128, kSlabs = HD / 64, kTile = kSlabs * kSlab;
+    static constexpr uint32_t oQ = 0;
+    static constexpr uint32_t oK = oQ + NQ * kTile;
+    static constexpr uint32_t oV = oK + NK * kTile;
+    static constexpr uint32_t oX = oV + NV * kTile;            // merge of the two partial softmaxes (one query tile)
+    static constexpr uint32_t oBar = oX + (PAIR ? 0 : 4 * 128 * 4);
+    static constexpr uint32_t oMisc = oBar + 24 * 8;
+    static constexpr uint32_t kUsed = oMisc + 64;
+    static_assert(kUsed <= 227 * 1024, "shared memory budget");
+    static constexpr uint32_t kBytes = kUsed < 117 * 1024 ? 117 * 1024 : kUsed;   // one CTA per SM: all of tensor memory
+    static constexpr uint32_t tP = NX * 128, tO = tP + 128;    // tensor-memory columns
+    static_assert(tO + 2 * HD == 512, "tensor memory");
+};
+enum { F4_Q = 0, F4_KF = 2, F4_KE = 5, F4_VF = 8, F4_VE = 11, F4_S = 14, F4_XF = 16, F4_PE = 18, F4_P = 20, F4_O = 22 };
+
+// P = exp2(v * sl2 + noff) as bf16 pairs into columns of its own; returns the sum of the row of P before rounding.  `free` waits
+// until the columns may be written, by when 64 keys are ready.  The first 96 keys are handed over (`early`, one arrival per
+// warp) as soon as they are stored: their part of O += P V is formed under the exponentials of the rest.
+template <typename Free>
+__device__ __forceinline__ float exp_row(const uint32_t (&v)[128], float sl2, float noff, uint32_t to, uint64_t *early, uint64_t *last, int lane, Free &&free)
+{
+    uint64_t s2, n2, sum[4] = {0ull, 0ull, 0ull, 0ull};
+    asm("mov.b64 %0, {%1, %1};" : "=l"(s2) : "f"(sl2));
+    asm("mov.b64 %0, {%1, %1};" : "=l"(n2) : "f"(noff));
+    auto pair = [&](int c) {
+        float x0, x1;
+        exp_pair(v[c], v[c + 1], s2, n2, sum[(c / 2) & 3], x0, x1);
+        return pack_bf16(x0, x1);
+    };
+    {
+        uint32_t pp[32];
+#pragma unroll
+        for (int e = 0; e < 32; ++e) pp[e] = pair(2 * e);
+        free();
+        tmem_st32(to, pp);
+    }
+#pragma unroll
+    for (int c = 64; c < 128; c += 32) {
+        uint32_t pp[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) pp[e] = pair(c + 2 * e);
+        tmem_st16(to + c / 2, pp);
+        tmem_wait_st();
+        tcgen05_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(c == 64 ? early : last);
+    }
+    return sum_of(sum);
+}
+
+template <int HD, bool PAIR, bool FINE>
+__global__ void __launch_bounds__(kThreadsRows, 1)
+tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CUtensorMap mK,
+                   const __grid_constant__ CUtensorMap mV, const FwdArgs a)
+{
+    using C = FlowCfg<HD, PAIR>;
+    constexpr int TKF = 128, NK = C::NK, NV = C::NV, NX = C::NX;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + C::oBar);
+    uint32_t *tmem_base_s = reinterpret_cast<uint32_t *>(smem + C::oMisc);
+    volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(smem + C::oMisc + 4);
+    float *xm = reinterpret_cast<float *>(smem + C::oX);   // !PAIR: [2 warpgroups][128 rows] reference maxima
+    float *xl = xm + 256;                                  // [2][128] row sums
+    const Abort ab{abort_flag, a.status};
+
+    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+    const int n = a.n;
+    constexpr int QROWS = C::NQ * TQ;
+    const int i0 = ((n + QROWS - 1) / QROWS - 1 - (int)blockIdx.x / a.group) * QROWS;   // heaviest causal tiles first
+    const long bh = (long)blockIdx.y * a.group + blockIdx.x % a.group;
+    const bool causal = mask_is_causal(a.mask_kind);
+
+    if ((smem_u32(smem) & 1023u) != 0) {
+        chain_wait();
+        if (tid == 0) atomicExch(a.status, 9u);
+        return;
+    }
+    if (tid == 0) {
+        *abort_flag = 0;
+        for (int b = 0; b < 24; ++b) {
+            const bool warps = b >= F4_XF && b < F4_O;   // XF, PE, P: the four warps of a warpgroup
+            mbar_init(&bars[b], warps ? 4 : 1);
+        }
+        fence_barrier_init();
+        prefetch_tensormap(&mQ); prefetch_tensormap(&mK); prefetch_tensormap(&mV);
+    }
+    chain_wait();
+    if (warp == 0) tmem_alloc(tmem_base_s, 512);
+    tcgen05_fence_before();
+    __syncthreads();
+    tcgen05_fence_after();
+    chain_release();
+    if (tid == 0 && blockIdx.x == 0 && blockIdx.y == 0) *a.status = 0u;
+    const uint32_t tm = *tmem_base_s;
+
+    // Items in the order in which their S is formed.  PAIR: (query tile w, key tile k) = (0, 0), (1, 0), (0, 1), ..., then what one
+    // query tile has left; otherwise item k is key tile k of warpgroup k % 2.
+    const KeyIter<TKF> iter(a, PAIR ? 0 : i0 / TQ, bh);
+    int n0, n1;   // items of the warpgroups
+    if constexpr (PAIR) {
+        auto count = [&](int w) {   // key tiles of query tile w (the second one may lie beyond n)
+            const int first = i0 + w * TQ;
+            if (first >= n) return 0;
+            return causal ? (min(first + TQ, n) - 1) / TKF + 1 : (n + TKF - 1) / TKF;
+        };
+        n0 = count(0), n1 = count(1);
+    } else {
+        int kept = 0;
+        for (int idx = 0; idx < iter.raw; ++idx) kept += iter.tile(idx) >= 0;
+        n0 = (kept + 1) / 2, n1 = kept / 2;
+    }
+    const int both = min(n0, n1), items = n0 + n1, tiles = PAIR ? max(n0, n1) : items;
+    auto item_of = [&](int w, int c) { return c < both ? 2 * c + w : both + c; };             // c-th item of warpgroup w
+    auto group_of = [&](int i) { return i < 2 * both ? i & 1 : n0 > n1 ? 0 : 1; };
+    auto nth_of = [&](int i) { return i < 2 * both ? i >> 1 : i - both; };                    // its index there
+    auto tile_of = [&](int i) { return PAIR ? nth_of(i) : i; };
+    auto tile_ends = [&](int i) { return !PAIR || i >= 2 * both || (i & 1) != 0; };           // nothing after item i uses its key tile
+
+    if (warp >= 8) {
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+      if (warp == 9) {
+        // ------------------------------------------------------------ TMA producer
+        if (lane == 0) {
+            auto load = [&](uint32_t to, const CUtensorMap *m, uint64_t *bar, int row) {
+#pragma unroll
+                for (uint32_t sl = 0; sl < C::kSlabs; ++sl) tma_load_3d(smem + to + sl * C::kSlab, m, bar, sl * 64, row, (int)bh);
+            };
+            mbar_expect_tx(&bars[F4_Q], C::kTile);
+            load(C::oQ, &mQ, &bars[F4_Q], i0);
+            int k = 0;
+            for (int idx = 0; idx < (PAIR ? tiles : iter.raw); ++idx) {
+                const int jt = PAIR ? idx : iter.tile(idx);
+                if (jt < 0) continue;
+                const int sk = k % NK, sv = k % NV;
+                if (k >= NK) mbar_wait(&bars[F4_KE + sk], (k / NK - 1) & 1, ab);
+                mbar_expect_tx(&bars[F4_KF + sk], C::kTile);
+                load(C::oK + sk * C::kTile, &mK, &bars[F4_KF + sk], jt * TKF);
+                if (PAIR && k == 0 && n1 > 0) {
+                    mbar_expect_tx(&bars[F4_Q + 1], C::kTile);
+                    load(C::oQ + C::kTile, &mQ, &bars[F4_Q + 1], i0 + TQ);
+                }
+                if (k >= NV) mbar_wait(&bars[F4_VE + sv], (k / NV - 1) & 1, ab);
+                mbar_expect_tx(&bars[F4_VF + sv], C::kTile);
+                load(C::oV + sv * C::kTile, &mV, &bars[F4_VF + sv], jt * TKF);
+                ++k;
+            }
+            if (items == 0) mbar_wait(&bars[F4_Q], 0, ab);   // let the Q load land before exit
+        }
+      } else if (warp == 8) {
+        // ------------------------------------------------------------ MMA issuer A: S = Q K^T
+        if (lane == 0) {
+            constexpr uint32_t idesc_s = idesc_bf16(128, TKF, 0, 0);
+            const uint32_t kQ = desc_lo_kmajor(smem_u32(smem + C::oQ));
+            for (int i = 0; i < items; ++i) {
+                const int w = group_of(i), k = tile_of(i), x = i % NX;
+                if (i == 0 || (PAIR && i == 1 && w == 1)) mbar_wait(&bars[F4_Q + (PAIR ? w : 0)], 0, ab);
+                if (!PAIR || i >= 2 * both || w == 0) mbar_wait(&bars[F4_KF + k % NK], (k / NK) & 1, ab);
+                if (i >= NX) mbar_wait(&bars[F4_XF + x], (i / NX - 1) & 1, ab);
+                // two items of one warpgroup in a row: the barrier of its S may not complete a second time before it has seen the first
+                if (PAIR && NX > 1 && i >= 2 * both && i > 0) mbar_wait(&bars[F4_XF + (i - 1) % NX], ((i - 1) / NX) & 1, ab);
+                tcgen05_fence_after();
+                const uint32_t kK = desc_lo_kmajor(smem_u32(smem + C::oK + (k % NK) * C::kTile));
+                const uint32_t kQw = kQ + (PAIR ? w : 0) * (C::kTile >> 4);
+#pragma unroll
+                for (int kk = 0; kk < HD / 16; ++kk) {
+                    const uint32_t off = (kk / 4) * (C::kSlab >> 4) + (kk % 4) * 2;
+                    mma_ss_lo(tm + x * 128, kQw + off, kK + off, idesc_s, kk > 0);
+                }
+                mma_commit(&bars[F4_S + w]);
+                if (tile_ends(i) && k + NK < tiles) mma_commit(&bars[F4_KE + k % NK]);
+            }
+        }
+      } else if (warp == 10) {
+        // ------------------------------------------------------------ MMA issuer B: O += P V
+        if (lane == 0) {
+            constexpr uint32_t idesc_o = idesc_bf16(128, HD, 0, 1);
+            for (int i = 0; i < items; ++i) {
+                const int w = group_of(i), c = nth_of(i), k = tile_of(i);
+                const uint32_t mV_ = desc_lo_mnmajor(smem_u32(smem + C::oV + (k % NV) * C::kTile), C::kSlab);
+                const uint32_t tO = tm + C::tO + w * HD, tP = tm + C::tP + w * 64;
+                if (!PAIR || i >= 2 * both || w == 0) mbar_wait(&bars[F4_VF + k % NV], (k / NV) & 1, ab);
+                mbar_wait(&bars[F4_PE + w], c & 1, ab);   // the first 96 keys, then the rest
+                tcgen05_fence_after();
+#pragma unroll
+                for (int kk = 0; kk < TKF / 16; ++kk) {
+                    if (kk == 6) {
+                        mbar_wait(&bars[F4_P + w], c & 1, ab);
+                        tcgen05_fence_after();
+                    }
+                    mma_ts_lo(tO, tP + kk * 8, mV_ + kk * 128, idesc_o, (c > 0) || (kk > 0));
+                }
+                if (tile_ends(i) && k + NV < tiles) mma_commit(&bars[F4_VE + k % NV]);
+                mma_commit(&bars[F4_O + w]);
+            }
+        }
+      }
+    } else {
+        // ------------------------------------------------------------ softmax warpgroup w
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
+        const int w = warp / 4;
+        const int row = (warp % 4) * 32 + lane;
+        const uint32_t lane_addr = (uint32_t)((warp % 4) * 32) << 16;
+        const int iw = i0 + (PAIR ? w * TQ : 0), ig = iw + row, mine = w == 0 ? n0 : n1;
+        const float sl2 = a.scale * kLog2e;
+        const uint32_t T_P = tm + C::tP + w * 64 + lane_addr, T_O = tm + C::tO + w * HD + lane_addr;
+        float m_ref = -INFINITY, l_run = 0.f;
+        int raw = 0, seen = 0;   // !PAIR: position in the list of key tiles
+        for (int c = 0; c < mine; ++c) {
+            const int i = item_of(w, c), x = i % NX;
+            int jt = c;
+            if constexpr (!PAIR) {
+                for (;; ++raw) {
+                    jt = iter.tile(raw);
+                    if (jt >= 0 && seen++ == i) break;
+                }
+                ++raw;
+            }
+            const int j0 = jt * TKF;
+            const bool edge = (causal && j0 + TKF - 1 > iw) || j0 + TKF > n;   // entries dropped by position
+            // a mask finer than the tile: the keep bits of this thread's query row, all four words in flight before the wait
+            // for S (fetched one after the other behind it they were most of a tile's time: 16 heads, n = 4096, d = 128,
+            // a window of 512 keys: 72 us a launch, 64 us this way)
+            uint32_t kws[FINE ? TKF / 32 : 1];
+            if constexpr (FINE) {
+#pragma unroll
+                for (int q = 0; q < TKF / 32; ++q)
+                    kws[q] = (ig < n && j0 + q * 32 < n) ? fine_word(a.fine, a.mask_heads, bh, true, ig, j0 + q * 32) : 0u;
+            }
+            mbar_wait(&bars[F4_S + w], c & 1, ab);
+            tcgen05_fence_after();
+            uint32_t v[TKF];   // the whole row of raw scores in registers: four loads in flight, one wait
+#pragma unroll
+            for (int e = 0; e < TKF; e += 32) tmem_ld32(tm + x * 128 + lane_addr + e, *reinterpret_cast<uint32_t(*)[32]>(&v[e]));
+            tmem_wait_ld();
+            tcgen05_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars[F4_XF + x]);   // the buffer may take the next S
+            if constexpr (FINE) {
+#pragma unroll
+                for (int q = 0; q < TKF / 32; ++q) {
+                    // a word that keeps all or nothing (the rule with 32- and 64-wide blocks) needs no test per entry
+                    const uint32_t kw = kws[q];
+                    if (!edge && kw == 0xffffffffu) continue;
+                    if (kw == 0u) {
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) v[q * 32 + e] = 0xff800000u;   // -inf
+                        continue;
+                    }
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) {
+                        const int jg = j0 + q * 32 + e;
+                        if (jg >= n || (causal && jg > ig) || !((kw >> e) & 1u)) v[q * 32 + e] = 0xff800000u;
+                    }
+                }
+            } else if (edge) {
+                const int keep = min(n, causal ? ig + 1 : n) - j0;   // the row keeps its first `keep` entries of the tile
+#pragma unroll
+                for (int e = 0; e < TKF; ++e)
+                    if (e >= keep) v[e] = 0xff800000u;   // -inf
+            }
+            const float m_tile = row_max(v) * sl2;   // scale > 0: the maximum commutes with it
+            bool need = m_tile > m_ref + kRescaleThreshold || (m_ref == -INFINITY && m_tile != -INFINITY);
+            float m_new = need ? fmaxf(m_ref, m_tile) : m_ref;
+            if (PAIR && c - 1u < kExactTiles && m_ref != -INFINITY && m_tile != -INFINITY) {
+                // the next reference from which the tile's maximum is a whole number of powers of two away, by less than one
+                // unit up also where the sum is rounded (references of 2^24 and more)
+                m_new = m_tile > m_ref ? m_tile : fminf(fmaxf(m_tile + ceilf(m_ref - m_tile), m_ref), m_ref + 1.f);
+                need = true;
+            }
+            // O_w += P V of this warpgroup's previous tile: it reads P_w and adds to O_w
+            bool landed = c == 0;
+            auto wait_landed = [&] {
+                if (!landed) {
+                    mbar_wait(&bars[F4_O + w], (c - 1) & 1, ab);
+                    tcgen05_fence_after();
+                    landed = true;
+                }
+            };
+            if (__any_sync(0xffffffffu, need)) {
+                const float alpha = (need && m_ref != -INFINITY) ? ex2_fast_f(m_ref - m_new) : 1.f;
+                if (c > 0) {
+                    wait_landed();
+#pragma unroll
+                    for (int e0 = 0; e0 < HD; e0 += 32) {
+                        uint32_t o[32];
+                        tmem_ld32(T_O + e0, o);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+                        tmem_st32(T_O + e0, o);
+                    }
+                }
+                l_run *= alpha;
+                m_ref = m_new;
+            }
+            const float noff = m_ref == -INFINITY ? 0.f : -m_ref;
+            l_run += exp_row(v, sl2, noff, T_P, &bars[F4_PE + w], &bars[F4_P + w], lane, wait_landed);
+        }
+        // ------------------------------------------------------------ epilogue
+        if constexpr (PAIR) {
+            if (mine > 0) {
+                const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+                mbar_wait(&bars[F4_O + w], (mine - 1) & 1, ab);
+                tcgen05_fence_after();
+                const int ic = ig < n ? ig : 0;
+                __nv_bfloat16 *po = a.O + ((size_t)bh * n + ic) * HD;
+#pragma unroll
+                for (int c = 0; c < HD; c += 32) {
+                    uint32_t o[32];
+                    tmem_ld32(T_O + c, o);
+                    tmem_wait_ld();
+                    if (ig < n) {
+#pragma unroll
+                        for (int e = 0; e < 32; e += 8) {
+                            float y[8];
+#pragma unroll
+                            for (int u = 0; u < 8; ++u) y[u] = __uint_as_float(o[e + u]) * inv;
+                            *reinterpret_cast<uint4 *>(po + c + e) = make_uint4(pack_bf16(y[0], y[1]), pack_bf16(y[2], y[3]),
+                                                                                pack_bf16(y[4], y[5]), pack_bf16(y[6], y[7]));
+                        }
+                    }
+                }
+                if (ig < n) a.LSE[(size_t)bh * n + ig] = row_lse(m_ref, l_run);
+            }
+        } else {
+            // merge the two partial softmaxes
+            xm[w * 128 + row] = m_ref;
+            xl[w * 128 + row] = l_run;
+            named_bar_sync_f(1, kSoftmaxThreads);
+            const float m0 = xm[row], m1 = xm[128 + row], l0 = xl[row], l1 = xl[128 + row];
+            const float m_all = fmaxf(m0, m1);
+            const float a0 = m0 == -INFINITY ? 0.f : ex2_fast_f(m0 - m_all), a1 = m1 == -INFINITY ? 0.f : ex2_fast_f(m1 - m_all);
+            const float l_tot = a0 * l0 + a1 * l1;
+            const float inv = l_tot > 0.f ? 1.f / l_tot : 0.f;
+            const float c0 = a0 * inv, c1 = a1 * inv;
+            // the other warpgroup's last product: it may be two completions of its barrier ahead of what this one has seen of it,
+            // but none can follow the last
+            if (n0 > 0) mbar_wait(&bars[F4_O], (n0 - 1) & 1, ab);
+            if (n1 > 0) mbar_wait(&bars[F4_O + 1], (n1 - 1) & 1, ab);
+            tcgen05_fence_after();
+            const int ic = ig < n ? ig : 0;
+            __nv_bfloat16 *po = a.O + ((size_t)bh * n + ic) * HD + w * (HD / 2);
+#pragma unroll
+            for (int c = 0; c < HD / 2; c += 32) {
+                uint32_t v0[32], v1[32];
+                if (n0 > 0) tmem_ld32(tm + C::tO + lane_addr + w * (HD / 2) + c, v0);
+                if (n1 > 0) tmem_ld32(tm + C::tO + HD + lane_addr + w * (HD / 2) + c, v1);
+                tmem_wait_ld();
+                float o[32];
+#pragma unroll
+                for (int e = 0; e < 32; ++e) {
+                    // a partial accumulator that never received a product holds stale bits: select, do not multiply
+                    const float x0 = n0 > 0 ? __uint_as_float(v0[e]) * c0 : 0.f;
+                    const float x1 = n1 > 0 ? __uint_as_float(v1[e]) * c1 : 0.f;
+                    o[e] = x0 + x1;
+                }
+                if (ig < n) {
+#pragma unroll
+                    for (int e = 0; e < 32; e += 8)
+                        *reinterpret_cast<uint4 *>(po + c + e) = make_uint4(pack_bf16(o[e], o[e + 1]), pack_bf16(o[e + 2], o[e + 3]),
+                                                                            pack_bf16(o[e + 4], o[e + 5]), pack_bf16(o[e + 6], o[e + 7]));
+                }
+            }
+            if (w == 0 && ig < n) a.LSE[(size_t)bh * n + ig] = row_lse(m_all, l_tot);
         }
     }
     tcgen05_fence_before();
@@ -1018,12 +1407,16 @@ attn_status launch_fwd(const Problem &p)
     a.status = p.status;
     a.group = fwd_head_group(p);
     if constexpr (HD != 256) {
-        if (pair_pays(p)) {
-            auto kernel = p.split ? tc_fwd_pair_kernel<HD, true> : tc_fwd_pair_kernel<HD, false>;
-            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg<HD>::kBytes) != cudaSuccess)
-                return ATTN_ERR_LAUNCH;
+        const bool pair = pair_pays(p);
+        if (pair || !p.split) {
+            void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, FwdArgs) =
+                p.split ? tc_fwd_pair_kernel<HD> : pair ? tc_fwd_flow_kernel<HD, true, false>
+                : p.fine.mode ? tc_fwd_flow_kernel<HD, false, true> : tc_fwd_flow_kernel<HD, false, false>;
+            const uint32_t bytes = p.split ? PairCfg<HD>::kBytes : pair ? FlowCfg<HD, true>::kBytes : FlowCfg<HD, false>::kBytes;
+            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return ATTN_ERR_LAUNCH;
+            const int rows = pair ? 256 : 128;
             launch_begin("tc_fwd", p.stream);
-            const bool ok = launch_chained(kernel, dim3((p.n + 255) / 256 * a.group, (unsigned)p.BH / a.group), kThreadsRows, PairCfg<HD>::kBytes, p.stream, mQ, mK, mV, a);
+            const bool ok = launch_chained(kernel, dim3((p.n + rows - 1) / rows * a.group, (unsigned)p.BH / a.group), kThreadsRows, bytes, p.stream, mQ, mK, mV, a);
             launch_end(p.stream);
             return ok ? ATTN_OK : ATTN_ERR_LAUNCH;
         }
@@ -1032,8 +1425,7 @@ attn_status launch_fwd(const Problem &p)
     using C = typename std::conditional<HD == 256, FwdCfg<HD>, RowsCfg<HD>>::type;
     const uint32_t bytes = C::kBytes;
     if constexpr (HD == 256) kernel = tc_fwd_kernel<HD>;
-    else if (p.split) kernel = p.fine.mode ? tc_fwd_rows_kernel<HD, true, true> : tc_fwd_rows_kernel<HD, false, true>;
-    else kernel = p.fine.mode ? tc_fwd_rows_kernel<HD, true, false> : tc_fwd_rows_kernel<HD, false, false>;
+    else kernel = p.fine.mode ? tc_fwd_rows_kernel<HD, true> : tc_fwd_rows_kernel<HD, false>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
         return ATTN_ERR_LAUNCH;
     const dim3 grid((p.n + TQ - 1) / TQ * a.group, (unsigned)p.BH / a.group);
@@ -1047,7 +1439,7 @@ attn_status launch_fwd(const Problem &p)
 
 size_t fwd_smem_bytes(int d)
 {
-    return d == 64 ? RowsCfg<64>::kUsed : d == 128 ? RowsCfg<128>::kUsed : d == 256 ? FwdCfg<256>::kUsed : 0;
+    return d == 64 ? FlowCfg<64, false>::kUsed : d == 128 ? FlowCfg<128, false>::kUsed : d == 256 ? FwdCfg<256>::kUsed : 0;
 }
 
 attn_status tc_fwd(const Problem &p)
