@@ -16,7 +16,7 @@
 // are free as soon as it has been copied out.  PAIR (no mask or causal, calls with enough tiles): two query tiles per CTA, a
 // softmax warpgroup each.  Otherwise one query tile, the two softmax warpgroups take alternate key tiles, each with a partial
 // accumulator of its own, and the two partial softmaxes are merged in the epilogue.  tc_fwd_pair_kernel and
-// tc_fwd_rows_kernel: the same two shapes for calls whose P must not be rounded to one bf16 term; its second term takes the
+// tc_fwd_rows_kernel: the same two shapes, a CTA per unit of work, for calls whose P must not be rounded to one bf16 term; its second term takes the
 // tensor memory that the S buffers would need.  tc_fwd_kernel (d = 256; key tiles of 64): both warpgroups
 // split the columns of every tile and exchange row maxima through shared memory, one accumulator of
 // 256 columns.  The roles and the tensor-memory layout are described at each kernel.
@@ -114,6 +114,13 @@ __device__ __forceinline__ float ex2_fast_f(float x)
 __device__ __forceinline__ void named_bar_sync_f(int id, int count)
 {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
+// one arrival per warp: every lane has finished (and fenced) its part
+__device__ __forceinline__ void warp_arrive_f(uint64_t *bar, int lane)
+{
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar);
 }
 
 // LSE of a row from its reference m (log2 units) and its sum l: m ln2 + ln l with one rounding of the size of the result.
@@ -625,9 +632,7 @@ tc_fwd_rows_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
             const int j0 = jt * TKF;
             const bool causal = mask_is_causal(a.mask_kind);
             const bool need_mask = (causal && j0 + TKF - 1 > i0) || j0 + TKF > n || FINE;
-            // a mask finer than the tile: the keep bits of this thread's query row, all four words in flight before the wait
-            // for S (fetched one after the other behind it they were most of a tile's time: 16 heads, n = 4096, d = 128,
-            // a window of 512 keys: 72 us a launch, 64 us this way)
+            // a mask finer than the tile: the keep bits of this thread's query row, all four words in flight before the wait for S
             uint32_t kws[TKF / 32];
             if constexpr (FINE) {
 #pragma unroll
@@ -978,6 +983,16 @@ tc_fwd_pair_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
 // 32 heads, n = 8192, d = 128, causal: 566 -> 525 us; block-sparse, 32 heads, n = 32768, 10 %: 1844 -> 1794 us; 24 heads,
 // n = 3000, d = 64, one query tile: 109 -> 105 us; 64 heads, n = 2048, d = 64: 127 us both.
 //
+// A CTA stays on its SM and takes the block indices of CTAs that have not started yet (cluster launch control), in the order of
+// the launch.  The loading warp publishes each unit of work in one of two slots; every role walks from one unit to the next by
+// itself, with its barriers running on: Q of the next unit is loaded once the last S of this one has been formed, and its first
+// S is there when a warpgroup has written its O.  With a CTA per unit 7.4 to 7.8 us a CTA passed outside its tiles (launch 0.7,
+// set-up 0.6, lists and first loads 1.5 to 3.0, epilogue and the slower warpgroup 3.0 to 4.5), as long as five tiles take.
+// 32 heads, n = 8192, d = 128, causal: 450 -> 432 us; 32 heads, n = 4096: 133 -> 121; block-sparse as above: 1794 -> 1605;
+// block-sparse and causal, 16 heads, n = 8192, 20 %: 129 -> 84; window of 512 keys, 16 heads, n = 4096: 66 -> 64, and 51 with the
+// keep words fetched a tile ahead and tested by one predicate an entry; 64 heads, n = 2048, d = 64: 127 -> 119 (a session at
+// full clock, kernel alone).
+//
 // A row's largest probabilities are what the rounding of P to bf16 costs most, and the one that the reference was taken from is
 // exactly 1.  Two partial softmaxes a row (one query tile) have two such entries, one softmax has one, and its O is one per cent further
 // from 64 bits.  So the first kExactTiles tiles after the first one move the reference (up, by less than one unit beyond what the
@@ -996,14 +1011,25 @@ struct FlowCfg {
     static constexpr uint32_t oV = oK + NK * kTile;
     static constexpr uint32_t oX = oV + NV * kTile;            // merge of the two partial softmaxes (one query tile)
     static constexpr uint32_t oBar = oX + (PAIR ? 0 : 4 * 128 * 4);
-    static constexpr uint32_t oMisc = oBar + 24 * 8;
-    static constexpr uint32_t kUsed = oMisc + 64;
+    static constexpr uint32_t oWork = oBar + 32 * 8;           // two slots of FlowWork, the answer of the scheduler
+    static constexpr uint32_t oMisc = oWork + 2 * 32 + 16;
+    static constexpr uint32_t kUsed = oMisc + 16;
     static_assert(kUsed <= 227 * 1024, "shared memory budget");
     static constexpr uint32_t kBytes = kUsed < 117 * 1024 ? 117 * 1024 : kUsed;   // one CTA per SM: all of tensor memory
     static constexpr uint32_t tP = NX * 128, tO = tP + 128;    // tensor-memory columns
     static_assert(tO + 2 * HD == 512, "tensor memory");
 };
-enum { F4_Q = 0, F4_KF = 2, F4_KE = 5, F4_VF = 8, F4_VE = 11, F4_S = 14, F4_XF = 16, F4_PE = 18, F4_P = 20, F4_O = 22 };
+enum { F4_QF = 0, F4_QE = 2, F4_KF = 4, F4_KE = 7, F4_VF = 10, F4_VE = 13, F4_S = 16, F4_O = 18, F4_CLC = 20, F4_WF = 21, F4_WE = 23,
+       F4_XF = 25, F4_PE = 27, F4_P = 29, F4_COUNT = 31 };
+
+// One unit of work: a query tile (or two) of one head
+struct FlowWork {
+    int i0, bh;        // first query; -1: there is no more work
+    int n0, n1;        // items of the warpgroups
+    const int *cols;   // key blocks of a mask with lists
+    int pad[2];
+};
+static_assert(sizeof(FlowWork) == 32, "two slots in shared memory");
 
 // P = exp2(v * sl2 + noff) as bf16 pairs into columns of its own; returns the sum of the row of P before rounding.  `free` waits
 // until the columns may be written, by when 64 keys are ready.  The first 96 keys are handed over (`early`, one arrival per
@@ -1046,21 +1072,20 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                    const __grid_constant__ CUtensorMap mV, const FwdArgs a)
 {
     using C = FlowCfg<HD, PAIR>;
-    constexpr int TKF = 128, NK = C::NK, NV = C::NV, NX = C::NX;
+    constexpr int TKF = 128, NK = C::NK, NV = C::NV, NX = C::NX, QROWS = C::NQ * TQ;
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + C::oBar);
     uint32_t *tmem_base_s = reinterpret_cast<uint32_t *>(smem + C::oMisc);
     volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(smem + C::oMisc + 4);
+    volatile FlowWork *slots = reinterpret_cast<volatile FlowWork *>(smem + C::oWork);
     float *xm = reinterpret_cast<float *>(smem + C::oX);   // !PAIR: [2 warpgroups][128 rows] reference maxima
     float *xl = xm + 256;                                  // [2][128] row sums
     const Abort ab{abort_flag, a.status};
 
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     const int n = a.n;
-    constexpr int QROWS = C::NQ * TQ;
-    const int i0 = ((n + QROWS - 1) / QROWS - 1 - (int)blockIdx.x / a.group) * QROWS;   // heaviest causal tiles first
-    const long bh = (long)blockIdx.y * a.group + blockIdx.x % a.group;
-    const bool causal = mask_is_causal(a.mask_kind);
+    const bool causal = mask_is_causal(a.mask_kind), lists = mask_is_block(a.mask_kind);
+    const int sub = lists ? a.block / TKF : 1;
 
     if ((smem_u32(smem) & 1023u) != 0) {
         chain_wait();
@@ -1069,10 +1094,8 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
     }
     if (tid == 0) {
         *abort_flag = 0;
-        for (int b = 0; b < 24; ++b) {
-            const bool warps = b >= F4_XF && b < F4_O;   // XF, PE, P: the four warps of a warpgroup
-            mbar_init(&bars[b], warps ? 4 : 1);
-        }
+        for (int b = 0; b < F4_COUNT; ++b)   // XF, PE, P: the four warps of a warpgroup; WE: both issuers and eight warps
+            mbar_init(&bars[b], b >= F4_XF ? 4 : b >= F4_WE ? 10 : 1);
         fence_barrier_init();
         prefetch_tensormap(&mQ); prefetch_tensormap(&mK); prefetch_tensormap(&mV);
     }
@@ -1085,104 +1108,177 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
     if (tid == 0 && blockIdx.x == 0 && blockIdx.y == 0) *a.status = 0u;
     const uint32_t tm = *tmem_base_s;
 
-    // Items in the order in which their S is formed.  PAIR: (query tile w, key tile k) = (0, 0), (1, 0), (0, 1), ..., then what one
-    // query tile has left; otherwise item k is key tile k of warpgroup k % 2.
-    const KeyIter<TKF> iter(a, PAIR ? 0 : i0 / TQ, bh);
-    int n0, n1;   // items of the warpgroups
-    if constexpr (PAIR) {
-        auto count = [&](int w) {   // key tiles of query tile w (the second one may lie beyond n)
-            const int first = i0 + w * TQ;
-            if (first >= n) return 0;
-            return causal ? (min(first + TQ, n) - 1) / TKF + 1 : (n + TKF - 1) / TKF;
-        };
-        n0 = count(0), n1 = count(1);
-    } else {
-        int kept = 0;
-        for (int idx = 0; idx < iter.raw; ++idx) kept += iter.tile(idx) >= 0;
-        n0 = (kept + 1) / 2, n1 = kept / 2;
-    }
-    const int both = min(n0, n1), items = n0 + n1, tiles = PAIR ? max(n0, n1) : items;
-    auto item_of = [&](int w, int c) { return c < both ? 2 * c + w : both + c; };             // c-th item of warpgroup w
-    auto group_of = [&](int i) { return i < 2 * both ? i & 1 : n0 > n1 ? 0 : 1; };
-    auto nth_of = [&](int i) { return i < 2 * both ? i >> 1 : i - both; };                    // its index there
-    auto tile_of = [&](int i) { return PAIR ? nth_of(i) : i; };
-    auto tile_ends = [&](int i) { return !PAIR || i >= 2 * both || (i & 1) != 0; };           // nothing after item i uses its key tile
+    // Items of a unit of work in the order in which their S is formed.  PAIR: (query tile w, key tile k) = (0, 0), (1, 0), (0, 1),
+    // ..., then what one query tile has left; otherwise item k is key tile k of warpgroup k % 2.
+    struct Order {
+        int both, items, tiles;
+        bool zero;   // the rest belongs to warpgroup 0
+        __device__ Order(int n0, int n1) : both(min(n0, n1)), items(n0 + n1), tiles(PAIR ? max(n0, n1) : n0 + n1), zero(n0 > n1) {}
+        __device__ int item(int w, int c) const { return c < both ? 2 * c + w : both + c; }   // c-th item of warpgroup w
+        __device__ int group(int i) const { return i < 2 * both ? i & 1 : zero ? 0 : 1; }
+        __device__ int nth(int i) const { return i < 2 * both ? i >> 1 : i - both; }          // its index there
+        __device__ int tile(int i) const { return PAIR ? nth(i) : i; }
+        __device__ bool begins(int i) const { return !PAIR || i >= 2 * both || (i & 1) == 0; }  // the first item of its key tile
+        __device__ bool ends(int i) const { return !PAIR || i >= 2 * both || (i & 1) != 0; }    // the last one
+    };
+    // the t-th unit of work of this CTA as the loading warp has published it (false: there is none)
+    auto work = [&](int t, FlowWork &f) {
+        if (!mbar_wait(&bars[F4_WF + (t & 1)], (t >> 1) & 1, ab)) return false;
+        const volatile FlowWork &v = slots[t & 1];
+        f.i0 = v.i0; f.bh = v.bh; f.n0 = v.n0; f.n1 = v.n1; f.cols = v.cols;
+        return f.i0 >= 0;
+    };
 
     if (warp >= 8) {
       asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
       if (warp == 9) {
-        // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
-            auto load = [&](uint32_t to, const CUtensorMap *m, uint64_t *bar, int row) {
+        // ------------------------------------------------------------ TMA producer, and the schedule
+        auto load = [&](uint32_t to, const CUtensorMap *m, uint64_t *bar, int row, int bh) {
+            mbar_expect_tx(bar, C::kTile);
 #pragma unroll
-                for (uint32_t sl = 0; sl < C::kSlabs; ++sl) tma_load_3d(smem + to + sl * C::kSlab, m, bar, sl * 64, row, (int)bh);
-            };
-            mbar_expect_tx(&bars[F4_Q], C::kTile);
-            load(C::oQ, &mQ, &bars[F4_Q], i0);
-            int k = 0;
-            for (int idx = 0; idx < (PAIR ? tiles : iter.raw); ++idx) {
-                const int jt = PAIR ? idx : iter.tile(idx);
-                if (jt < 0) continue;
-                const int sk = k % NK, sv = k % NV;
-                if (k >= NK) mbar_wait(&bars[F4_KE + sk], (k / NK - 1) & 1, ab);
-                mbar_expect_tx(&bars[F4_KF + sk], C::kTile);
-                load(C::oK + sk * C::kTile, &mK, &bars[F4_KF + sk], jt * TKF);
-                if (PAIR && k == 0 && n1 > 0) {
-                    mbar_expect_tx(&bars[F4_Q + 1], C::kTile);
-                    load(C::oQ + C::kTile, &mQ, &bars[F4_Q + 1], i0 + TQ);
+            for (uint32_t sl = 0; sl < C::kSlabs; ++sl) tma_load_3d(smem + to + sl * C::kSlab, m, bar, sl * 64, row, bh);
+        };
+        int bx = blockIdx.x, by = blockIdx.y;
+        int kt = 0;                // key tiles loaded so far
+        int nq0 = 0, nq1 = 0;      // loads of each Q buffer so far
+        bool more = true;
+        for (int t = 0; more; ++t) {
+            const int i0 = ((n + QROWS - 1) / QROWS - 1 - bx / a.group) * QROWS;   // heaviest causal tiles first
+            const int bh = by * a.group + bx % a.group;
+            int n0, n1;
+            const int *cols = nullptr;
+            if constexpr (PAIR) {
+                auto count = [&](int w) {   // key tiles of query tile w (the second one may lie beyond n)
+                    const int first = i0 + w * TQ;
+                    if (first >= n) return 0;
+                    return causal ? (min(first + TQ, n) - 1) / TKF + 1 : (n + TKF - 1) / TKF;
+                };
+                n0 = count(0), n1 = count(1);
+            } else {
+                int kept = 0;
+                const int last_i = min(i0 + TQ, n) - 1;
+                if (lists) {
+                    // the lists ascend, so what lies beyond n or (block mask AND causal) begins after the last query is at their end
+                    const long mh = a.mask_heads == 1 ? 0 : bh;
+                    const int *rp = a.row_ptr + mh * 2 * a.nb + 2 * (i0 / a.block);
+                    const int first = rp[0], raw = (rp[1] - first) * sub, limit = causal ? last_i : n - 1;
+                    cols = a.col_idx + mh * (long)a.nb * a.nb + first;
+                    for (int e = lane; e < raw; e += 32) kept += (cols[e / sub] * sub + e % sub) * TKF <= limit;
+                    kept = __reduce_add_sync(0xffffffffu, kept);
+                } else {
+                    kept = causal ? last_i / TKF + 1 : (n + TKF - 1) / TKF;
                 }
-                if (k >= NV) mbar_wait(&bars[F4_VE + sv], (k / NV - 1) & 1, ab);
-                mbar_expect_tx(&bars[F4_VF + sv], C::kTile);
-                load(C::oV + sv * C::kTile, &mV, &bars[F4_VF + sv], jt * TKF);
-                ++k;
+                n0 = (kept + 1) / 2, n1 = kept / 2;
             }
-            if (items == 0) mbar_wait(&bars[F4_Q], 0, ab);   // let the Q load land before exit
+            const Order o(n0, n1);
+            if (lane == 0) {
+                if (t >= 2) mbar_wait(&bars[F4_WE + (t & 1)], ((t >> 1) - 1) & 1, ab);
+                volatile FlowWork &f = slots[t & 1];
+                f.i0 = i0; f.bh = bh; f.n0 = n0; f.n1 = n1; f.cols = cols;
+                mbar_arrive(&bars[F4_WF + (t & 1)]);
+                if (o.items > 0) {
+                    if (nq0 > 0) mbar_wait(&bars[F4_QE], (nq0 - 1) & 1, ab);
+                    load(C::oQ, &mQ, &bars[F4_QF], i0, bh);
+                    ++nq0;
+                }
+                int jt = lists && o.tiles > 0 ? cols[0] * sub : 0;
+                for (int k = 0; k < o.tiles; ++k, ++kt) {
+                    const int sk = kt % NK, sv = kt % NV;
+                    const int here = jt;
+                    if (k + 1 < o.tiles) jt = lists ? cols[(k + 1) / sub] * sub + (k + 1) % sub : k + 1;
+                    // the next unit of work, asked for early enough that the answer is there when the loads get to it
+                    if (k == max(o.tiles - 2, 0)) clc_request(smem + C::oWork + 2 * sizeof(FlowWork), &bars[F4_CLC]);
+                    if (kt >= NK) mbar_wait(&bars[F4_KE + sk], (kt / NK - 1) & 1, ab);
+                    load(C::oK + sk * C::kTile, &mK, &bars[F4_KF + sk], here * TKF, bh);
+                    if (PAIR && k == 0 && n1 > 0) {
+                        if (nq1 > 0) mbar_wait(&bars[F4_QE + 1], (nq1 - 1) & 1, ab);
+                        load(C::oQ + C::kTile, &mQ, &bars[F4_QF + 1], i0 + TQ, bh);
+                        ++nq1;
+                    }
+                    if (kt >= NV) mbar_wait(&bars[F4_VE + sv], (kt / NV - 1) & 1, ab);
+                    load(C::oV + sv * C::kTile, &mV, &bars[F4_VF + sv], here * TKF, bh);
+                }
+                if (o.tiles == 0) clc_request(smem + C::oWork + 2 * sizeof(FlowWork), &bars[F4_CLC]);
+                more = mbar_wait(&bars[F4_CLC], t & 1, ab) && clc_answer(smem + C::oWork + 2 * sizeof(FlowWork), bx, by);
+                if (!more) {
+                    if (t >= 1) mbar_wait(&bars[F4_WE + ((t + 1) & 1)], (((t + 1) >> 1) - 1) & 1, ab);
+                    slots[(t + 1) & 1].i0 = -1;
+                    mbar_arrive(&bars[F4_WF + ((t + 1) & 1)]);
+                }
+            }
+            more = __shfl_sync(0xffffffffu, (int)more, 0) != 0;
+            bx = __shfl_sync(0xffffffffu, bx, 0);
+            by = __shfl_sync(0xffffffffu, by, 0);
         }
       } else if (warp == 8) {
         // ------------------------------------------------------------ MMA issuer A: S = Q K^T
         if (lane == 0) {
             constexpr uint32_t idesc_s = idesc_bf16(128, TKF, 0, 0);
             const uint32_t kQ = desc_lo_kmajor(smem_u32(smem + C::oQ));
-            for (int i = 0; i < items; ++i) {
-                const int w = group_of(i), k = tile_of(i), x = i % NX;
-                if (i == 0 || (PAIR && i == 1 && w == 1)) mbar_wait(&bars[F4_Q + (PAIR ? w : 0)], 0, ab);
-                if (!PAIR || i >= 2 * both || w == 0) mbar_wait(&bars[F4_KF + k % NK], (k / NK) & 1, ab);
-                if (i >= NX) mbar_wait(&bars[F4_XF + x], (i / NX - 1) & 1, ab);
-                // two items of one warpgroup in a row: the barrier of its S may not complete a second time before it has seen the first
-                if (PAIR && NX > 1 && i >= 2 * both && i > 0) mbar_wait(&bars[F4_XF + (i - 1) % NX], ((i - 1) / NX) & 1, ab);
-                tcgen05_fence_after();
-                const uint32_t kK = desc_lo_kmajor(smem_u32(smem + C::oK + (k % NK) * C::kTile));
-                const uint32_t kQw = kQ + (PAIR ? w : 0) * (C::kTile >> 4);
+            FlowWork f;
+            int g = 0, kt0 = 0, last_w = -1;   // items and key tiles before this unit of work; warpgroup of the item before
+            int nq0 = 0, nq1 = 0;
+            for (int t = 0; work(t, f); ++t) {
+                mbar_arrive(&bars[F4_WE + (t & 1)]);
+                const Order o(f.n0, f.n1);
+                for (int i = 0; i < o.items; ++i, ++g) {
+                    const int w = o.group(i), k = kt0 + o.tile(i), x = g % NX;
+                    const int q = PAIR ? w : 0;
+                    if (i == 0 || (PAIR && i == 1 && w == 1)) {
+                        mbar_wait(&bars[F4_QF + q], (q == 0 ? nq0 : nq1) & 1, ab);
+                        if (q == 0) ++nq0; else ++nq1;
+                    }
+                    if (o.begins(i)) mbar_wait(&bars[F4_KF + k % NK], (k / NK) & 1, ab);
+                    if (g >= NX) mbar_wait(&bars[F4_XF + x], (g / NX - 1) & 1, ab);
+                    // two items of one warpgroup in a row: the barrier of its S may not complete a second time before it has seen the first
+                    if (NX > 1 && w == last_w) mbar_wait(&bars[F4_XF + (g - 1) % NX], ((g - 1) / NX) & 1, ab);
+                    last_w = w;
+                    tcgen05_fence_after();
+                    const uint32_t kK = desc_lo_kmajor(smem_u32(smem + C::oK + (k % NK) * C::kTile));
+                    const uint32_t kQw = kQ + q * (C::kTile >> 4);
 #pragma unroll
-                for (int kk = 0; kk < HD / 16; ++kk) {
-                    const uint32_t off = (kk / 4) * (C::kSlab >> 4) + (kk % 4) * 2;
-                    mma_ss_lo(tm + x * 128, kQw + off, kK + off, idesc_s, kk > 0);
+                    for (int kk = 0; kk < HD / 16; ++kk) {
+                        const uint32_t off = (kk / 4) * (C::kSlab >> 4) + (kk % 4) * 2;
+                        mma_ss_lo(tm + x * 128, kQw + off, kK + off, idesc_s, kk > 0);
+                    }
+                    mma_commit(&bars[F4_S + w]);
+                    if (o.ends(i)) mma_commit(&bars[F4_KE + k % NK]);
+                    if (PAIR ? o.nth(i) + 1 == (w == 0 ? f.n0 : f.n1) : i + 1 == o.items) mma_commit(&bars[F4_QE + q]);
                 }
-                mma_commit(&bars[F4_S + w]);
-                if (tile_ends(i) && k + NK < tiles) mma_commit(&bars[F4_KE + k % NK]);
+                kt0 += o.tiles;
             }
         }
       } else if (warp == 10) {
         // ------------------------------------------------------------ MMA issuer B: O += P V
         if (lane == 0) {
             constexpr uint32_t idesc_o = idesc_bf16(128, HD, 0, 1);
-            for (int i = 0; i < items; ++i) {
-                const int w = group_of(i), c = nth_of(i), k = tile_of(i);
-                const uint32_t mV_ = desc_lo_mnmajor(smem_u32(smem + C::oV + (k % NV) * C::kTile), C::kSlab);
-                const uint32_t tO = tm + C::tO + w * HD, tP = tm + C::tP + w * 64;
-                if (!PAIR || i >= 2 * both || w == 0) mbar_wait(&bars[F4_VF + k % NV], (k / NV) & 1, ab);
-                mbar_wait(&bars[F4_PE + w], c & 1, ab);   // the first 96 keys, then the rest
-                tcgen05_fence_after();
+            FlowWork f;
+            int kt0 = 0, c0 = 0, c1 = 0;   // key tiles and items of each warpgroup before this unit of work
+            for (int t = 0; work(t, f); ++t) {
+                mbar_arrive(&bars[F4_WE + (t & 1)]);
+                const Order o(f.n0, f.n1);
+                for (int i = 0; i < o.items; ++i) {
+                    const int w = o.group(i), c = o.nth(i), k = kt0 + o.tile(i);
+                    const uint32_t parity = (c + (w == 0 ? c0 : c1)) & 1;
+                    const uint32_t mV_ = desc_lo_mnmajor(smem_u32(smem + C::oV + (k % NV) * C::kTile), C::kSlab);
+                    const uint32_t tO = tm + C::tO + w * HD, tP = tm + C::tP + w * 64;
+                    if (o.begins(i)) mbar_wait(&bars[F4_VF + k % NV], (k / NV) & 1, ab);
+                    mbar_wait(&bars[F4_PE + w], parity, ab);   // the first 96 keys, then the rest
+                    tcgen05_fence_after();
 #pragma unroll
-                for (int kk = 0; kk < TKF / 16; ++kk) {
-                    if (kk == 6) {
-                        mbar_wait(&bars[F4_P + w], c & 1, ab);
-                        tcgen05_fence_after();
+                    for (int kk = 0; kk < TKF / 16; ++kk) {
+                        if (kk == 6) {
+                            mbar_wait(&bars[F4_P + w], parity, ab);
+                            tcgen05_fence_after();
+                        }
+                        mma_ts_lo(tO, tP + kk * 8, mV_ + kk * 128, idesc_o, (c > 0) || (kk > 0));
                     }
-                    mma_ts_lo(tO, tP + kk * 8, mV_ + kk * 128, idesc_o, (c > 0) || (kk > 0));
+                    if (o.ends(i)) mma_commit(&bars[F4_VE + k % NV]);
+                    mma_commit(&bars[F4_O + w]);
                 }
-                if (tile_ends(i) && k + NV < tiles) mma_commit(&bars[F4_VE + k % NV]);
-                mma_commit(&bars[F4_O + w]);
+                kt0 += o.tiles;
+                c0 += f.n0;
+                c1 += f.n1;
             }
         }
       }
@@ -1192,168 +1288,179 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
         const int w = warp / 4;
         const int row = (warp % 4) * 32 + lane;
         const uint32_t lane_addr = (uint32_t)((warp % 4) * 32) << 16;
-        const int iw = i0 + (PAIR ? w * TQ : 0), ig = iw + row, mine = w == 0 ? n0 : n1;
         const float sl2 = a.scale * kLog2e;
         const uint32_t T_P = tm + C::tP + w * 64 + lane_addr, T_O = tm + C::tO + w * HD + lane_addr;
-        float m_ref = -INFINITY, l_run = 0.f;
-        int raw = 0, seen = 0;   // !PAIR: position in the list of key tiles
-        for (int c = 0; c < mine; ++c) {
-            const int i = item_of(w, c), x = i % NX;
-            int jt = c;
-            if constexpr (!PAIR) {
-                for (;; ++raw) {
-                    jt = iter.tile(raw);
-                    if (jt >= 0 && seen++ == i) break;
-                }
-                ++raw;
-            }
-            const int j0 = jt * TKF;
-            const bool edge = (causal && j0 + TKF - 1 > iw) || j0 + TKF > n;   // entries dropped by position
-            // a mask finer than the tile: the keep bits of this thread's query row, all four words in flight before the wait
-            // for S (fetched one after the other behind it they were most of a tile's time: 16 heads, n = 4096, d = 128,
-            // a window of 512 keys: 72 us a launch, 64 us this way)
-            uint32_t kws[FINE ? TKF / 32 : 1];
-            if constexpr (FINE) {
-#pragma unroll
-                for (int q = 0; q < TKF / 32; ++q)
-                    kws[q] = (ig < n && j0 + q * 32 < n) ? fine_word(a.fine, a.mask_heads, bh, true, ig, j0 + q * 32) : 0u;
-            }
-            mbar_wait(&bars[F4_S + w], c & 1, ab);
-            tcgen05_fence_after();
-            uint32_t v[TKF];   // the whole row of raw scores in registers: four loads in flight, one wait
-#pragma unroll
-            for (int e = 0; e < TKF; e += 32) tmem_ld32(tm + x * 128 + lane_addr + e, *reinterpret_cast<uint32_t(*)[32]>(&v[e]));
-            tmem_wait_ld();
-            tcgen05_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&bars[F4_XF + x]);   // the buffer may take the next S
-            if constexpr (FINE) {
+        const bool wide = ((uintptr_t)a.O & 31) == 0;
+        FlowWork f;
+        int g0 = 0, c0 = 0;   // items of both warpgroups and of this one before this unit of work
+        for (int t = 0; work(t, f); ++t) {
+            warp_arrive_f(&bars[F4_WE + (t & 1)], lane);
+            const Order o(f.n0, f.n1);
+            const int iw = f.i0 + (PAIR ? w * TQ : 0), ig = iw + row, mine = w == 0 ? f.n0 : f.n1;
+            const long bh = f.bh;
+            float m_ref = -INFINITY, l_run = 0.f;
+            // key tiles of this warpgroup's next two items and the keep bits of the next one are fetched ahead
+            auto tile_at = [&](int c) {
+                if (PAIR || !lists) return PAIR ? c : o.item(w, c);
+                const int i = min(o.item(w, c), o.items - 1);
+                return sub == 1 ? f.cols[i] : f.cols[i / sub] * sub + i % sub;
+            };
+            auto keep_words = [&](int j0, uint32_t (&to)[TKF / 32]) {
+                const int last = min(n - 1, causal ? ig : n - 1);   // of the keys that the row may keep by position
 #pragma unroll
                 for (int q = 0; q < TKF / 32; ++q) {
-                    // a word that keeps all or nothing (the rule with 32- and 64-wide blocks) needs no test per entry
-                    const uint32_t kw = kws[q];
-                    if (!edge && kw == 0xffffffffu) continue;
-                    if (kw == 0u) {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) v[q * 32 + e] = 0xff800000u;   // -inf
-                        continue;
-                    }
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) {
-                        const int jg = j0 + q * 32 + e;
-                        if (jg >= n || (causal && jg > ig) || !((kw >> e) & 1u)) v[q * 32 + e] = 0xff800000u;
-                    }
-                }
-            } else if (edge) {
-                const int keep = min(n, causal ? ig + 1 : n) - j0;   // the row keeps its first `keep` entries of the tile
-#pragma unroll
-                for (int e = 0; e < TKF; ++e)
-                    if (e >= keep) v[e] = 0xff800000u;   // -inf
-            }
-            const float m_tile = row_max(v) * sl2;   // scale > 0: the maximum commutes with it
-            bool need = m_tile > m_ref + kRescaleThreshold || (m_ref == -INFINITY && m_tile != -INFINITY);
-            float m_new = need ? fmaxf(m_ref, m_tile) : m_ref;
-            if (PAIR && c - 1u < kExactTiles && m_ref != -INFINITY && m_tile != -INFINITY) {
-                // the next reference from which the tile's maximum is a whole number of powers of two away, by less than one
-                // unit up also where the sum is rounded (references of 2^24 and more)
-                m_new = m_tile > m_ref ? m_tile : fminf(fmaxf(m_tile + ceilf(m_ref - m_tile), m_ref), m_ref + 1.f);
-                need = true;
-            }
-            // O_w += P V of this warpgroup's previous tile: it reads P_w and adds to O_w
-            bool landed = c == 0;
-            auto wait_landed = [&] {
-                if (!landed) {
-                    mbar_wait(&bars[F4_O + w], (c - 1) & 1, ab);
-                    tcgen05_fence_after();
-                    landed = true;
+                    const int left = last - (j0 + q * 32);
+                    to[q] = ig < n && left >= 0 ? fine_word(a.fine, a.mask_heads, bh, true, ig, j0 + q * 32) & (0xffffffffu >> (31 - min(left, 31))) : 0u;
                 }
             };
-            if (__any_sync(0xffffffffu, need)) {
-                const float alpha = (need && m_ref != -INFINITY) ? ex2_fast_f(m_ref - m_new) : 1.f;
-                if (c > 0) {
-                    wait_landed();
-#pragma unroll
-                    for (int e0 = 0; e0 < HD; e0 += 32) {
-                        uint32_t o[32];
-                        tmem_ld32(T_O + e0, o);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-                        tmem_st32(T_O + e0, o);
-                    }
-                }
-                l_run *= alpha;
-                m_ref = m_new;
+            int jt = mine > 0 ? tile_at(0) : 0, jt1 = mine > 1 ? tile_at(1) : 0;
+            uint32_t kws[TKF / 32], kws1[TKF / 32];
+            if constexpr (FINE) {
+                if (mine > 0) keep_words(jt * TKF, kws);
             }
-            const float noff = m_ref == -INFINITY ? 0.f : -m_ref;
-            l_run += exp_row(v, sl2, noff, T_P, &bars[F4_PE + w], &bars[F4_P + w], lane, wait_landed);
-        }
-        // ------------------------------------------------------------ epilogue
-        if constexpr (PAIR) {
-            if (mine > 0) {
-                const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
-                mbar_wait(&bars[F4_O + w], (mine - 1) & 1, ab);
+            for (int c = 0; c < mine; ++c) {
+                const int x = (g0 + o.item(w, c)) % NX;
+                const int j0 = jt * TKF;
+                const bool edge = (causal && j0 + TKF - 1 > iw) || j0 + TKF > n;   // entries dropped by position
+                jt = jt1;
+                if (c + 2 < mine) jt1 = tile_at(c + 2);
+                if constexpr (FINE) {
+                    if (c + 1 < mine) keep_words(jt * TKF, kws1);
+                }
+                mbar_wait(&bars[F4_S + w], (c0 + c) & 1, ab);
                 tcgen05_fence_after();
-                const int ic = ig < n ? ig : 0;
-                __nv_bfloat16 *po = a.O + ((size_t)bh * n + ic) * HD;
+                uint32_t v[TKF];   // the whole row of raw scores in registers: four loads in flight, one wait
 #pragma unroll
-                for (int c = 0; c < HD; c += 32) {
-                    uint32_t o[32];
-                    tmem_ld32(T_O + c, o);
-                    tmem_wait_ld();
-                    if (ig < n) {
+                for (int e = 0; e < TKF; e += 32) tmem_ld32(tm + x * 128 + lane_addr + e, *reinterpret_cast<uint32_t(*)[32]>(&v[e]));
+                tmem_wait_ld();
+                tcgen05_fence_before();
+                warp_arrive_f(&bars[F4_XF + x], lane);   // the buffer may take the next S
+                if constexpr (FINE) {
 #pragma unroll
-                        for (int e = 0; e < 32; e += 8) {
-                            float y[8];
+                    for (int q = 0; q < TKF / 32; ++q) {
+                        if (__all_sync(0xffffffffu, kws[q] == 0xffffffffu)) continue;
 #pragma unroll
-                            for (int u = 0; u < 8; ++u) y[u] = __uint_as_float(o[e + u]) * inv;
-                            *reinterpret_cast<uint4 *>(po + c + e) = make_uint4(pack_bf16(y[0], y[1]), pack_bf16(y[2], y[3]),
-                                                                                pack_bf16(y[4], y[5]), pack_bf16(y[6], y[7]));
+                        for (int e = 0; e < 32; ++e)
+                            if (!(kws[q] & (1u << e))) v[q * 32 + e] = 0xff800000u;   // -inf
+                    }
+                } else if (edge) {
+                    const int keep = min(n, causal ? ig + 1 : n) - j0;   // the row keeps its first `keep` entries of the tile
+#pragma unroll
+                    for (int e = 0; e < TKF; ++e)
+                        if (e >= keep) v[e] = 0xff800000u;   // -inf
+                }
+                const float m_tile = row_max(v) * sl2;   // scale > 0: the maximum commutes with it
+                bool need = m_tile > m_ref + kRescaleThreshold || (m_ref == -INFINITY && m_tile != -INFINITY);
+                float m_new = need ? fmaxf(m_ref, m_tile) : m_ref;
+                if (PAIR && c - 1u < kExactTiles && m_ref != -INFINITY && m_tile != -INFINITY) {
+                    // the next reference from which the tile's maximum is a whole number of powers of two away, by less than one
+                    // unit up also where the sum is rounded (references of 2^24 and more)
+                    m_new = m_tile > m_ref ? m_tile : fminf(fmaxf(m_tile + ceilf(m_ref - m_tile), m_ref), m_ref + 1.f);
+                    need = true;
+                }
+                // O_w += P V of this warpgroup's previous item: it reads P_w and adds to O_w
+                bool landed = c == 0;
+                auto wait_landed = [&] {
+                    if (!landed) {
+                        mbar_wait(&bars[F4_O + w], (c0 + c - 1) & 1, ab);
+                        tcgen05_fence_after();
+                        landed = true;
+                    }
+                };
+                if (__any_sync(0xffffffffu, need)) {
+                    const float alpha = (need && m_ref != -INFINITY) ? ex2_fast_f(m_ref - m_new) : 1.f;
+                    if (c > 0) {
+                        wait_landed();
+#pragma unroll
+                        for (int e0 = 0; e0 < HD; e0 += 32) {
+                            uint32_t ov[32];
+                            tmem_ld32(T_O + e0, ov);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int e = 0; e < 32; ++e) ov[e] = __float_as_uint(__uint_as_float(ov[e]) * alpha);
+                            tmem_st32(T_O + e0, ov);
                         }
                     }
+                    l_run *= alpha;
+                    m_ref = m_new;
                 }
-                if (ig < n) a.LSE[(size_t)bh * n + ig] = row_lse(m_ref, l_run);
+                const float noff = m_ref == -INFINITY ? 0.f : -m_ref;
+                l_run += exp_row(v, sl2, noff, T_P, &bars[F4_PE + w], &bars[F4_P + w], lane, wait_landed);
+                if constexpr (FINE) {
+#pragma unroll
+                    for (int q = 0; q < TKF / 32; ++q) kws[q] = kws1[q];
+                }
             }
-        } else {
-            // merge the two partial softmaxes
-            xm[w * 128 + row] = m_ref;
-            xl[w * 128 + row] = l_run;
-            named_bar_sync_f(1, kSoftmaxThreads);
-            const float m0 = xm[row], m1 = xm[128 + row], l0 = xl[row], l1 = xl[128 + row];
-            const float m_all = fmaxf(m0, m1);
-            const float a0 = m0 == -INFINITY ? 0.f : ex2_fast_f(m0 - m_all), a1 = m1 == -INFINITY ? 0.f : ex2_fast_f(m1 - m_all);
-            const float l_tot = a0 * l0 + a1 * l1;
-            const float inv = l_tot > 0.f ? 1.f / l_tot : 0.f;
-            const float c0 = a0 * inv, c1 = a1 * inv;
-            // the other warpgroup's last product: it may be two completions of its barrier ahead of what this one has seen of it,
-            // but none can follow the last
-            if (n0 > 0) mbar_wait(&bars[F4_O], (n0 - 1) & 1, ab);
-            if (n1 > 0) mbar_wait(&bars[F4_O + 1], (n1 - 1) & 1, ab);
-            tcgen05_fence_after();
+            g0 += o.items;
+            c0 += mine;
+            // -------------------------------------------------------- epilogue, while S of the next unit of work is formed
             const int ic = ig < n ? ig : 0;
-            __nv_bfloat16 *po = a.O + ((size_t)bh * n + ic) * HD + w * (HD / 2);
+            if constexpr (PAIR) {
+                if (mine > 0) {
+                    const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+                    mbar_wait(&bars[F4_O + w], (c0 - 1) & 1, ab);
+                    tcgen05_fence_after();
+                    __nv_bfloat16 *po = a.O + ((size_t)bh * n + ic) * HD;
 #pragma unroll
-            for (int c = 0; c < HD / 2; c += 32) {
-                uint32_t v0[32], v1[32];
-                if (n0 > 0) tmem_ld32(tm + C::tO + lane_addr + w * (HD / 2) + c, v0);
-                if (n1 > 0) tmem_ld32(tm + C::tO + HD + lane_addr + w * (HD / 2) + c, v1);
-                tmem_wait_ld();
-                float o[32];
+                    for (int e0 = 0; e0 < HD; e0 += 32) {
+                        uint32_t ov[32];
+                        tmem_ld32(T_O + e0, ov);
+                        tmem_wait_ld();
+                        if (ig < n) {
 #pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    // a partial accumulator that never received a product holds stale bits: select, do not multiply
-                    const float x0 = n0 > 0 ? __uint_as_float(v0[e]) * c0 : 0.f;
-                    const float x1 = n1 > 0 ? __uint_as_float(v1[e]) * c1 : 0.f;
-                    o[e] = x0 + x1;
+                            for (int e = 0; e < 32; e += 16) {
+                                uint32_t y[8];
+#pragma unroll
+                                for (int u = 0; u < 8; ++u)
+                                    y[u] = pack_bf16(__uint_as_float(ov[e + 2 * u]) * inv, __uint_as_float(ov[e + 2 * u + 1]) * inv);
+                                store32(po + e0 + e, y, wide);
+                            }
+                        }
+                    }
+                    if (ig < n) a.LSE[(size_t)bh * n + ig] = row_lse(m_ref, l_run);
                 }
-                if (ig < n) {
+            } else {
+                // merge the two partial softmaxes
+                xm[w * 128 + row] = m_ref;
+                xl[w * 128 + row] = l_run;
+                named_bar_sync_f(1, kSoftmaxThreads);
+                const float m0 = xm[row], m1 = xm[128 + row], l0 = xl[row], l1 = xl[128 + row];
+                const float m_all = fmaxf(m0, m1);
+                const float a0 = m0 == -INFINITY ? 0.f : ex2_fast_f(m0 - m_all), a1 = m1 == -INFINITY ? 0.f : ex2_fast_f(m1 - m_all);
+                const float l_tot = a0 * l0 + a1 * l1;
+                const float inv = l_tot > 0.f ? 1.f / l_tot : 0.f;
+                const float s0 = a0 * inv, s1 = a1 * inv;
+                // the other warpgroup's last product as well: that warpgroup has come this far, so it has seen the one before
+                // complete, and the barrier is at most one completion behind
+                const int c_0 = w == 0 ? c0 : g0 - c0, c_1 = w == 0 ? g0 - c0 : c0;
+                if (f.n0 > 0) mbar_wait(&bars[F4_O], (c_0 - 1) & 1, ab);
+                if (f.n1 > 0) mbar_wait(&bars[F4_O + 1], (c_1 - 1) & 1, ab);
+                tcgen05_fence_after();
+                __nv_bfloat16 *po = a.O + ((size_t)bh * n + ic) * HD + w * (HD / 2);
 #pragma unroll
-                    for (int e = 0; e < 32; e += 8)
-                        *reinterpret_cast<uint4 *>(po + c + e) = make_uint4(pack_bf16(o[e], o[e + 1]), pack_bf16(o[e + 2], o[e + 3]),
-                                                                            pack_bf16(o[e + 4], o[e + 5]), pack_bf16(o[e + 6], o[e + 7]));
+                for (int e0 = 0; e0 < HD / 2; e0 += 16) {
+                    uint32_t v0[16], v1[16], z[8];
+                    tmem_ld16(tm + C::tO + lane_addr + w * (HD / 2) + e0, v0);
+                    tmem_ld16(tm + C::tO + HD + lane_addr + w * (HD / 2) + e0, v1);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        // a partial accumulator that never received a product holds stale bits: select, do not multiply
+                        float y[2];
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const float x1 = f.n1 > 0 ? __uint_as_float(v1[2 * u + e]) * s1 : 0.f;
+                            y[e] = f.n0 > 0 ? fmaf(__uint_as_float(v0[2 * u + e]), s0, x1) : x1;
+                        }
+                        z[u] = pack_bf16(y[0], y[1]);
+                    }
+                    if (ig < n) store32(po + e0, z, wide);
                 }
+                if (w == 0 && ig < n) a.LSE[(size_t)bh * n + ig] = row_lse(m_all, l_tot);
+                // both accumulators and the exchange buffers have been read: P of the next unit of work may be handed over
+                tcgen05_fence_before();
+                named_bar_sync_f(1, kSoftmaxThreads);
             }
-            if (w == 0 && ig < n) a.LSE[(size_t)bh * n + ig] = row_lse(m_all, l_tot);
         }
     }
     tcgen05_fence_before();

@@ -299,6 +299,44 @@ __device__ __forceinline__ uint32_t pack_bf16_rest(float x, float y, uint32_t hi
     return pack_bf16(x - __uint_as_float(hi << 16), y - __uint_as_float(hi & 0xffff0000u));
 }
 
+// ------------------------------------------------------------------ schedule
+// The hardware's scheduler hands CTAs of the grid that have not started yet to CTAs that run (cluster launch control): the
+// answer, 16 bytes, arrives in shared memory and reports to `bar`.  After an answer without work no further one may be asked for.
+__device__ __forceinline__ void clc_request(void *answer, uint64_t *bar)
+{
+    mbar_expect_tx(bar, 16);
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+                 ::"r"(smem_u32(answer)), "r"(smem_u32(bar)) : "memory");
+}
+// The block index that was handed over; false: there is none left.
+__device__ __forceinline__ bool clc_answer(const void *answer, int &bx, int &by)
+{
+    uint32_t ok, x, y;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b128 r;\n\t.reg .b32 z, w;\n\t"
+        "ld.shared.b128 r, [%3];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t"
+        "mov.b32 %1, 0;\n\tmov.b32 %2, 0;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%1, %2, z, w}, r;\n\t}"
+        : "=r"(ok), "=r"(x), "=r"(y) : "r"(smem_u32(answer)) : "memory");
+    bx = (int)x; by = (int)y;
+    fence_proxy_async_smem();   // read before the next answer is written
+    return ok != 0;
+}
+
+// 32 bytes to global memory (a whole sector); `wide`: the address is a multiple of 32, else of 16
+__device__ __forceinline__ void store32(void *to, const uint32_t (&v)[8], bool wide)
+{
+    if (wide) {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(to), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
+                     "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+    } else {
+        reinterpret_cast<uint4 *>(to)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+        reinterpret_cast<uint4 *>(to)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+    }
+}
+
 }  // namespace tc
 
 // ------------------------------------------------------------------ host: tensor maps
