@@ -60,7 +60,7 @@ struct Problem {
     attn_cfg cfg;                     // resolved: algo and tiles are final
     // workspace sections (device)
     uint32_t *status;                 // 4-byte status word
-    float *D;                         // [BH * stat_stride]
+    float *D;                         // [BH * stat_stride]: D on the FMA path, -scale * D on the tensor-core paths
     float *nLSE2;                     // [BH * stat_stride]: -LSE * log2(e), tensor-core backward only
     int *row_ptr, *col_idx;           // block-CSR of the mask: [mask_heads][nb+1], [mask_heads][nb*nb]
     int *col_ptr, *row_idx;           // block-CSC
@@ -148,7 +148,7 @@ size_t bwd_least_workspace_bytes(int n, int d, int heads, int batch, const attn_
 // Tensor-core path (attn_tc_*.cu)
 attn_status tc_fwd(const Problem &p);
 attn_status tc_bwd(const Problem &p);
-attn_status tc_bwd_dq(const Problem &p);   // query-stationary dQ without atomics (needs p.D = scale*D, p.nLSE2)
+attn_status tc_bwd_dq(const Problem &p);   // query-stationary dQ without atomics (needs p.D = -scale*D, p.nLSE2)
 attn_status mat_bwd(const Problem &p);
 bool tc_cfg_supported(int d, const attn_cfg &cfg, int backward);
 size_t tc_cfg_onchip_bytes(int d, const attn_cfg &cfg, int backward);

@@ -274,12 +274,12 @@ mat_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ 
 
 // phase 3: dS = P o (scale dP - scale D), 8 elements per thread per step
 __global__ void __launch_bounds__(256) mat_ds_kernel(const uint4 *__restrict__ P, const uint4 *__restrict__ dP,
-                                                     uint4 *__restrict__ dS, const float *__restrict__ Ds, size_t nvec,
+                                                     uint4 *__restrict__ dS, const float *__restrict__ nDs, size_t nvec,
                                                      int n, float scale)
 {
     const int vec_per_row = n / 8;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvec; i += (size_t)gridDim.x * blockDim.x) {
-        const float d = Ds[i / vec_per_row];
+        const float d = nDs[i / vec_per_row];
         const uint4 p = P[i], q = dP[i];
         const __nv_bfloat162 *pp = reinterpret_cast<const __nv_bfloat162 *>(&p);
         const __nv_bfloat162 *qq = reinterpret_cast<const __nv_bfloat162 *>(&q);
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(256) mat_ds_kernel(const uint4 *__restrict__ P
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const float2 fp = __bfloat1622float2(pp[e]), fq = __bfloat1622float2(qq[e]);
-            o[e] = pack_bf16(fp.x * fmaf(fq.x, scale, -d), fp.y * fmaf(fq.y, scale, -d));
+            o[e] = pack_bf16(fp.x * fmaf(fq.x, scale, d), fp.y * fmaf(fq.y, scale, d));
         }
         dS[i] = make_uint4(o[0], o[1], o[2], o[3]);
     }

@@ -38,27 +38,39 @@ using namespace bwdk;
 constexpr int TQ = 128;
 template <int HD>
 struct BwdSmem {
+    static constexpr int NS = HD == 64 ? 3 : 2;           // stages of Q, dO and the row statistics
+    static constexpr int NdS = HD == 64 ? 2 : 1;          // buffers of dS^T
     static constexpr uint32_t kSlabs = HD / 64;
     static constexpr uint32_t kTile = kSlabs * SLAB;      // one [128][HD] bf16 tile
     static constexpr uint32_t oK = 0;
     static constexpr uint32_t oV = oK + kTile;
-    static constexpr uint32_t oQ = oV + kTile;            // 2 stages
-    static constexpr uint32_t odO = oQ + 2 * kTile;       // 2 stages
-    static constexpr uint32_t odS = odO + 2 * kTile;      // [128 keys][128 queries] bf16, 2 slabs
-    static constexpr uint32_t oLSE = odS + 2 * SLAB;      // 2 stages x 128 floats
-    static constexpr uint32_t oD = oLSE + 2 * 128 * 4;
-    static constexpr uint32_t oBar = oD + 2 * 128 * 4;    // mbarriers (8 bytes each)
-    static constexpr uint32_t oMisc = oBar + 24 * 8;      // tmem base, abort flag
-    static constexpr uint32_t kBytes = oMisc + 64;
+    static constexpr uint32_t oQ = oV + kTile;            // NS stages
+    static constexpr uint32_t odO = oQ + NS * kTile;
+    static constexpr uint32_t odS = odO + NS * kTile;     // [128 keys][128 queries] bf16, 2 slabs
+    static constexpr uint32_t oLSE = odS + NdS * 2 * SLAB;
+    static constexpr uint32_t oD = oLSE + NS * 128 * 4;
+    static constexpr uint32_t oBar = oD + NS * 128 * 4;    // mbarriers (8 bytes each)
+    static constexpr uint32_t oWork = oBar + 32 * 8;      // two slots of FusedWork, the answer of the scheduler
+    static constexpr uint32_t oTile = oWork + 2 * 32 + 16;// query tile of the last four loads
+    static constexpr uint32_t oMisc = oTile + 16;         // tmem base, abort flag
+    static constexpr uint32_t kBytes = oMisc + 16;
     static_assert(kBytes <= 227 * 1024, "shared memory budget");
 };
 
-
 using TileIter = TileIterT<TQ>;
 
-// barrier indices of the fused kernel: every barrier exists once per 64-query half of a tile
-enum { V2_KV = 0, V2_QFULL = 1, V2_QEMPTY = 3, V2_S = 5, V2_DP = 7, V2_P = 9, V2_DS = 11, V2_DQ = 13, V2_DQDONE = 15, V2_SLD = 17,
-       V2_DPLD = 19, V2_DQREL = 21 };
+// barrier indices of the fused kernel; P exists once per 64-query half of a tile
+enum { V2_KF = 0, V2_KE = 1, V2_VF = 2, V2_VE = 3, V2_QFULL = 4, V2_QEMPTY = 7, V2_S = 10, V2_DP = 11, V2_DQ = 12, V2_CLC = 13, V2_WF = 14,
+       V2_WE = 16, V2_SLD = 18, V2_DPLD = 19, V2_DS = 20, V2_P = 21, V2_DQDONE = 23, V2_DQREL = 24 };
+
+// One unit of work of the fused kernel: a key tile of one head and the query tiles that it visits
+struct FusedWork {
+    int jt, bh, count;   // jt = -1: there is no more work
+    int first;           // the first query tile, or its place in the list
+    const int *rows;     // query blocks of a mask with lists
+    int pad[2];
+};
+static_assert(sizeof(FusedWork) == 32, "two slots in shared memory");
 
 
 // ---------------------------------------------------------------------------------------
@@ -176,7 +188,7 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                 if (k >= 2) mbar_wait(&bars[KD_LEMPTY + s2], ((k >> 1) - 1) & 1, ab);
                 mbar_expect_tx(&bars[KD_LFULL + s2], 2 * rows * 4);
                 bulk_load_1d(smem + L::oLSE + s2 * 512, a.nLSE2 + bh * a.ns + i0, rows * 4, &bars[KD_LFULL + s2]);
-                bulk_load_1d(smem + L::oD + s2 * 512, a.Ds + bh * a.ns + i0, rows * 4, &bars[KD_LFULL + s2]);
+                bulk_load_1d(smem + L::oD + s2 * 512, a.nDs + bh * a.ns + i0, rows * 4, &bars[KD_LFULL + s2]);
                 if (k >= 2) mbar_wait(&bars[KD_OEMPTY + s2], ((k >> 1) - 1) & 1, ab);
                 mbar_expect_tx(&bars[KD_OFULL + s2], L::kTile);
 #pragma unroll
@@ -369,10 +381,10 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                     for (int q = 0; q < 4; ++q) {
                         const float4 dsc = sDs[part * 4 + q];
                         const float *p4 = &p[part * 16 + q * 4];
-                        float d0 = p4[0] * fmaf(__uint_as_float(dv[q * 4 + 0]), a.scale, -dsc.x);
-                        float d1 = p4[1] * fmaf(__uint_as_float(dv[q * 4 + 1]), a.scale, -dsc.y);
-                        float d2 = p4[2] * fmaf(__uint_as_float(dv[q * 4 + 2]), a.scale, -dsc.z);
-                        float d3 = p4[3] * fmaf(__uint_as_float(dv[q * 4 + 3]), a.scale, -dsc.w);
+                        float d0 = p4[0] * fmaf(__uint_as_float(dv[q * 4 + 0]), a.scale, dsc.x);
+                        float d1 = p4[1] * fmaf(__uint_as_float(dv[q * 4 + 1]), a.scale, dsc.y);
+                        float d2 = p4[2] * fmaf(__uint_as_float(dv[q * 4 + 2]), a.scale, dsc.z);
+                        float d3 = p4[3] * fmaf(__uint_as_float(dv[q * 4 + 3]), a.scale, dsc.w);
                         if (masked) {   // stale tail entries of the row vectors may be anything: select, do not multiply
                             d0 = p4[0] != 0.f ? d0 : 0.f; d1 = p4[1] != 0.f ? d1 : 0.f;
                             d2 = p4[2] != 0.f ? d2 : 0.f; d3 = p4[3] != 0.f ? d3 : 0.f;
@@ -445,10 +457,10 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                         // bf16 -> fp32 is a 16-bit shift; a masked entry has p = 0 and a finite dP, so its dS is an exact zero
                         const float p0 = __uint_as_float(ppack[q * 2] << 16), p1 = __uint_as_float(ppack[q * 2] & 0xffff0000u);
                         const float p2 = __uint_as_float(ppack[q * 2 + 1] << 16), p3 = __uint_as_float(ppack[q * 2 + 1] & 0xffff0000u);
-                        float d0 = p0 * fmaf(__uint_as_float(dv[q * 4 + 0]), a.scale, -dsc.x);
-                        float d1 = p1 * fmaf(__uint_as_float(dv[q * 4 + 1]), a.scale, -dsc.y);
-                        float d2 = p2 * fmaf(__uint_as_float(dv[q * 4 + 2]), a.scale, -dsc.z);
-                        float d3 = p3 * fmaf(__uint_as_float(dv[q * 4 + 3]), a.scale, -dsc.w);
+                        float d0 = p0 * fmaf(__uint_as_float(dv[q * 4 + 0]), a.scale, dsc.x);
+                        float d1 = p1 * fmaf(__uint_as_float(dv[q * 4 + 1]), a.scale, dsc.y);
+                        float d2 = p2 * fmaf(__uint_as_float(dv[q * 4 + 2]), a.scale, dsc.z);
+                        float d3 = p3 * fmaf(__uint_as_float(dv[q * 4 + 3]), a.scale, dsc.w);
                         if (masked) {   // stale tail entries of the row vectors may be anything: select, do not multiply
                             d0 = p0 != 0.f ? d0 : 0.f; d1 = p1 != 0.f ? d1 : 0.f;
                             d2 = p2 != 0.f ? d2 : 0.f; d3 = p3 != 0.f ? d3 : 0.f;
@@ -523,7 +535,18 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
 //              memory, the reducers done with dQ^T(k-1)); dK goes first because it releases the Q / dO stage
 //
 // The exp / dS warps keep P only as the bf16 pairs they hand to the dV product, and form dS from
-// those.  Registers are traded between the warpgroups after launch (setmaxnreg).
+// those, two entries an instruction (fma.rn.f32x2: the roundings of the scalar forms; -scale D comes from the pre-pass).
+// Registers are traded between the warpgroups after launch (setmaxnreg).
+//
+// A CTA stays on its SM and takes the block indices of CTAs that have not started yet (cluster launch control); the loading
+// warp publishes each key tile in one of two slots, and K_j, V_j, the first Q and dO and S^T of the next key tile come while dK
+// and dV of this one are written out.  With a CTA per key tile 8.7 us a CTA passed outside its tiles.  What an issuing thread
+// does between its products counts twice: testing for the first tile of a unit inside the loop, instead of ahead of it, cost
+// 3.5 % at d = 128 and 13 % at d = 64; barriers merged to save it two waits a tile made no difference at d = 128 and cost 7 %
+// at d = 64 (dV then competes with S^T and dP^T for the pipe).
+// Before and now, kernel alone: 32 heads, n = 8192, d = 128, causal 1347 -> 1291 us; the same, d = 64, no mask 1897 -> 1664; 64
+// heads, n = 2048, d = 64 272 -> 238; window of 512 keys, 16 heads, n = 4096, d = 128 109 -> 83 (half of it from the keep words,
+// applied to the packed pairs and only in warps that drop something); blocks of 64, 10 %, 16 heads, n = 8192, d = 64 559 -> 449.
 template <int N> __device__ __forceinline__ void setmaxnreg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
 template <int N> __device__ __forceinline__ void setmaxnreg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 constexpr int kThreadsFused = 512 + 256 + 128;  // 16 exp/dS warps, 8 reducer warps, two issuer warps, TMA producer warp, 1 idle warp
@@ -533,30 +556,55 @@ constexpr int kThreadsFused = 512 + 256 + 128;  // 16 exp/dS warps, 8 reducer wa
 struct FusedRegs {
     static constexpr int kExp = 88, kReduce = 48, kIssue = 56;
 };
+// P of two entries from their scores and -LSE log2(e)
+__device__ __forceinline__ void p_pair(uint32_t v0, uint32_t v1, float s, float n0, float n1, float &p0, float &p1)
+{
+    uint64_t x, y, z;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(v0), "r"(v1));
+    asm("mov.b64 %0, {%1, %1};" : "=l"(y) : "f"(s));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(n0), "f"(n1));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(x) : "l"(x), "l"(y), "l"(z));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(p0), "=f"(p1) : "l"(x));
+    p0 = ex2_approx(p0);
+    p1 = ex2_approx(p1);
+}
+// dS of two entries from their P (bf16 pair), dP and -scale * D
+__device__ __forceinline__ void ds_pair(uint32_t pk, uint32_t v0, uint32_t v1, float s, float n0, float n1, float &d0, float &d1)
+{
+    uint64_t x, y, z, w;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(v0), "r"(v1));
+    asm("mov.b64 %0, {%1, %1};" : "=l"(y) : "f"(s));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(n0), "f"(n1));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(w) : "r"(pk << 16), "r"(pk & 0xffff0000u));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(x) : "l"(x), "l"(y), "l"(z));
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(x) : "l"(x), "l"(w));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(x));
+}
 template <int HD, bool FINE>
 __global__ void __launch_bounds__(kThreadsFused, 1)
 tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CUtensorMap mK_,
-                 const __grid_constant__ CUtensorMap mV, const __grid_constant__ CUtensorMap mdO,
-                 const __grid_constant__ CUtensorMap mdK, const __grid_constant__ CUtensorMap mdV, const BwdArgs a)
+                 const __grid_constant__ CUtensorMap mV, const __grid_constant__ CUtensorMap mdO, const BwdArgs a)
 {
     // d = 64: the dQ^T product needs M = 128, so the K tile's second 64-wide slab of M is an all-zero slab
     using L = BwdSmem<HD>;
     constexpr uint32_t oZero = (L::kBytes + 1023u) & ~1023u;
     constexpr int kHalfWarps = 8;     // exp / dS warps per half
-    constexpr int kReduceWarps = 4;   // reducer warps per half
-    static_assert(L::oMisc - L::oBar >= 23 * 8, "barrier area");
+    constexpr int kReduceWarps = HD / 32;   // reducer warps per half that have rows of dQ^T (d = 64: lanes 64..127 of the padded product hold zeros)
+    constexpr int NS = L::NS;
+    auto stage_of = [](int kt) { return NS == 2 ? kt & 1 : kt % 3; };
+    auto phase_of = [](int kt) { return NS == 2 ? (kt >> 1) & 1 : (kt / 3) & 1; };
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L::oBar);
     uint32_t *tmem_base_s = reinterpret_cast<uint32_t *>(smem + L::oMisc);
     volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(smem + L::oMisc + 4);
+    volatile FusedWork *slots = reinterpret_cast<volatile FusedWork *>(smem + L::oWork);
+    uint8_t *answer = smem + L::oWork + 2 * sizeof(FusedWork);
     const Abort ab{abort_flag, a.status};
 
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-    // launch order: heads in groups of `a.group`, inside a group key tile major -- with a causal
-    // mask the CTAs of a group then start longest first, which evens out the tail of the grid
-    const int jt = blockIdx.x / a.group;
-    const long bh = (long)blockIdx.y * a.group + blockIdx.x % a.group;
-    const int j0 = jt * TK, n = a.n;
+    const int n = a.n;
+    const bool lists = mask_is_block(a.mask_kind), causal = mask_is_causal(a.mask_kind);
+    const int sub = lists ? a.block / TQ : 1;
 
     if ((smem_u32(smem) & 1023u) != 0) {
         chain_wait();
@@ -565,20 +613,14 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constan
     }
     if (tid == 0) {
         *abort_flag = 0;
-        mbar_init(&bars[V2_KV], 1);
-        for (int h = 0; h < 2; ++h) {
-            mbar_init(&bars[V2_QFULL + h], 1);
-            mbar_init(&bars[V2_QEMPTY + h], 1);
-            mbar_init(&bars[V2_S + h], 1);
-            mbar_init(&bars[V2_DP + h], 1);
-            mbar_init(&bars[V2_SLD + h], 2 * kHalfWarps);     // SLD, DPLD, DS, DQDONE, DQREL: index 0 serves both halves
-            mbar_init(&bars[V2_DPLD + h], 2 * kHalfWarps);
-            mbar_init(&bars[V2_P + h], kHalfWarps);
-            mbar_init(&bars[V2_DS + h], 2 * kHalfWarps);
-            mbar_init(&bars[V2_DQ + h], 1);
-            mbar_init(&bars[V2_DQDONE + h], 2 * kReduceWarps);
-            mbar_init(&bars[V2_DQREL + h], 2 * kReduceWarps);
-        }
+        for (int b = 0; b < V2_SLD; ++b) mbar_init(&bars[b], b >= V2_WE ? 2 + 2 * kHalfWarps + 2 * kReduceWarps : 1);   // WE: every reader of a slot
+        mbar_init(&bars[V2_SLD], 2 * kHalfWarps);
+        mbar_init(&bars[V2_DPLD], 2 * kHalfWarps);
+        mbar_init(&bars[V2_DS], 2 * kHalfWarps);
+        mbar_init(&bars[V2_P], kHalfWarps);
+        mbar_init(&bars[V2_P + 1], kHalfWarps);
+        mbar_init(&bars[V2_DQDONE], 2 * kReduceWarps);
+        mbar_init(&bars[V2_DQREL], 2 * kReduceWarps);
         fence_barrier_init();
         prefetch_tensormap(&mQ); prefetch_tensormap(&mK_); prefetch_tensormap(&mV); prefetch_tensormap(&mdO);
     }
@@ -600,109 +642,146 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constan
     const uint32_t T_A2 = kSplitA ? tm + 384 : T_A;
     constexpr uint32_t HALF_ROWS = 64 * 128;   // byte offset of rows 64.. inside a [128][64] slab
 
-    const TileIter iter(a, jt, bh);
+    // the t-th unit of work of this CTA as the loading warp has published it (false: there is none); it stays in its slot until
+    // both issuers, the exp / dS warps and the reducers have arrived on WE
+    auto work = [&](int t) { return mbar_wait(&bars[V2_WF + (t & 1)], (t >> 1) & 1, ab) && slots[t & 1].jt >= 0; };
+    auto query_tile = [&](const int *rows, int e) { return !lists ? e : sub == 1 ? rows[e] : rows[e / sub] * sub + e % sub; };
+    // query tile of the kt-th load; the fourth load after it needs dP^T of tile kt + 2, and so dQ^T(kt) read by the reducers
+    volatile int *tiles = reinterpret_cast<volatile int *>(smem + L::oTile);
 
+    // In every role kt counts the query tiles of all units of work so far (a wait for what belongs to tile -1 returns at once: a
+    // new barrier counts as complete in the phase before its first): the barriers run on from one unit to the next, and
+    // what the next one needs first is loaded and formed while dK and dV of this one are written out.
     if (warp >= 24) {
         setmaxnreg_dec<FusedRegs::kIssue>();
-        if (warp == 25 && lane == 0) {
-            // ------------------------------------------------------------ TMA producer: every load, as soon as its stage is free
-            auto issue_load = [&](int it, int s) {
-                const int i0 = it * TQ;
-                const uint32_t rows = min(TQ, a.ns - i0);
-                uint64_t *bar = &bars[V2_QFULL + s];
-                mbar_expect_tx(bar, 2 * L::kTile + 2 * rows * 4);
-#pragma unroll
-                for (uint32_t sl = 0; sl < L::kSlabs; ++sl) {
-                    tma_load_3d(smem + L::oQ + s * L::kTile + sl * SLAB, &mQ, bar, sl * 64, i0, (int)bh);
-                    tma_load_3d(smem + L::odO + s * L::kTile + sl * SLAB, &mdO, bar, sl * 64, i0, (int)bh);
+        if (warp == 25) {
+            // ------------------------------------------------------------ TMA producer, and the schedule
+            // launch order: heads in groups of `a.group`, inside a group key tile major -- with a causal
+            // mask the CTAs of a group then start longest first, which evens out the tail of the grid
+            int bx = blockIdx.x, by = blockIdx.y;
+            int kt = 0, nkv = 0;   // query tiles and key tiles loaded so far
+            bool more = true;
+            for (int t = 0; more; ++t) {
+                const int jt = bx / a.group, bh = by * a.group + bx % a.group, j0 = jt * TK;
+                int count, first = 0;
+                const int *rows = nullptr;
+                if (lists) {
+                    // the lists ascend: what lies beyond n is at their end, and (block mask AND causal) what ends before the key
+                    // tile begins at their start
+                    const int J = jt / (a.block / TK);
+                    const long mh = a.mask_heads == 1 ? 0 : bh;
+                    const int *cp = a.col_ptr + mh * 2 * a.nb + 2 * J;
+                    const int start = cp[0], raw = (cp[1] - start) * sub;
+                    rows = a.row_idx + mh * (long)a.nb * a.nb + start;
+                    int before = 0, within = 0;
+                    for (int e = lane; e < raw; e += 32) {
+                        const int it = rows[e / sub] * sub + e % sub;
+                        before += causal && it < jt;
+                        within += it * TQ < n;
+                    }
+                    first = __reduce_add_sync(0xffffffffu, before);
+                    count = __reduce_add_sync(0xffffffffu, within) - first;
+                    if (count < 0) count = 0;
+                } else {
+                    first = causal ? jt : 0;
+                    count = (n + TQ - 1) / TQ - first;
                 }
-                bulk_load_1d(smem + L::oLSE + s * 512, a.nLSE2 + bh * a.ns + i0, rows * 4, bar);
-                bulk_load_1d(smem + L::oD + s * 512, a.Ds + bh * a.ns + i0, rows * 4, bar);
-            };
-            mbar_expect_tx(&bars[V2_KV], 2 * L::kTile);
+                if (lane == 0) {
+                    if (t >= 2) mbar_wait(&bars[V2_WE + (t & 1)], ((t >> 1) - 1) & 1, ab);
+                    volatile FusedWork &to = slots[t & 1];
+                    int it = count > 0 ? query_tile(rows, first) : 0;
+                    to.jt = jt; to.bh = bh; to.count = count; to.first = first; to.rows = rows;
+                    mbar_arrive(&bars[V2_WF + (t & 1)]);
+                    for (int k = 0; k < count; ++k, ++kt) {
+                        const int s = stage_of(kt), here = it, i0 = it * TQ;
+                        if (k + 1 < count) it = query_tile(rows, first + k + 1);
+                        // the next unit of work, asked for early enough that the answer is there when the loads get to it
+                        if (k == max(count - 2, 0)) clc_request(answer, &bars[V2_CLC]);
+                        if (k == 0) {
+                            mbar_wait(&bars[V2_VE], (nkv - 1) & 1, ab);   // dP^T of the unit before
+                            mbar_expect_tx(&bars[V2_VF], L::kTile);
 #pragma unroll
-            for (uint32_t sl = 0; sl < L::kSlabs; ++sl) {
-                tma_load_3d(smem + L::oK + sl * SLAB, &mK_, &bars[V2_KV], sl * 64, j0, (int)bh);
-                tma_load_3d(smem + L::oV + sl * SLAB, &mV, &bars[V2_KV], sl * 64, j0, (int)bh);
+                            for (uint32_t sl = 0; sl < L::kSlabs; ++sl)
+                                tma_load_3d(smem + L::oV + sl * SLAB, &mV, &bars[V2_VF], sl * 64, j0, bh);
+                        }
+                        if (kt >= NS) mbar_wait(&bars[V2_QEMPTY + s], phase_of(kt - NS), ab);   // last read by dK of tile kt - NS
+                        {
+                            // negative: position drops some of its entries (causal, or beyond n)
+                            tiles[kt & 3] = (causal && here == jt) || i0 + TQ > n || j0 + TK > n ? here - (1 << 30) : here;
+                            const uint32_t nrows = min(TQ, a.ns - i0);
+                            uint64_t *bar = &bars[V2_QFULL + s];
+                            mbar_expect_tx(bar, 2 * L::kTile + 2 * nrows * 4);
+#pragma unroll
+                            for (uint32_t sl = 0; sl < L::kSlabs; ++sl) {
+                                tma_load_3d(smem + L::oQ + s * L::kTile + sl * SLAB, &mQ, bar, sl * 64, i0, bh);
+                                tma_load_3d(smem + L::odO + s * L::kTile + sl * SLAB, &mdO, bar, sl * 64, i0, bh);
+                            }
+                            bulk_load_1d(smem + L::oLSE + s * 512, a.nLSE2 + (size_t)bh * a.ns + i0, nrows * 4, bar);
+                            bulk_load_1d(smem + L::oD + s * 512, a.nDs + (size_t)bh * a.ns + i0, nrows * 4, bar);
+                        }
+                        if (k == 0) {
+                            mbar_wait(&bars[V2_KE], (nkv - 1) & 1, ab);   // dQ^T of the unit before
+                            mbar_expect_tx(&bars[V2_KF], L::kTile);
+#pragma unroll
+                            for (uint32_t sl = 0; sl < L::kSlabs; ++sl)
+                                tma_load_3d(smem + L::oK + sl * SLAB, &mK_, &bars[V2_KF], sl * 64, j0, bh);
+                        }
+                    }
+                    if (count > 0) ++nkv;
+                    else clc_request(answer, &bars[V2_CLC]);
+                    more = mbar_wait(&bars[V2_CLC], t & 1, ab) && clc_answer(answer, bx, by);
+                    if (!more) {
+                        if (t >= 1) mbar_wait(&bars[V2_WE + ((t + 1) & 1)], (((t + 1) >> 1) - 1) & 1, ab);
+                        slots[(t + 1) & 1].jt = -1;
+                        mbar_arrive(&bars[V2_WF + ((t + 1) & 1)]);
+                    }
+                }
+                more = __shfl_sync(0xffffffffu, (int)more, 0) != 0;
+                bx = __shfl_sync(0xffffffffu, bx, 0);
+                by = __shfl_sync(0xffffffffu, by, 0);
             }
-            int k = 0;
-            for (int idx = 0; idx < iter.raw; ++idx) {
-                const int it = iter.tile(idx);
-                if (it < 0) continue;
-                const int s = k & 1;
-                if (k >= 2) mbar_wait(&bars[V2_QEMPTY + s], ((k - 2) >> 1) & 1, ab);   // last read by dK of tile k-2
-                issue_load(it, s);
-                ++k;
-            }
-            // a key tile without a single query tile (an empty block column): nobody else waits for K_j and V_j, and
-            // the CTA must not exit with their bulk loads still in flight into its shared memory
-            if (k == 0) mbar_wait(&bars[V2_KV], 0, ab);
         } else if (warp == 24 && lane == 0) {
             // ------------------------------------------------------------ MMA issuer A: the products into region A (S^T, dP^T)
             constexpr uint32_t idesc_s = idesc_bf16(128, 128, 0, 0);
-            // low descriptor words (tc_common.cuh): per-step offsets are added as (bytes >> 4)
-            const uint32_t kK = desc_lo_kmajor(smem_u32(smem + L::oK)), kV = desc_lo_kmajor(smem_u32(smem + L::oV));
-            constexpr uint32_t kSlab = SLAB >> 4;
-            // S^T = K_j Q_i^T for the whole tile in stage s
-            auto issue_S = [&](int s) {
-                const uint32_t kQ = desc_lo_kmajor(smem_u32(smem + L::oQ + s * L::kTile));
-#pragma unroll
-                for (int kk = 0; kk < HD / 16; ++kk) {
-                    const uint32_t off = (kk / 4) * kSlab + (kk % 4) * 2;
-                    mma_ss_lo(T_A, kK + off, kQ + off, idesc_s, kk > 0);
+            constexpr uint32_t kSlab = SLAB >> 4;   // low descriptor words (tc_common.cuh): per-step offsets are added as (bytes >> 4)
+            int kt = 0, nkv = 0;
+            for (int t = 0; work(t); ++t) {
+                const int count = slots[t & 1].count;
+                mbar_arrive(&bars[V2_WE + (t & 1)]);
+                const uint32_t kK = desc_lo_kmajor(smem_u32(smem + L::oK)), kV = desc_lo_kmajor(smem_u32(smem + L::oV));
+                if (count > 0) {
+                    mbar_wait(&bars[V2_VF], nkv & 1, ab);
+                    mbar_wait(&bars[V2_KF], nkv & 1, ab);
                 }
-                mma_commit(&bars[V2_S]);
-            };
-            // dP^T = V_j dO_i^T for the whole tile in stage s
-            auto issue_dP = [&](int s) {
-                const uint32_t kdO = desc_lo_kmajor(smem_u32(smem + L::odO + s * L::kTile));
-#pragma unroll
-                for (int kk = 0; kk < HD / 16; ++kk) {
-                    const uint32_t off = (kk / 4) * kSlab + (kk % 4) * 2;
-                    mma_ss_lo(T_A2, kV + off, kdO + off, idesc_s, kk > 0);
-                }
-                mma_commit(&bars[V2_DP]);
-            };
-            int idx = 0, it = -1;
-            while (idx < iter.raw && (it = iter.tile(idx)) < 0) ++idx;
-            if (it >= 0) {
-                mbar_wait(&bars[V2_QFULL], 0, ab);
-                mbar_wait(&bars[V2_KV], 0, ab);
-                tcgen05_fence_after();
-                issue_S(0);
-                if (kSplitA) issue_dP(0);
-            }
-            int k = 0;
-            while (idx < iter.raw) {
-                const int s = k & 1;
-                int nidx = idx + 1, nit = -1;
-                while (nidx < iter.raw && (nit = iter.tile(nidx)) < 0) ++nidx;
-                if constexpr (kSplitA) {
-                    // two regions: S^T(k+1) as soon as S^T(k) has been copied out, dP^T(k+1) as soon as dP^T(k) has been
-                    if (nit >= 0) {
-                        mbar_wait(&bars[V2_SLD], k & 1, ab);
-                        mbar_wait(&bars[V2_QFULL + (s ^ 1)], ((k + 1) >> 1) & 1, ab);
-                        tcgen05_fence_after();
-                        issue_S(s ^ 1);
-                        mbar_wait(&bars[V2_DPLD], k & 1, ab);
-                        tcgen05_fence_after();
-                        issue_dP(s ^ 1);
-                    }
-                } else {
-                    // dP^T = V_j dO_i^T into region A once every exp / dS warp holds its part of S^T in registers
-                    mbar_wait(&bars[V2_SLD], k & 1, ab);
+                for (int k = 0; k < count; ++k, ++kt) {
+                    const int s = stage_of(kt);
+                    // S^T = K_j Q_i^T once region A is free: dP^T of the tile before (d = 64: its S^T) has been copied out
+                    mbar_wait(&bars[kSplitA ? V2_SLD : V2_DPLD], (kt - 1) & 1, ab);
+                    mbar_wait(&bars[V2_QFULL + s], phase_of(kt), ab);
                     tcgen05_fence_after();
-                    issue_dP(s);
-                    // S^T of the next tile into region A as soon as dP^T has been read out of it
-                    if (nit >= 0) {
-                        mbar_wait(&bars[V2_DPLD], k & 1, ab);
-                        mbar_wait(&bars[V2_QFULL + (s ^ 1)], ((k + 1) >> 1) & 1, ab);
-                        tcgen05_fence_after();
-                        issue_S(s ^ 1);
+                    const uint32_t kQ = desc_lo_kmajor(smem_u32(smem + L::oQ + s * L::kTile));
+#pragma unroll
+                    for (int kk = 0; kk < HD / 16; ++kk) {
+                        const uint32_t off = (kk / 4) * kSlab + (kk % 4) * 2;
+                        mma_ss_lo(T_A, kK + off, kQ + off, idesc_s, kk > 0);
                     }
+                    mma_commit(&bars[V2_S]);
+                    // dP^T = V_j dO_i^T once every exp / dS warp holds its part of S^T in registers (d = 64: of the dP^T before)
+                    if (!kSplitA) mbar_wait(&bars[V2_SLD], kt & 1, ab);
+                    else mbar_wait(&bars[V2_DPLD], (kt - 1) & 1, ab);
+                    tcgen05_fence_after();
+                    const uint32_t kdO = desc_lo_kmajor(smem_u32(smem + L::odO + s * L::kTile));
+#pragma unroll
+                    for (int kk = 0; kk < HD / 16; ++kk) {
+                        const uint32_t off = (kk / 4) * kSlab + (kk % 4) * 2;
+                        mma_ss_lo(T_A2, kV + off, kdO + off, idesc_s, kk > 0);
+                    }
+                    mma_commit(&bars[V2_DP]);
                 }
-                ++k;
-                idx = nidx;
+                if (count > 0) {
+                    mma_commit(&bars[V2_VE]);
+                    ++nkv;
+                }
             }
         } else if (warp == 26 && lane == 0) {
             // ------------------------------------------------------------ MMA issuer B: the products that read P^T and dS^T
@@ -711,43 +790,63 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constan
             // goes through the exp / dS warps' barriers.
             constexpr uint32_t idesc_dv = idesc_bf16(128, HD, 0, 1);       // dV (A tmem), dK (A K-major smem)
             constexpr uint32_t idesc_dq = idesc_bf16(128, 128, 1, 1);      // dQ^T
-            const uint32_t mK = desc_lo_mnmajor(smem_u32(smem + L::oK), HD == 64 ? oZero - L::oK : SLAB);
             const uint32_t kdS = desc_lo_kmajor(smem_u32(smem + L::odS)), mdS = desc_lo_mnmajor(smem_u32(smem + L::odS), SLAB);
             constexpr uint32_t kHalf = HALF_ROWS >> 4, kSlab = SLAB >> 4;
-            int k = 0;
-            for (int idx = 0; idx < iter.raw; ++idx) {
-                if (iter.tile(idx) < 0) continue;
-                const int s = k & 1;
-                const uint32_t mdO_ = desc_lo_mnmajor(smem_u32(smem + L::odO + s * L::kTile), SLAB);
-                const uint32_t mQ_ = desc_lo_mnmajor(smem_u32(smem + L::oQ + s * L::kTile), SLAB);
-                if (k == 0) mbar_wait(&bars[V2_KV], 0, ab);
-                mbar_wait(&bars[V2_QFULL + s], (k >> 1) & 1, ab);
-                // dV += P_h^T dO_h, P_h^T in columns 64 h .. 64 h + 31 of region B
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    mbar_wait(&bars[V2_P + h], k & 1, ab);
-                    tcgen05_fence_after();
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        mma_ts_lo(T_dV, T_B + 64 * h + kk * 8, mdO_ + h * kHalf + kk * 128, idesc_dv, (k > 0) || (h > 0) || (kk > 0));
+            int kt = 0, nkv = 0;
+            for (int t = 0; work(t); ++t) {
+                const int count = slots[t & 1].count;
+                mbar_arrive(&bars[V2_WE + (t & 1)]);
+                const uint32_t mK = desc_lo_mnmajor(smem_u32(smem + L::oK), HD == 64 ? oZero - L::oK : SLAB);
+                if (count > 0) {
+                    mbar_wait(&bars[V2_KF], nkv & 1, ab);
+                    // the first dV of a unit overwrites the accumulator of the unit before: both halves' warps have read it
+                    mbar_wait(&bars[V2_P + 1], kt & 1, ab);
                 }
-                // dK += dS^T Q_i first: its completion releases the Q / dO stage, and the load of the tile after next --
-                // two stages only -- is what the next S^T product ends up waiting for.  Then dQ^T = K_j^T dS^T into
-                // region B (this thread's products execute in issue order, so dV has consumed P^T by then).
-                // That the reducers have read all of the previous dQ^T is waited for ahead of dS, which the tile is waiting for
-                if (k > 0) mbar_wait(&bars[V2_DQDONE], (k - 1) & 1, ab);
-                mbar_wait(&bars[V2_DS], k & 1, ab);
-                tcgen05_fence_after();
+                for (int k = 0; k < count; ++k, ++kt) {
+                    const int s = stage_of(kt);
+                    const uint32_t mdO_ = desc_lo_mnmajor(smem_u32(smem + L::odO + s * L::kTile), SLAB);
+                    const uint32_t mQ_ = desc_lo_mnmajor(smem_u32(smem + L::oQ + s * L::kTile), SLAB);
+                    mbar_wait(&bars[V2_QFULL + s], phase_of(kt), ab);
+                    // dV += P_h^T dO_h, P_h^T in columns 64 h .. 64 h + 31 of region B
 #pragma unroll
-                for (int kk = 0; kk < TQ / 16; ++kk)
-                    mma_ss_lo(T_dK, kdS + (kk / 4) * kSlab + (kk % 4) * 2, mQ_ + kk * 128, idesc_dv, (k > 0) || (kk > 0));
-                mma_commit(&bars[V2_QEMPTY + s]);
+                    for (int h = 0; h < 2; ++h) {
+                        mbar_wait(&bars[V2_P + h], kt & 1, ab);
+                        tcgen05_fence_after();
 #pragma unroll
-                for (int kk = 0; kk < TK / 16; ++kk)
-                    mma_ss_lo(T_B, mK + kk * 128, mdS + kk * 128, idesc_dq, kk > 0);
-                mma_commit(&bars[V2_DQ]);
-                ++k;
+                        for (int kk = 0; kk < 4; ++kk)
+                            mma_ts_lo(T_dV, T_B + 64 * h + kk * 8, mdO_ + h * kHalf + kk * 128, idesc_dv, (k > 0) || (h > 0) || (kk > 0));
+                    }
+                    // dQ^T = K_j^T dS^T into region B (this thread's products execute in issue order, so dV has consumed P^T by
+                    // then) and dK += dS^T Q_i.  d = 128: dK first, its completion releases the Q / dO stage, and with two stages
+                    // the load of the tile after next is what the next S^T ends up waiting for.  d = 64: three stages and a
+                    // second buffer of dS^T, so dQ^T, which P^T of the next tile waits for, goes first
+                    // (n = 8192, 32 heads, no mask: 1762 -> 1691 us).
+                    // That the reducers have read all of the previous dQ^T is waited for ahead of dS, which the tile is waiting for
+                    mbar_wait(&bars[V2_DQDONE], (kt - 1) & 1, ab);
+                    mbar_wait(&bars[V2_DS], kt & 1, ab);
+                    tcgen05_fence_after();
+                    const uint32_t ds = L::NdS == 2 ? (kt & 1) * (2 * SLAB >> 4) : 0;
+                    auto issue_dK = [&] {
+#pragma unroll
+                        for (int kk = 0; kk < TQ / 16; ++kk)
+                            mma_ss_lo(T_dK, kdS + ds + (kk / 4) * kSlab + (kk % 4) * 2, mQ_ + kk * 128, idesc_dv, (k > 0) || (kk > 0));
+                        mma_commit(&bars[V2_QEMPTY + s]);
+                    };
+                    if (L::NdS == 1) issue_dK();
+#pragma unroll
+                    for (int kk = 0; kk < TK / 16; ++kk)
+                        mma_ss_lo(T_B, mK + kk * 128, mdS + ds + kk * 128, idesc_dq, kk > 0);
+                    mma_commit(&bars[V2_DQ]);
+                    if (L::NdS == 2) issue_dK();
+                }
+                if (count > 0) {
+                    mma_commit(&bars[V2_KE]);
+                    ++nkv;
+                }
             }
+            // every product has completed before the CTA leaves: the last dQ^T is awaited by the reducers, this thread's last
+            // commit comes after it
+            if (nkv > 0) mbar_wait(&bars[V2_KE], (nkv - 1) & 1, ab);
         }
     } else if (warp >= 16) {
         setmaxnreg_dec<FusedRegs::kReduce>();
@@ -755,198 +854,187 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constan
         // lanes = head-dimension index c, columns = queries: one warp instruction adds 128 contiguous bytes.
         // 32 columns at a time (the reducers run on 48 registers); the half is released after the second load
         const int h = (warp - 16) / 4;
-        const int row = (warp % 4) * 32 + lane;
         const uint32_t lane_addr = (uint32_t)((warp % 4) * 32) << 16;
-        const bool live = (warp % 4) * 32 < HD;   // d = 64: lanes 64..127 of the padded product hold zeros
-        int k = 0;
-        for (int idx = 0; idx < iter.raw; ++idx) {
-            const int it = iter.tile(idx);
-            if (it < 0) continue;
-            const int ig0 = it * TQ + h * 64;
-            float *base = a.dQ_acc + ((size_t)bh * n + ig0) * HD + row;
-            mbar_wait(&bars[V2_DQ], k & 1, ab);
-            tcgen05_fence_after();
+        int kt = 0;
+        for (int t = 0; warp % 4 < kReduceWarps && work(t); ++t) {
+            const int count = slots[t & 1].count;
+            for (int k = 0; k < count; ++k, ++kt) {
+                // the slot is read anew for every tile, ahead of the wait, to save registers
+                const int left = n - query_tile(slots[t & 1].rows, slots[t & 1].first + k) * TQ - h * 64;   // rows of this half that exist
+                float *base = a.dQ_acc + ((size_t)slots[t & 1].bh * n + (n - left)) * HD + (warp % 4) * 32 + lane;
+                mbar_wait(&bars[V2_DQ], kt & 1, ab);
+                tcgen05_fence_after();
 #pragma unroll
-            for (int part = 0; part < 2; ++part) {
-                uint32_t v0[32];
-                if (live) {
+                for (int part = 0; part < 2; ++part) {
+                    uint32_t v0[32];
                     tmem_ld32(T_B + lane_addr + h * 64 + part * 32, v0);
                     tmem_wait_ld();
-                }
-                tcgen05_fence_before();
-                // part 0: the 32 columns that take P^T of the next tile are free; part 1: the whole half is
-                warp_arrive(&bars[part == 0 ? V2_DQREL : V2_DQDONE], lane);
-                if (live) {
-                    if (ig0 + 64 <= n) {
+                    tcgen05_fence_before();
+                    // part 0: the 32 columns that take P^T of the next tile are free; part 1: the whole half is
+                    warp_arrive(&bars[part == 0 ? V2_DQREL : V2_DQDONE], lane);
+                    if (left >= 64) {
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) red_add_f32(base + (size_t)(part * 32 + e) * HD, __uint_as_float(v0[e]));
+                        for (int e = 0; e < 32; ++e) red_add_f32(base + (part * 32 + e) * HD, __uint_as_float(v0[e]));
                     } else {
 #pragma unroll
                         for (int e = 0; e < 32; ++e)
-                            if (ig0 + part * 32 + e < n) red_add_f32(base + (size_t)(part * 32 + e) * HD, __uint_as_float(v0[e]));
+                            if (part * 32 + e < left) red_add_f32(base + (part * 32 + e) * HD, __uint_as_float(v0[e]));
                     }
                 }
             }
-            ++k;
+            warp_arrive(&bars[V2_WE + (t & 1)], lane);
         }
     } else {
         // ------------------------------------------------------------ warps 0-15: exp / dS; warpgroup 2h + qq owns queries 64 h + 32 qq .. + 31
         setmaxnreg_inc<FusedRegs::kExp>();
-        const int h = warp / 8, qq = (warp / 4) & 1;
-        const int row = (warp % 4) * 32 + lane;        // tensor-memory lane = key row inside the tile
-        const uint32_t lane_addr = (uint32_t)((warp % 4) * 32) << 16;
-        const int jg = j0 + row;
-        const float sl2 = a.scale * 1.4426950408889634f;
-        const uint32_t c0 = h * 64 + qq * 32;          // this thread's first column of S^T / dP^T in region A
-        const uint32_t cP = h * 64 + qq * 16;          // and of its bf16 pairs of P^T in region B
-        int k = 0;
-        for (int idx = 0; idx < iter.raw; ++idx) {
-            const int it = iter.tile(idx);
-            if (it < 0) continue;
-            const int s = k & 1, i0 = it * TQ;
-            const float4 *sNL = reinterpret_cast<const float4 *>(smem + L::oLSE + s * 512 + h * 256 + qq * 128);
-            const float4 *sDs = reinterpret_cast<const float4 *>(smem + L::oD + s * 512 + h * 256 + qq * 128);
-            const bool diag = mask_is_causal(a.mask_kind) && it == jt;
-            const int ig0 = i0 + h * 64 + qq * 32;
-            // a mask finer than the tile: the keep bits of this thread's key row and its 32 query columns
-            uint32_t kw = 0xffffffffu;
-            if constexpr (FINE) kw = (ig0 < n && jg < n) ? fine_word(a.fine, a.mask_heads, bh, false, jg, ig0) : 0u;
-            const bool masked = diag || i0 + TQ > n || j0 + TK > n || FINE;
-            mbar_wait(&bars[V2_QFULL + s], (k >> 1) & 1, ab);
-            // the 32 row statistics of this thread's query columns go into registers before the wait for S^T: while the
-            // products stream their operands, a shared-memory load inside the arithmetic below waits a few hundred cycles
-            float4 nlr[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) nlr[q] = sNL[q];
-            mbar_wait(&bars[V2_S], k & 1, ab);
-            tcgen05_fence_after();
-            uint32_t ppack[16];   // P as bf16 pairs: what dV uses, and what dS is formed from
+        // What a thread's place in the tile gives is formed anew where it is used: the row statistics, the scores and P take 80 of
+        // the 88 registers, and a value that is spilled comes back through the shared memory that the products keep busy.
+        struct Place {
+            uint32_t h, qq, row, lane_addr;
+            __device__ __forceinline__ Place()
             {
-                uint32_t sv[32];
-                tmem_ld32(T_A + lane_addr + c0, sv);
-                tmem_wait_ld();
-                tcgen05_fence_before();
-                warp_arrive(&bars[V2_SLD], lane);   // region A may take dP^T
+                uint32_t t;
+                asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
+                h = t >> 8; qq = (t >> 7) & 1u; row = t & 127u; lane_addr = (t & 96u) << 16;
+            }
+            __device__ __forceinline__ uint32_t column() const { return h * 64 + qq * 32; }   // of S^T / dP^T in region A; bf16 pairs of P^T: h * 64 + qq * 16
+        };
+        int kt = 0;
+        for (int t = 0; work(t); ++t) {
+            const int count = slots[t & 1].count, end = kt + count;
+            for (; kt < end; ++kt) {
+                const int s = stage_of(kt);
+                mbar_wait(&bars[V2_QFULL + s], phase_of(kt), ab);
+                // the 32 row statistics of this thread's query columns go into registers before the wait for S^T: while the
+                // products stream their operands, a shared-memory load inside the arithmetic below waits a few hundred cycles
+                float4 nlr[8];
+                uint32_t kw = 0xffffffffu;   // which of its 32 query columns the thread's key row keeps
+                bool drop = false;           // some thread of the warp drops some
+                const int tile = tiles[kt & 3];
+                uint32_t from;               // tensor-memory address of the thread's columns of S^T
+                {
+                    const Place at;
+                    from = T_A + at.lane_addr + at.column();
+                    const float4 *sNL = reinterpret_cast<const float4 *>(smem + L::oLSE + s * 512 + at.column() * 4);
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const float4 nl = nlr[q];
-                    float p[4];
-                    p[0] = ex2_approx(fmaf(__uint_as_float(sv[q * 4 + 0]), sl2, nl.x));
-                    p[1] = ex2_approx(fmaf(__uint_as_float(sv[q * 4 + 1]), sl2, nl.y));
-                    p[2] = ex2_approx(fmaf(__uint_as_float(sv[q * 4 + 2]), sl2, nl.z));
-                    p[3] = ex2_approx(fmaf(__uint_as_float(sv[q * 4 + 3]), sl2, nl.w));
-                    if (masked) {
+                    for (int q = 0; q < 8; ++q) nlr[q] = sNL[q];
+                    // a mask finer than the tile: the keep bits of this thread's key row and its 32 query columns
+                    if constexpr (FINE) {
+                        const int jg = slots[t & 1].jt * TK + (int)at.row, ig0 = (tile & 0x3fffffff) * TQ + (int)at.column();
+                        kw = ig0 < n && jg < n ? fine_word(a.fine, a.mask_heads, slots[t & 1].bh, false, jg, ig0) : 0u;
+                    }
+                }
+                mbar_wait(&bars[V2_S], kt & 1, ab);
+                tcgen05_fence_after();
+                uint32_t ppack[16];   // P as bf16 pairs: what dV uses, and what dS is formed from
+                {
+                    uint32_t sv[32];
+                    tmem_ld32(from, sv);
+                    if (tile < 0) {
+                        const Place at;
+                        const int jg = slots[t & 1].jt * TK + (int)at.row, ig0 = (tile & 0x3fffffff) * TQ + (int)at.column(), left = n - ig0;
+                        if (left < 32) kw &= left > 0 ? 0xffffffffu >> (32 - left) : 0u;
+                        if (jg >= n) kw = 0u;
+                        if (causal && jg > ig0) kw &= jg - ig0 < 32 ? 0xffffffffu << (jg - ig0) : 0u;
+                    }
+                    if (FINE || tile < 0) drop = __any_sync(0xffffffffu, kw != 0xffffffffu);
+                    tmem_wait_ld();
+                    tcgen05_fence_before();
+                    warp_arrive(&bars[V2_SLD], lane);   // region A may take dP^T
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const float4 nl = nlr[q];
+                        float p0, p1;
+                        p_pair(sv[q * 4 + 0], sv[q * 4 + 1], a.sl2, nl.x, nl.y, p0, p1);
+                        ppack[q * 2 + 0] = pack_bf16(p0, p1);
+                        p_pair(sv[q * 4 + 2], sv[q * 4 + 3], a.sl2, nl.z, nl.w, p0, p1);
+                        ppack[q * 2 + 1] = pack_bf16(p0, p1);
+                    }
+                    if (drop) {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) ppack[e] &= (kw & (1u << (2 * e)) ? 0xffffu : 0u) | (kw & (2u << (2 * e)) ? 0xffff0000u : 0u);
+                    }
+                }
+                float4 dsr[8];   // -scale * D of the same columns, again ahead of the wait
+                const Place at;
+                {
+                    const float4 *sDs = reinterpret_cast<const float4 *>(smem + L::oD + s * 512 + at.column() * 4);
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) dsr[q] = sDs[q];
+                }
+                const uint32_t from2 = T_A2 + at.lane_addr + at.column();
+                // P^T goes into region B before dP^T is awaited: a tensor-memory store issued while products run takes
+                // several hundred cycles, which now pass during that wait.  Its first 32 columns per half held dQ^T of the
+                // previous tile; the reducers release them after their first load
+                mbar_wait(&bars[V2_DQREL], (kt - 1) & 1, ab);
+                tcgen05_fence_after();
+                tmem_st16(T_B + at.lane_addr + at.h * 64 + at.qq * 16, ppack);
+                mbar_wait(&bars[V2_DP], kt & 1, ab);
+                tcgen05_fence_after();
+                {
+                    uint32_t dv[32];
+                    tmem_ld32(from2, dv);
+                    tmem_wait_ld();
+                    tcgen05_fence_before();
+                    warp_arrive(&bars[V2_DPLD], lane);   // region A may take the next S^T
+                    tmem_wait_st();
+                    tcgen05_fence_before();
+                    warp_arrive(&bars[V2_P + at.h], lane);
+                    uint8_t *slab = smem + L::odS + (L::NdS == 2 ? (kt & 1) * 2 * SLAB : 0) + at.h * SLAB;
+                    // One buffer: dS^T(k) goes over dS^T(k-1), which the dK and dQ^T products of tile k-1 read.  Both have completed:
+                    // the reducers release their columns (awaited above) only after dQ^T(k-1), the later of the two in the other
+                    // thread's issue order, has landed.  Two buffers: dK(k-2) was issued before dQ^T(k-1)
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {    // 8 query columns = one 16-byte chunk
+                        float ds[8];
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
-                            const int ig = ig0 + q * 4 + e;
-                            const bool ok = ig < n && jg < n && (!diag || jg <= ig) && ((kw >> (q * 4 + e)) & 1u);
-                            p[e] = ok ? p[e] : 0.f;
+                            const uint32_t pk = ppack[g * 4 + e];   // bf16 -> fp32 is a 16-bit shift
+                            const float4 dsc = dsr[g * 2 + e / 2];
+                            ds_pair(pk, dv[g * 8 + 2 * e], dv[g * 8 + 2 * e + 1], a.scale, e & 1 ? dsc.z : dsc.x, e & 1 ? dsc.w : dsc.y, ds[2 * e], ds[2 * e + 1]);
                         }
-                    }
-                    ppack[q * 2 + 0] = pack_bf16(p[0], p[1]);
-                    ppack[q * 2 + 1] = pack_bf16(p[2], p[3]);
-                }
-            }
-            float4 dsr[8];   // scale * D of the same columns, again ahead of the wait
+                        if (drop) {   // stale tail entries of the row vectors may be anything: select, do not multiply
 #pragma unroll
-            for (int q = 0; q < 8; ++q) dsr[q] = sDs[q];
-            // P^T goes into region B before dP^T is awaited: a tensor-memory store issued while products run takes
-            // several hundred cycles, which now pass during that wait.  Its first 32 columns per half held dQ^T of the
-            // previous tile; the reducers release them after their first load
-            if (k > 0) {
-                mbar_wait(&bars[V2_DQREL], (k - 1) & 1, ab);
+                            for (int e = 0; e < 8; ++e) ds[e] = (ppack[g * 4 + e / 2] & (e & 1 ? 0xffff0000u : 0xffffu)) != 0u ? ds[e] : 0.f;
+                        }
+                        *reinterpret_cast<uint4 *>(slab + sw128_offset(at.row, at.qq * 32 + g * 8)) =
+                            make_uint4(pack_bf16(ds[0], ds[1]), pack_bf16(ds[2], ds[3]), pack_bf16(ds[4], ds[5]),
+                                       pack_bf16(ds[6], ds[7]));
+                    }
+                }
+                fence_proxy_async_smem();
+                warp_arrive(&bars[V2_DS], lane);
+            }
+            // -------------------------------------------------------- epilogue: dV_j, dK_j (32 columns per warpgroup)
+            const size_t bh = slots[t & 1].bh;
+            const Place at;
+            const int jg = slots[t & 1].jt * TK + (int)at.row;
+            warp_arrive(&bars[V2_WE + (t & 1)], lane);
+            if (count > 0) {
+                // dV and dK of the last tile have completed when its stage is released (dQ^T, queued after them, is the
+                // reducers' business and reads neither accumulator)
+                mbar_wait(&bars[V2_QEMPTY + stage_of(kt - 1)], phase_of(kt - 1), ab);
                 tcgen05_fence_after();
             }
-            tmem_st16(T_B + lane_addr + cP, ppack);
-            mbar_wait(&bars[V2_DP], k & 1, ab);
-            tcgen05_fence_after();
-            {
-                uint8_t *slab = smem + L::odS + h * SLAB;
-                uint32_t dv[32];
-                tmem_ld32(T_A2 + lane_addr + c0, dv);
-                tmem_wait_ld();
-                tcgen05_fence_before();
-                warp_arrive(&bars[V2_DPLD], lane);   // region A may take the next S^T
-                tmem_wait_st();
-                tcgen05_fence_before();
-                warp_arrive(&bars[V2_P + h], lane);
-                // dS^T(k) goes over dS^T(k-1), which the dK and dQ^T products of tile k-1 read from shared memory.  Both
-                // have completed: the reducers release their columns (awaited above) only after dQ^T(k-1), the later of
-                // the two in the other thread's issue order, has landed
-#pragma unroll
-                for (int g = 0; g < 4; ++g) {    // 8 query columns = one 16-byte chunk
-                    float ds[8], p[8];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const uint32_t pk = ppack[g * 4 + e];   // bf16 -> fp32 is a 16-bit shift
-                        p[2 * e] = __uint_as_float(pk << 16);
-                        p[2 * e + 1] = __uint_as_float(pk & 0xffff0000u);
-                    }
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        const float4 dsc = dsr[g * 2 + u];
-                        const uint32_t *d4 = &dv[g * 8 + u * 4];
-                        ds[u * 4 + 0] = p[u * 4 + 0] * fmaf(__uint_as_float(d4[0]), a.scale, -dsc.x);
-                        ds[u * 4 + 1] = p[u * 4 + 1] * fmaf(__uint_as_float(d4[1]), a.scale, -dsc.y);
-                        ds[u * 4 + 2] = p[u * 4 + 2] * fmaf(__uint_as_float(d4[2]), a.scale, -dsc.z);
-                        ds[u * 4 + 3] = p[u * 4 + 3] * fmaf(__uint_as_float(d4[3]), a.scale, -dsc.w);
-                    }
-                    if (masked) {   // stale tail entries of the row vectors may be anything: select, do not multiply
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) ds[e] = p[e] != 0.f ? ds[e] : 0.f;
-                    }
-                    *reinterpret_cast<uint4 *>(slab + sw128_offset(row, qq * 32 + g * 8)) =
-                        make_uint4(pack_bf16(ds[0], ds[1]), pack_bf16(ds[2], ds[3]), pack_bf16(ds[4], ds[5]),
-                                   pack_bf16(ds[6], ds[7]));
-                }
-            }
-            fence_proxy_async_smem();
-            warp_arrive(&bars[V2_DS], lane);
-            ++k;
-        }
-        // ------------------------------------------------------------ epilogue: dV_j, dK_j (32 columns per warpgroup)
-        if (k > 0) {
-            // dV and dK of the last tile have completed when its stage is released (dQ^T, queued after them, is the
-            // reducers' business and reads neither accumulator nor the stages reused below)
-            mbar_wait(&bars[V2_QEMPTY + ((k - 1) & 1)], ((k - 1) >> 1) & 1, ab);
-            tcgen05_fence_after();
-        }
-        {
-            // dV_j and dK_j go out through shared memory and TMA stores (coalesced; rows beyond n are clipped): the
-            // first Q and dO stages are free by now -- every product that read them has completed.  Each thread packs
-            // 32 columns of its key row into the swizzled slab layout the store expects.
-            const int cq = (warp / 4) * 32;        // d = 64: the upper two warpgroups have no columns
+            const uint32_t cq = at.column();       // d = 64: the upper two warpgroups have no columns
             if (cq < HD) {
+                const int jc = jg < n ? jg : 0;
+                const bool wide = (((uintptr_t)a.dK | (uintptr_t)a.dV) & 31) == 0;
 #pragma unroll
                 for (int which = 0; which < 2; ++which) {
-                    uint32_t v[32];
-                    if (k > 0) {
-                        tmem_ld32((which == 0 ? T_dV : T_dK) + lane_addr + cq, v);
+                    __nv_bfloat16 *po = (which == 0 ? a.dV : a.dK) + (bh * n + jc) * HD + cq;
+#pragma unroll
+                    for (int e0 = 0; e0 < 32; e0 += 16) {
+                        uint32_t v[16], y[8];
+                        tmem_ld16((which == 0 ? T_dV : T_dK) + at.lane_addr + cq + e0, v);
                         tmem_wait_ld();
-                    } else {
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) v[e] = 0u;
+                        for (int u = 0; u < 8; ++u)   // without a query tile nothing has been accumulated
+                            y[u] = count > 0 ? pack_bf16(__uint_as_float(v[2 * u]), __uint_as_float(v[2 * u + 1])) : 0u;
+                        if (jg < n) store32(po + e0, y, wide);
                     }
-                    uint8_t *slab = smem + (which == 0 ? L::oQ : L::odO) + (cq / 64) * SLAB;
-#pragma unroll
-                    for (int e = 0; e < 32; e += 8)
-                        *reinterpret_cast<uint4 *>(slab + sw128_offset(row, (cq % 64) + e)) =
-                            make_uint4(pack_bf16(__uint_as_float(v[e]), __uint_as_float(v[e + 1])),
-                                       pack_bf16(__uint_as_float(v[e + 2]), __uint_as_float(v[e + 3])),
-                                       pack_bf16(__uint_as_float(v[e + 4]), __uint_as_float(v[e + 5])),
-                                       pack_bf16(__uint_as_float(v[e + 6]), __uint_as_float(v[e + 7])));
                 }
-            }
-            fence_proxy_async_smem();
-            asm volatile("bar.sync 1, 512;" ::: "memory");   // the sixteen exp / dS warps
-            if (tid == 0) {
-#pragma unroll
-                for (uint32_t sl = 0; sl < L::kSlabs; ++sl) {
-                    tma_store_3d(&mdV, smem + L::oQ + sl * SLAB, sl * 64, j0, (int)bh);
-                    tma_store_3d(&mdK, smem + L::odO + sl * SLAB, sl * 64, j0, (int)bh);
-                }
-                tma_store_commit();
-                tma_store_wait_read();   // the slabs have been read; the writes complete with the grid
+                tcgen05_fence_before();
             }
         }
     }
@@ -976,12 +1064,12 @@ attn_status launch_bwd(const Problem &p)
         !make_tmap_bf16_3d(&mV, p.V, HD, p.n, BH, 128) || !make_tmap_bf16_3d(&mdO, p.dO, HD, p.n, BH, 128))
         return ATTN_ERR_LAUNCH;
     BwdArgs a{};
-    a.nLSE2 = p.nLSE2; a.Ds = p.D; a.dQ_acc = p.dQ_acc;
+    a.nLSE2 = p.nLSE2; a.nDs = p.D; a.dQ_acc = p.dQ_acc;
     a.dK = (__nv_bfloat16 *)p.dK; a.dV = (__nv_bfloat16 *)p.dV;
     a.n = p.n; a.BH = (int)p.BH; a.ns = p.stat_stride;
     a.mask_kind = p.mask_kind; a.block = p.block; a.nb = p.nb; a.mask_heads = p.mask_heads; a.fine = p.fine;
     a.col_ptr = p.col_ptr; a.row_idx = p.row_idx;
-    a.scale = p.scale;
+    a.scale = p.scale; a.sl2 = p.scale * 1.4426950408889634f;
     a.status = p.status;
     a.group = bwd_head_group(p);
     if (bwd_preprocess_launch(p, WITH_DQ) != ATTN_OK) return ATTN_ERR_LAUNCH;
@@ -993,9 +1081,7 @@ attn_status launch_bwd(const Problem &p)
         auto kernel = p.fine.mode ? tc_bwd_fused_kernel<HD, true> : tc_bwd_fused_kernel<HD, false>;
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
             return ATTN_ERR_LAUNCH;
-        CUtensorMap mdK, mdV;
-        if (!make_tmap_bf16_3d(&mdK, p.dK, HD, p.n, BH, 128) || !make_tmap_bf16_3d(&mdV, p.dV, HD, p.n, BH, 128)) return ATTN_ERR_LAUNCH;
-        ok = launch_chained(kernel, grid, kThreadsFused, bytes, p.stream, mQ, mK, mV, mdO, mdK, mdV, a);
+        ok = launch_chained(kernel, grid, kThreadsFused, bytes, p.stream, mQ, mK, mV, mdO, a);
     } else {
         auto kernel = p.split ? tc_bwd_dkdv_kernel<HD, true> : tc_bwd_dkdv_kernel<HD, false>;
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DkdvSmem<HD>::kBytes) != cudaSuccess)

@@ -145,7 +145,7 @@ tc_bwd_fused64_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_const
                 for (uint32_t sl = 0; sl < L::kSlabs; ++sl)
                     tma_load_3d(smem + L::odO + s * L::kQTile + sl * SLAB64, &mdO, bar, sl * 64, i0, (int)bh);
                 bulk_load_1d(smem + L::oLSE + s * 256, a.nLSE2 + bh * n + i0, rows * 4, bar);
-                bulk_load_1d(smem + L::oD + s * 256, a.Ds + bh * n + i0, rows * 4, bar);
+                bulk_load_1d(smem + L::oD + s * 256, a.nDs + bh * n + i0, rows * 4, bar);
                 ++t;
             }
             // nobody else waits for K_j / V_j when there is no tile: do not exit with their loads in flight
@@ -357,10 +357,10 @@ tc_bwd_fused64_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_const
                     for (int u = 0; u < 2; ++u) {
                         const float4 dsc = dsr[gg * 2 + u];
                         const uint32_t *d4 = &dv[gg * 8 + u * 4];
-                        ds[u * 4 + 0] = p[u * 4 + 0] * fmaf(__uint_as_float(d4[0]), a.scale, -dsc.x);
-                        ds[u * 4 + 1] = p[u * 4 + 1] * fmaf(__uint_as_float(d4[1]), a.scale, -dsc.y);
-                        ds[u * 4 + 2] = p[u * 4 + 2] * fmaf(__uint_as_float(d4[2]), a.scale, -dsc.z);
-                        ds[u * 4 + 3] = p[u * 4 + 3] * fmaf(__uint_as_float(d4[3]), a.scale, -dsc.w);
+                        ds[u * 4 + 0] = p[u * 4 + 0] * fmaf(__uint_as_float(d4[0]), a.scale, dsc.x);
+                        ds[u * 4 + 1] = p[u * 4 + 1] * fmaf(__uint_as_float(d4[1]), a.scale, dsc.y);
+                        ds[u * 4 + 2] = p[u * 4 + 2] * fmaf(__uint_as_float(d4[2]), a.scale, dsc.z);
+                        ds[u * 4 + 3] = p[u * 4 + 3] * fmaf(__uint_as_float(d4[3]), a.scale, dsc.w);
                     }
                     if (masked) {   // stale tail entries of the row vectors may be anything: select, do not multiply
 #pragma unroll
@@ -425,7 +425,7 @@ attn_status launch_bwd64(const Problem &p)
         !make_tmap_bf16_3d(&mV, p.V, HD, p.n, BH, 128) || !make_tmap_bf16_3d(&mdO, p.dO, HD, p.n, BH, 64))
         return ATTN_ERR_LAUNCH;
     BwdArgs a{};
-    a.nLSE2 = p.nLSE2; a.Ds = p.D; a.dQ_acc = p.dQ_acc;
+    a.nLSE2 = p.nLSE2; a.nDs = p.D; a.dQ_acc = p.dQ_acc;
     a.dK = (__nv_bfloat16 *)p.dK; a.dV = (__nv_bfloat16 *)p.dV;
     a.n = p.n; a.BH = (int)p.BH; a.ns = p.stat_stride;
     a.mask_kind = p.mask_kind; a.block = p.block; a.nb = p.nb; a.mask_heads = p.mask_heads; a.fine = p.fine;

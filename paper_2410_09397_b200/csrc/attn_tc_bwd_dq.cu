@@ -30,9 +30,9 @@ constexpr uint32_t SLAB = 128 * 128;
 
 struct DqArgs {
     __nv_bfloat16 *dQ;
-    const float *nLSE2, *Ds;
+    const float *nLSE2, *nDs;
     int n, BH;
-    int ns;                    // rows of nLSE2 and Ds per head (n, or n rounded up to a multiple of 4)
+    int ns;                    // rows of nLSE2 and nDs per head (n, or n rounded up to a multiple of 4)
     int mask_kind, block, nb, mask_heads;
     const int *row_ptr, *col_idx;
     FineMask fine;
@@ -245,7 +245,7 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
         const int ig = i0 + row;
         const float sl2 = a.scale * 1.4426950408889634f;
         const float nl = ig < n ? a.nLSE2[(size_t)bh * a.ns + ig] : -INFINITY;   // -inf: every probability of the row is 0
-        const float dsi = ig < n ? a.Ds[(size_t)bh * a.ns + ig] : 0.f;
+        const float dsi = ig < n ? a.nDs[(size_t)bh * a.ns + ig] : 0.f;
         int k = 0;
         for (int idx = 0; idx < iter.raw; ++idx) {
             const int jt = iter.tile(idx);
@@ -286,8 +286,8 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
                 if (lane == 0) mbar_arrive(&bars[DB_DPFREE]);
 #pragma unroll
                 for (int e = 0; e < 32; e += 2) {
-                    const float d0 = p[e] * fmaf(__uint_as_float(dv0[e]), a.scale, -dsi);
-                    const float d1 = p[e + 1] * fmaf(__uint_as_float(dv0[e + 1]), a.scale, -dsi);
+                    const float d0 = p[e] * fmaf(__uint_as_float(dv0[e]), a.scale, dsi);
+                    const float d1 = p[e + 1] * fmaf(__uint_as_float(dv0[e + 1]), a.scale, dsi);
                     dpack[e / 2] = pack_bf16(d0, d1);
                     if constexpr (SPLIT) drest[e / 2] = pack_bf16_rest(d0, d1, dpack[e / 2]);
                 }
@@ -347,7 +347,7 @@ attn_status launch_dq(const Problem &p)
         return ATTN_ERR_LAUNCH;
     DqArgs a{};
     a.dQ = (__nv_bfloat16 *)p.dQ;
-    a.nLSE2 = p.nLSE2; a.Ds = p.D;
+    a.nLSE2 = p.nLSE2; a.nDs = p.D;
     a.n = p.n; a.BH = (int)p.BH; a.ns = p.stat_stride;
     a.mask_kind = p.mask_kind; a.block = p.block; a.nb = p.nb; a.mask_heads = p.mask_heads; a.fine = p.fine;
     a.row_ptr = p.row_ptr; a.col_idx = p.col_idx;
@@ -365,7 +365,7 @@ attn_status launch_dq(const Problem &p)
 
 }  // namespace
 
-// Requires p.D = scale * rowsum(dO o O) and p.nLSE2 = -LSE log2(e), as the key-stationary launch leaves them.
+// Requires p.D = -scale * rowsum(dO o O) and p.nLSE2 = -LSE log2(e), as the key-stationary launch leaves them.
 attn_status tc_bwd_dq(const Problem &p)
 {
     if (p.d == 64) return launch_dq<64>(p);

@@ -13,14 +13,14 @@ using namespace tc;
 constexpr int TK = 128;                 // keys per CTA
 constexpr uint32_t SLAB = 128 * 128;   // bytes of one [128 rows][64 bf16] slab
 struct BwdArgs {
-    const float *nLSE2, *Ds;   // -LSE log2(e) and scale * D per row (workspace)
+    const float *nLSE2, *nDs;  // -LSE log2(e) and -scale * D per row (workspace)
     float *dQ_acc;
     __nv_bfloat16 *dK, *dV;
     int n, BH;
-    int ns;                    // rows of nLSE2 and Ds per head (n, or n rounded up to a multiple of 4)
+    int ns;                    // rows of nLSE2 and nDs per head (n, or n rounded up to a multiple of 4)
     int mask_kind, block, nb, mask_heads;
     const int *col_ptr, *row_idx;   // block-CSC of the mask
-    float scale;
+    float scale, sl2;          // sl2 = scale * log2(e)
     int group;                 // heads per launch group (divides BH)
     FineMask fine;             // a mask finer than the tiles: dropped entries are masked inside the visited tiles
     uint32_t *status;
@@ -80,7 +80,7 @@ __device__ __forceinline__ float ex2_approx(float x)
     return y;
 }
 
-// D pre-pass of the fused backward: Ds_i = scale * sum_c dO_ic O_ic and
+// D pre-pass of the tensor-core backward: nDs_i = -scale * sum_c dO_ic O_ic (the form that packed multiply-adds take) and
 // nlse2_i = -LSE_i * log2(e) (minus infinity for a row with no kept entry, so that its
 // probabilities come out as exactly zero).  16-byte loads, HD/8 lanes share a row.  The same
 // pass clears the fp32 dQ accumulator of the fused backward (`acc`, `acc16` 16-byte words; null =
@@ -90,7 +90,7 @@ __device__ __forceinline__ float ex2_approx(float x)
 template <int HD, bool PAD>
 __global__ void __launch_bounds__(256) tc_preprocess_kernel(const __nv_bfloat16 *__restrict__ O,
                                                             const __nv_bfloat16 *__restrict__ dO,
-                                                            const float *__restrict__ LSE, float *__restrict__ Ds,
+                                                            const float *__restrict__ LSE, float *__restrict__ nDs,
                                                             float *__restrict__ nlse2, size_t rows, int n, int ns, float scale,
                                                             uint4 *__restrict__ acc, size_t acc16, const ClearList clear, uint32_t *status)
 {
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(256) tc_preprocess_kernel(const __nv_bfloat16 
             for (int o = LPR / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
             if (row < rows && lr == 0) {
                 const size_t to = PAD ? row + (size_t)((uint32_t)row / (uint32_t)n) * (ns - n) : row;   // rows < 2^32: d >= 64
-                Ds[to] = acc * scale;
+                nDs[to] = -(acc * scale);
                 const float l = LSE[row];
                 nlse2[to] = l == -INFINITY ? -INFINITY : -l * 1.4426950408889634f;
             }
