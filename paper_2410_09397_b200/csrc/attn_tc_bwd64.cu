@@ -22,8 +22,8 @@
 // dQ^T) | V_j 128 (d = 256 only).
 //
 // Roles: warps 0-7 exp / dS (lane quarter = warp % 4, 32 query columns each), warps 8-11 reducers
-// (dQ^T tile -> registers -> fp32 accumulator), warp 12 lane 0 issues every product in a fixed
-// order, warp 13 lane 0 every TMA load.  All waits are bounded (tc_common.cuh).
+// (dQ^T tile -> registers -> fp32 accumulator), warp 12 lane 0 issues S^T and dP^T, warp 14 lane 0 dV, dQ^T and dK, warp 13
+// lane 0 every TMA load.  All waits are bounded (tc_common.cuh).
 #include "tc_bwd_common.cuh"
 
 namespace attn {
@@ -35,7 +35,7 @@ using namespace bwdk;
 constexpr int TQ64 = 64;
 constexpr uint32_t SLAB = 128 * 128;     // [128 rows][64 bf16]
 constexpr uint32_t SLAB64 = 64 * 128;    // [64 rows][64 bf16]
-constexpr int kThreads64 = 8 * 32 + 4 * 32 + 2 * 32;
+constexpr int kThreads64 = 8 * 32 + 4 * 32 + 3 * 32;
 
 template <int HD>
 struct B64 {
@@ -61,7 +61,7 @@ struct B64 {
     static constexpr uint32_t kBytes = kUsed < 117 * 1024 ? 117 * 1024 : kUsed;   // one CTA per SM
 };
 
-enum { B_KV = 0, B_VDONE = 1, B_S = 2, B_DP = 3, B_P = 4, B_DS = 5, B_DQ = 6, B_DQDONE = 7, B_DONE = 8,
+enum { B_KV = 0, B_VDONE = 1, B_S = 2, B_DP = 3, B_P = 4, B_DS = 5, B_DQ = 6, B_DQDONE = 7, B_DV = 8,
        B_QFULL = 9, B_QEMPTY = 13 };
 
 template <int HD>
@@ -100,7 +100,7 @@ tc_bwd_fused64_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_const
         mbar_init(&bars[B_DS], kExpWarps);
         mbar_init(&bars[B_DQ], 1);
         mbar_init(&bars[B_DQDONE], kReduceWarps);
-        mbar_init(&bars[B_DONE], 1);
+        mbar_init(&bars[B_DV], 1);
         for (int s = 0; s < NS; ++s) { mbar_init(&bars[B_QFULL + s], 1); mbar_init(&bars[B_QEMPTY + s], 1); }
         fence_barrier_init();
         prefetch_tensormap(&mQ); prefetch_tensormap(&mK_); prefetch_tensormap(&mV); prefetch_tensormap(&mdO);
@@ -152,25 +152,28 @@ tc_bwd_fused64_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_const
             if (T == 0) mbar_wait(&bars[B_KV], 0, ab);
         }
     } else if (warp == 12) {
-        // ------------------------------------------------------------ MMA issuer: every product, in a fixed order
+        // ------------------------------------------------------------ MMA issuer A: S^T and dP^T
         if (lane == 0 && T > 0) {
-            constexpr uint32_t idesc_s = idesc_bf16(128, 64, 0, 0);        // S^T, dP^T: N = 64 queries
-            constexpr uint32_t idesc_acc = idesc_bf16(128, HA, 0, 1);      // dV, dK: B MN-major
-            constexpr uint32_t idesc_dq = idesc_bf16(128, 64, 1, 1);       // dQ^T: both MN-major
+            constexpr uint32_t idesc_s = idesc_bf16(128, 64, 0, 0);        // N = 64 queries
             constexpr uint32_t kSlab = SLAB >> 4, kSlab64 = SLAB64 >> 4;
             const uint32_t kK = desc_lo_kmajor(smem_u32(smem + L::oK));
             const uint32_t kV = desc_lo_kmajor(smem_u32(smem + L::oV));   // unused when V_j is in tensor memory
-            // K_j[:, c]^T: M = 128 head-dimension indices (two 64-wide slabs of the K tile), contraction over the keys
-            const uint32_t mK = desc_lo_mnmajor(smem_u32(smem + L::oK + (HA == 128 ? c * 2 : 0) * SLAB), SLAB);
-            const uint32_t kdS = desc_lo_kmajor(smem_u32(smem + L::odS)), mdS = desc_lo_mnmajor(smem_u32(smem + L::odS), SLAB);
-            auto issue_S = [&](int s) {
+            mbar_wait(&bars[B_KV], 0, ab);
+            if (L::kVinTmem) mbar_wait(&bars[B_VDONE], 0, ab);
+            for (int t = 0; t < T; ++t) {
+                const int s = t % NS;
+                // S^T over P^T of the tile before, which dV has consumed (tile -1: returns at once)
+                mbar_wait(&bars[B_QFULL + s], (t / NS) & 1, ab);
+                mbar_wait(&bars[B_DV], (t - 1) & 1, ab);
+                tcgen05_fence_after();
                 const uint32_t kQ = desc_lo_kmajor(smem_u32(smem + L::oQ + s * L::kQTile));
 #pragma unroll
                 for (int kk = 0; kk < HD / 16; ++kk)
                     mma_ss_lo(T_RS, kK + (kk / 4) * kSlab + (kk % 4) * 2, kQ + (kk / 4) * kSlab64 + (kk % 4) * 2, idesc_s, kk > 0);
                 mma_commit(&bars[B_S]);
-            };
-            auto issue_dP = [&](int s) {
+                // dP^T into RD once the reducers hold dQ^T of the tile before in registers
+                mbar_wait(&bars[B_DQDONE], (t - 1) & 1, ab);
+                tcgen05_fence_after();
                 const uint32_t kdO = desc_lo_kmajor(smem_u32(smem + L::odO + s * L::kQTile));
 #pragma unroll
                 for (int kk = 0; kk < HD / 16; ++kk) {
@@ -179,13 +182,16 @@ tc_bwd_fused64_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_const
                     else mma_ss_lo(T_RD, kV + (kk / 4) * kSlab + (kk % 4) * 2, kdO + boff, idesc_s, kk > 0);
                 }
                 mma_commit(&bars[B_DP]);
-            };
-            mbar_wait(&bars[B_KV], 0, ab);
-            if (L::kVinTmem) mbar_wait(&bars[B_VDONE], 0, ab);
-            mbar_wait(&bars[B_QFULL], 0, ab);
-            tcgen05_fence_after();
-            issue_S(0);
-            issue_dP(0);
+            }
+        }
+    } else if (warp == 14) {
+        // ------------------------------------------------------------ MMA issuer B: dV, dQ^T, dK
+        if (lane == 0 && T > 0) {
+            constexpr uint32_t idesc_acc = idesc_bf16(128, HA, 0, 1);      // dV, dK: B MN-major
+            constexpr uint32_t idesc_dq = idesc_bf16(128, 64, 1, 1);       // dQ^T: both MN-major
+            // K_j[:, c]^T: M = 128 head-dimension indices (two 64-wide slabs of the K tile), contraction over the keys
+            const uint32_t mK = desc_lo_mnmajor(smem_u32(smem + L::oK + (HA == 128 ? c * 2 : 0) * SLAB), SLAB);
+            const uint32_t kdS = desc_lo_kmajor(smem_u32(smem + L::odS)), mdS = desc_lo_mnmajor(smem_u32(smem + L::odS), SLAB);
             for (int t = 0; t < T; ++t) {
                 const int s = t % NS;
                 const uint32_t qbase = smem_u32(smem + L::oQ + s * L::kQTile + (HA == 128 ? c * 2 : 0) * SLAB64);
@@ -197,31 +203,20 @@ tc_bwd_fused64_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_const
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)
                     mma_ts_lo(T_dV, T_RS + (kk / 2) * 32 + (kk % 2) * 8, mdO_ + kk * 128, idesc_acc, (t > 0) || (kk > 0));
-                // S^T of the next tile over P^T: the products execute in issue order, dV has consumed it by then
-                if (t + 1 < T) {
-                    mbar_wait(&bars[B_QFULL + (t + 1) % NS], ((t + 1) / NS) & 1, ab);
-                    tcgen05_fence_after();
-                    issue_S((t + 1) % NS);
-                }
-                // dK[:, c] += dS^T Q[:, c], then dQ^T[c] = K_j[:, c]^T dS^T into RD (dP^T has been copied out of it)
+                mma_commit(&bars[B_DV]);
+                // dQ^T[c] = K_j[:, c]^T dS^T into RD (dP^T has been copied out of it) first: the next dP^T waits for the reducers
+                // to have read it.  Then dK[:, c] += dS^T Q[:, c], whose completion also says that dS^T has been read
                 mbar_wait(&bars[B_DS], t & 1, ab);
                 tcgen05_fence_after();
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    mma_ss_lo(T_dK, kdS + kk * 2, mQ_ + kk * 128, idesc_acc, (t > 0) || (kk > 0));
-                mma_commit(&bars[B_QEMPTY + s]);     // stage s: dO was last read by dV, Q by dK
 #pragma unroll
                 for (int kk = 0; kk < TK / 16; ++kk)
                     mma_ss_lo(T_RD, mK + kk * 128, mdS + kk * 128, idesc_dq, kk > 0);
                 mma_commit(&bars[B_DQ]);
-                // dP^T of the next tile into RD once the reducers hold dQ^T in registers
-                if (t + 1 < T) {
-                    mbar_wait(&bars[B_DQDONE], t & 1, ab);
-                    tcgen05_fence_after();
-                    issue_dP((t + 1) % NS);
-                }
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)
+                    mma_ss_lo(T_dK, kdS + kk * 2, mQ_ + kk * 128, idesc_acc, (t > 0) || (kk > 0));
+                mma_commit(&bars[B_QEMPTY + s]);     // stage s: dO was last read by dV, Q by dK
             }
-            mma_commit(&bars[B_DONE]);
         }
     } else if (warp >= 8) {
         // ------------------------------------------------------------ reducers: dQ^T[c] tile -> fp32 accumulator
@@ -332,16 +327,16 @@ tc_bwd_fused64_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_const
             for (int q = 0; q < 8; ++q) dsr[q] = sDs[q];
             // P^T over this thread's own S^T columns (it holds them in registers; no other thread reads them)
             tmem_st16(T_RS + lane_addr + c0, ppack);
+            tmem_wait_st();
+            tcgen05_fence_before();
+            warp_arrive(&bars[B_P], lane);
             mbar_wait(&bars[B_DP], t & 1, ab);
             tcgen05_fence_after();
             uint32_t dv[32];
             tmem_ld32(T_RD + lane_addr + c0, dv);
             tmem_wait_ld();
-            tmem_wait_st();
-            tcgen05_fence_before();
-            warp_arrive(&bars[B_P], lane);
-            // dS^T(t) goes over dS^T(t-1): the dK and dQ^T products of tile t-1 must be done with it
-            if (t > 0) mbar_wait(&bars[B_DQ], (t - 1) & 1, ab);
+            // dS^T(t) goes over dS^T(t-1): the dQ^T and dK products of tile t-1 must be done with it
+            if (t > 0) mbar_wait(&bars[B_QEMPTY + (t - 1) % NS], ((t - 1) / NS) & 1, ab);
             {
                 uint8_t *slab = smem + L::odS;
 #pragma unroll
@@ -378,7 +373,7 @@ tc_bwd_fused64_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_const
         }
         // ------------------------------------------------------------ epilogue: dV_j[:, c], dK_j[:, c]
         if (T > 0) {
-            mbar_wait(&bars[B_DONE], 0, ab);
+            mbar_wait(&bars[B_QEMPTY + (T - 1) % NS], ((T - 1) / NS) & 1, ab);
             tcgen05_fence_after();
         }
         if (g * 64 < HA) {

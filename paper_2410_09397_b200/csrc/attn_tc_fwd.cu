@@ -32,7 +32,7 @@ using namespace tc;
 
 constexpr int TQ = 128;
 constexpr int kSoftmaxThreads = 256;
-constexpr int kThreads = kSoftmaxThreads + 64;
+constexpr int kThreads = kSoftmaxThreads + 96;   // d = 256: two issuing warps and the loading warp
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kRescaleThreshold = 8.f;   // log2 units
@@ -138,6 +138,25 @@ __device__ __forceinline__ float row_lse(float m, float l)
     return fmaf(s, kLn2, fmaf(lost, kLn2, fmaf(s, kLn2Rest, logf(f) + 4.5e-8f)));
 }
 
+// x = exp2(v * s + n) of two scores; both are added to `sum`
+__device__ __forceinline__ void exp_pair(uint32_t v0, uint32_t v1, uint64_t s2, uint64_t n2, uint64_t &sum, float &x0, float &x1)
+{
+    uint64_t x;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(v0), "r"(v1));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(x) : "l"(x), "l"(s2), "l"(n2));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(x1) : "l"(x));
+    x0 = ex2_fast_f(x0);
+    x1 = ex2_fast_f(x1);
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(x0), "f"(x1));
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(sum) : "l"(sum), "l"(x));
+}
+__device__ __forceinline__ float sum_of(const uint64_t (&sum)[4])
+{
+    float a[8];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) asm("mov.b64 {%0, %1}, %2;" : "=f"(a[2 * e]), "=f"(a[2 * e + 1]) : "l"(sum[e]));
+    return ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+}
 template <int HD>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_fwd_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CUtensorMap mK,
@@ -169,7 +188,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CU
         *abort_flag = 0;
         mbar_init(&bars[FB_Q], 1);
         for (int s = 0; s < NST; ++s) { mbar_init(&bars[FB_KVFULL + s], 1); mbar_init(&bars[FB_KVEMPTY + s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&bars[FB_S + b], 1); mbar_init(&bars[FB_P + b], kSoftmaxThreads); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&bars[FB_S + b], 1); mbar_init(&bars[FB_P + b], kSoftmaxThreads / 32); }
         mbar_init(&bars[FB_O], 1);
         mbar_init(&bars[FB_OLAST], 1);
         fence_barrier_init();
@@ -214,14 +233,16 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CU
             }
         }
     } else if (warp == 8) {
-        // ------------------------------------------------------------ MMA issuer
+        // ------------------------------------------------------------ MMA issuer A: S = Q K^T, up to two tiles ahead
         if (lane == 0 && niter == 0) mbar_wait(&bars[FB_Q], 0, ab);   // let the Q load land before exit
         if (lane == 0 && niter > 0) {
             constexpr uint32_t idesc_s = idesc_bf16(128, TKF, 0, 0);
-            constexpr uint32_t idesc_o = idesc_bf16(128, HD, 0, 1);
             const uint32_t kQ = desc_lo_kmajor(smem_u32(smem + C::oQ));
-            auto issue_S = [&](int k) {
+            mbar_wait(&bars[FB_Q], 0, ab);
+            for (int k = 0; k < niter; ++k) {
                 const int s = k % NST;
+                // K of tile k goes where that of tile k - 2 was, so its load tells that O += P V of that tile, which read P from
+                // this S buffer, has completed
                 mbar_wait(&bars[FB_KVFULL + s], (k / NST) & 1, ab);
                 tcgen05_fence_after();
                 const uint32_t kK = desc_lo_kmajor(smem_u32(smem + C::oK + s * C::kKTile));
@@ -230,11 +251,13 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CU
                     mma_ss_lo(tm + (k & 1) * 128, kQ + (kk / 4) * (C::kQSlab >> 4) + (kk % 4) * 2,
                               kK + (kk / 4) * (C::kKSlab >> 4) + (kk % 4) * 2, idesc_s, kk > 0);
                 mma_commit(&bars[FB_S + (k & 1)]);
-            };
-            mbar_wait(&bars[FB_Q], 0, ab);
-            issue_S(0);
+            }
+        }
+    } else if (warp == 10) {
+        // ------------------------------------------------------------ MMA issuer B: O += P V
+        if (lane == 0) {
+            constexpr uint32_t idesc_o = idesc_bf16(128, HD, 0, 1);
             for (int k = 0; k < niter; ++k) {
-                if (k + 1 < niter) issue_S(k + 1);
                 const int s = k % NST, b = k & 1;
                 mbar_wait(&bars[FB_P + b], (k >> 1) & 1, ab);
                 tcgen05_fence_after();
@@ -316,18 +339,20 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CU
             }
             const float noff = m_ref == -INFINITY ? 0.f : -m_ref;
             uint32_t pp[CW / 2];
-            float rs = 0.f;
+            uint64_t s2, n2, sum[4] = {0ull, 0ull, 0ull, 0ull};
+            asm("mov.b64 %0, {%1, %1};" : "=l"(s2) : "f"(sl2));
+            asm("mov.b64 %0, {%1, %1};" : "=l"(n2) : "f"(noff));
 #pragma unroll
             for (int e = 0; e < CW; e += 2) {
-                const float p0 = ex2_fast_f(fmaf(sv[e], sl2, noff)), p1 = ex2_fast_f(fmaf(sv[e + 1], sl2, noff));
-                rs += p0 + p1;
+                float p0, p1;
+                exp_pair(__float_as_uint(sv[e]), __float_as_uint(sv[e + 1]), s2, n2, sum[(e / 2) & 3], p0, p1);
                 pp[e / 2] = pack_bf16(p0, p1);
             }
-            l_part += rs;
+            l_part += sum_of(sum);
             tmem_st16(T_S + lane_addr + wg * (CW / 2), pp);
             tmem_wait_st();
             tcgen05_fence_before();
-            mbar_arrive(&bars[FB_P + b]);
+            warp_arrive_f(&bars[FB_P + b], lane);
             ++k;
         }
         // ------------------------------------------------------------ epilogue
@@ -367,7 +392,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CU
                 }
             }
         }
-        if (wg == 0 && ig < n) a.LSE[(size_t)bh * n + ig] = l_tot > 0.f ? m_ref * kLn2 + logf(l_tot) : -INFINITY;
+        if (wg == 0 && ig < n) a.LSE[(size_t)bh * n + ig] = row_lse(m_ref, l_tot);
     }
     tcgen05_fence_before();
     __syncthreads();
@@ -394,25 +419,6 @@ __device__ __forceinline__ float row_max(const uint32_t (&v)[128])
 #pragma unroll
         for (int e = 0; e < 8; ++e) m[e] = max3(m[e], __uint_as_float(v[c + e]), __uint_as_float(v[c + e + 8]));
     return fmaxf(max3(max3(m[0], m[1], m[2]), m[3], m[4]), max3(m[5], m[6], m[7]));
-}
-// x = exp2(v * s + n) of two scores; both are added to `sum`
-__device__ __forceinline__ void exp_pair(uint32_t v0, uint32_t v1, uint64_t s2, uint64_t n2, uint64_t &sum, float &x0, float &x1)
-{
-    uint64_t x;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(v0), "r"(v1));
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(x) : "l"(x), "l"(s2), "l"(n2));
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(x1) : "l"(x));
-    x0 = ex2_fast_f(x0);
-    x1 = ex2_fast_f(x1);
-    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(x0), "f"(x1));
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(sum) : "l"(sum), "l"(x));
-}
-__device__ __forceinline__ float sum_of(const uint64_t (&sum)[4])
-{
-    float a[8];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) asm("mov.b64 {%0, %1}, %2;" : "=f"(a[2 * e]), "=f"(a[2 * e + 1]) : "l"(sum[e]));
-    return ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
 }
 // P = exp2(v * sl2 + noff) as two bf16 terms: pairs of leading terms over the first 64 columns of S (every thread overwrites
 // only its own lane, whose scores it already holds), what they lose over the other 64; returns the sum of the row of P before
