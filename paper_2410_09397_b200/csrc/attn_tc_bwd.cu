@@ -332,10 +332,8 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {
                         const float4 nl = sNL[q];
-                        p[q * 4 + 0] = ex2_approx(fmaf(__uint_as_float(sv[q * 4 + 0]), sl2, nl.x));
-                        p[q * 4 + 1] = ex2_approx(fmaf(__uint_as_float(sv[q * 4 + 1]), sl2, nl.y));
-                        p[q * 4 + 2] = ex2_approx(fmaf(__uint_as_float(sv[q * 4 + 2]), sl2, nl.z));
-                        p[q * 4 + 3] = ex2_approx(fmaf(__uint_as_float(sv[q * 4 + 3]), sl2, nl.w));
+                        p_pair(sv[q * 4 + 0], sv[q * 4 + 1], sl2, nl.x, nl.y, p[q * 4 + 0], p[q * 4 + 1]);
+                        p_pair(sv[q * 4 + 2], sv[q * 4 + 3], sl2, nl.z, nl.w, p[q * 4 + 2], p[q * 4 + 3]);
                     }
                     if (masked) {
 #pragma unroll
@@ -381,10 +379,9 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                     for (int q = 0; q < 4; ++q) {
                         const float4 dsc = sDs[part * 4 + q];
                         const float *p4 = &p[part * 16 + q * 4];
-                        float d0 = p4[0] * fmaf(__uint_as_float(dv[q * 4 + 0]), a.scale, dsc.x);
-                        float d1 = p4[1] * fmaf(__uint_as_float(dv[q * 4 + 1]), a.scale, dsc.y);
-                        float d2 = p4[2] * fmaf(__uint_as_float(dv[q * 4 + 2]), a.scale, dsc.z);
-                        float d3 = p4[3] * fmaf(__uint_as_float(dv[q * 4 + 3]), a.scale, dsc.w);
+                        float d0, d1, d2, d3;
+                        mul_pair(fma_pair(dv[q * 4 + 0], dv[q * 4 + 1], a.scale, dsc.x, dsc.y), __float_as_uint(p4[0]), __float_as_uint(p4[1]), d0, d1);
+                        mul_pair(fma_pair(dv[q * 4 + 2], dv[q * 4 + 3], a.scale, dsc.z, dsc.w), __float_as_uint(p4[2]), __float_as_uint(p4[3]), d2, d3);
                         if (masked) {   // stale tail entries of the row vectors may be anything: select, do not multiply
                             d0 = p4[0] != 0.f ? d0 : 0.f; d1 = p4[1] != 0.f ? d1 : 0.f;
                             d2 = p4[2] != 0.f ? d2 : 0.f; d3 = p4[3] != 0.f ? d3 : 0.f;
@@ -417,10 +414,8 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                     for (int q = 0; q < 8; ++q) {
                         const float4 nl = sNL[q];
                         float p[4];
-                        p[0] = ex2_approx(fmaf(__uint_as_float(sv[q * 4 + 0]), sl2, nl.x));
-                        p[1] = ex2_approx(fmaf(__uint_as_float(sv[q * 4 + 1]), sl2, nl.y));
-                        p[2] = ex2_approx(fmaf(__uint_as_float(sv[q * 4 + 2]), sl2, nl.z));
-                        p[3] = ex2_approx(fmaf(__uint_as_float(sv[q * 4 + 3]), sl2, nl.w));
+                        p_pair(sv[q * 4 + 0], sv[q * 4 + 1], sl2, nl.x, nl.y, p[0], p[1]);
+                        p_pair(sv[q * 4 + 2], sv[q * 4 + 3], sl2, nl.z, nl.w, p[2], p[3]);
                         if (masked) {
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
@@ -454,16 +449,14 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {
                         const float4 dsc = sDs[q];
-                        // bf16 -> fp32 is a 16-bit shift; a masked entry has p = 0 and a finite dP, so its dS is an exact zero
-                        const float p0 = __uint_as_float(ppack[q * 2] << 16), p1 = __uint_as_float(ppack[q * 2] & 0xffff0000u);
-                        const float p2 = __uint_as_float(ppack[q * 2 + 1] << 16), p3 = __uint_as_float(ppack[q * 2 + 1] & 0xffff0000u);
-                        float d0 = p0 * fmaf(__uint_as_float(dv[q * 4 + 0]), a.scale, dsc.x);
-                        float d1 = p1 * fmaf(__uint_as_float(dv[q * 4 + 1]), a.scale, dsc.y);
-                        float d2 = p2 * fmaf(__uint_as_float(dv[q * 4 + 2]), a.scale, dsc.z);
-                        float d3 = p3 * fmaf(__uint_as_float(dv[q * 4 + 3]), a.scale, dsc.w);
+                        // a masked entry has p = 0 and a finite dP, so its dS is an exact zero
+                        const uint32_t pa = ppack[q * 2], pb = ppack[q * 2 + 1];
+                        float d0, d1, d2, d3;
+                        ds_pair(pa, dv[q * 4 + 0], dv[q * 4 + 1], a.scale, dsc.x, dsc.y, d0, d1);
+                        ds_pair(pb, dv[q * 4 + 2], dv[q * 4 + 3], a.scale, dsc.z, dsc.w, d2, d3);
                         if (masked) {   // stale tail entries of the row vectors may be anything: select, do not multiply
-                            d0 = p0 != 0.f ? d0 : 0.f; d1 = p1 != 0.f ? d1 : 0.f;
-                            d2 = p2 != 0.f ? d2 : 0.f; d3 = p3 != 0.f ? d3 : 0.f;
+                            d0 = (pa & 0xffffu) != 0u ? d0 : 0.f; d1 = (pa >> 16) != 0u ? d1 : 0.f;
+                            d2 = (pb & 0xffffu) != 0u ? d2 : 0.f; d3 = (pb >> 16) != 0u ? d3 : 0.f;
                         }
                         dpack[q * 2 + 0] = pack_bf16(d0, d1);
                         dpack[q * 2 + 1] = pack_bf16(d2, d3);
@@ -556,30 +549,6 @@ constexpr int kThreadsFused = 512 + 256 + 128;  // 16 exp/dS warps, 8 reducer wa
 struct FusedRegs {
     static constexpr int kExp = 88, kReduce = 48, kIssue = 56;
 };
-// P of two entries from their scores and -LSE log2(e)
-__device__ __forceinline__ void p_pair(uint32_t v0, uint32_t v1, float s, float n0, float n1, float &p0, float &p1)
-{
-    uint64_t x, y, z;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(v0), "r"(v1));
-    asm("mov.b64 %0, {%1, %1};" : "=l"(y) : "f"(s));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(n0), "f"(n1));
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(x) : "l"(x), "l"(y), "l"(z));
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(p0), "=f"(p1) : "l"(x));
-    p0 = ex2_approx(p0);
-    p1 = ex2_approx(p1);
-}
-// dS of two entries from their P (bf16 pair), dP and -scale * D
-__device__ __forceinline__ void ds_pair(uint32_t pk, uint32_t v0, uint32_t v1, float s, float n0, float n1, float &d0, float &d1)
-{
-    uint64_t x, y, z, w;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(v0), "r"(v1));
-    asm("mov.b64 %0, {%1, %1};" : "=l"(y) : "f"(s));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(n0), "f"(n1));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(w) : "r"(pk << 16), "r"(pk & 0xffff0000u));
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(x) : "l"(x), "l"(y), "l"(z));
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(x) : "l"(x), "l"(w));
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(x));
-}
 template <int HD, bool FINE>
 __global__ void __launch_bounds__(kThreadsFused, 1)
 tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CUtensorMap mK_,

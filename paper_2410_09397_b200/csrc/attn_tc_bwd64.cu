@@ -306,10 +306,8 @@ tc_bwd_fused64_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_const
                 for (int q = 0; q < 8; ++q) {
                     const float4 nl = nlr[q];
                     float p[4];
-                    p[0] = ex2_approx(fmaf(__uint_as_float(sv[q * 4 + 0]), sl2, nl.x));
-                    p[1] = ex2_approx(fmaf(__uint_as_float(sv[q * 4 + 1]), sl2, nl.y));
-                    p[2] = ex2_approx(fmaf(__uint_as_float(sv[q * 4 + 2]), sl2, nl.z));
-                    p[3] = ex2_approx(fmaf(__uint_as_float(sv[q * 4 + 3]), sl2, nl.w));
+                    p_pair(sv[q * 4 + 0], sv[q * 4 + 1], sl2, nl.x, nl.y, p[0], p[1]);
+                    p_pair(sv[q * 4 + 2], sv[q * 4 + 3], sl2, nl.z, nl.w, p[2], p[3]);
                     if (masked) {
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
@@ -341,25 +339,16 @@ tc_bwd_fused64_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_const
                 uint8_t *slab = smem + L::odS;
 #pragma unroll
                 for (int gg = 0; gg < 4; ++gg) {    // 8 query columns = one 16-byte chunk
-                    float ds[8], p[8];
+                    float ds[8];
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        const uint32_t pk = ppack[gg * 4 + e];   // bf16 -> fp32 is a 16-bit shift
-                        p[2 * e] = __uint_as_float(pk << 16);
-                        p[2 * e + 1] = __uint_as_float(pk & 0xffff0000u);
-                    }
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        const float4 dsc = dsr[gg * 2 + u];
-                        const uint32_t *d4 = &dv[gg * 8 + u * 4];
-                        ds[u * 4 + 0] = p[u * 4 + 0] * fmaf(__uint_as_float(d4[0]), a.scale, dsc.x);
-                        ds[u * 4 + 1] = p[u * 4 + 1] * fmaf(__uint_as_float(d4[1]), a.scale, dsc.y);
-                        ds[u * 4 + 2] = p[u * 4 + 2] * fmaf(__uint_as_float(d4[2]), a.scale, dsc.z);
-                        ds[u * 4 + 3] = p[u * 4 + 3] * fmaf(__uint_as_float(d4[3]), a.scale, dsc.w);
+                        const float4 dsc = dsr[gg * 2 + e / 2];
+                        ds_pair(ppack[gg * 4 + e], dv[gg * 8 + 2 * e], dv[gg * 8 + 2 * e + 1], a.scale, e & 1 ? dsc.z : dsc.x,
+                                e & 1 ? dsc.w : dsc.y, ds[2 * e], ds[2 * e + 1]);
                     }
                     if (masked) {   // stale tail entries of the row vectors may be anything: select, do not multiply
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) ds[e] = p[e] != 0.f ? ds[e] : 0.f;
+                        for (int e = 0; e < 8; ++e) ds[e] = (ppack[gg * 4 + e / 2] & (e & 1 ? 0xffff0000u : 0xffffu)) != 0u ? ds[e] : 0.f;
                     }
                     *reinterpret_cast<uint4 *>(slab + sw128_offset(row, g * 32 + gg * 8)) =
                         make_uint4(pack_bf16(ds[0], ds[1]), pack_bf16(ds[2], ds[3]), pack_bf16(ds[4], ds[5]),

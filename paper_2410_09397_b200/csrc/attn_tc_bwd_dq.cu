@@ -264,7 +264,11 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
                 tmem_ld32(T_S + lane_addr + wg * 32, sv0);
                 tmem_wait_ld();
 #pragma unroll
-                for (int e = 0; e < 32; ++e) p[e] = ex2_fast(fmaf(__uint_as_float(sv0[e]), sl2, nl));
+                for (int e = 0; e < 32; e += 2) {
+                    asm("mov.b64 {%0, %1}, %2;" : "=f"(p[e]), "=f"(p[e + 1]) : "l"(fma_pair(sv0[e], sv0[e + 1], sl2, nl, nl)));
+                    p[e] = ex2_fast(p[e]);
+                    p[e + 1] = ex2_fast(p[e + 1]);
+                }
             }
             if (masked) {
                 const bool causal = mask_is_causal(a.mask_kind);
@@ -286,8 +290,8 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
                 if (lane == 0) mbar_arrive(&bars[DB_DPFREE]);
 #pragma unroll
                 for (int e = 0; e < 32; e += 2) {
-                    const float d0 = p[e] * fmaf(__uint_as_float(dv0[e]), a.scale, dsi);
-                    const float d1 = p[e + 1] * fmaf(__uint_as_float(dv0[e + 1]), a.scale, dsi);
+                    float d0, d1;
+                    mul_pair(fma_pair(dv0[e], dv0[e + 1], a.scale, dsi, dsi), __float_as_uint(p[e]), __float_as_uint(p[e + 1]), d0, d1);
                     dpack[e / 2] = pack_bf16(d0, d1);
                     if constexpr (SPLIT) drest[e / 2] = pack_bf16_rest(d0, d1, dpack[e / 2]);
                 }

@@ -80,6 +80,19 @@ __device__ __forceinline__ float ex2_approx(float x)
     return y;
 }
 
+// P of two entries from their scores and -LSE log2(e)
+__device__ __forceinline__ void p_pair(uint32_t v0, uint32_t v1, float s, float n0, float n1, float &p0, float &p1)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(p0), "=f"(p1) : "l"(fma_pair(v0, v1, s, n0, n1)));
+    p0 = ex2_approx(p0);
+    p1 = ex2_approx(p1);
+}
+// dS of two entries from their P (a bf16 pair; bf16 -> fp32 is a 16-bit shift), dP and -scale * D
+__device__ __forceinline__ void ds_pair(uint32_t pk, uint32_t v0, uint32_t v1, float s, float n0, float n1, float &d0, float &d1)
+{
+    mul_pair(fma_pair(v0, v1, s, n0, n1), pk << 16, pk & 0xffff0000u, d0, d1);
+}
+
 // D pre-pass of the tensor-core backward: nDs_i = -scale * sum_c dO_ic O_ic (the form that packed multiply-adds take) and
 // nlse2_i = -LSE_i * log2(e) (minus infinity for a row with no kept entry, so that its
 // probabilities come out as exactly zero).  16-byte loads, HD/8 lanes share a row.  The same

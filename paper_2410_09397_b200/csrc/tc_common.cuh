@@ -293,6 +293,24 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
     return *reinterpret_cast<uint32_t *>(&v);
 }
 
+// v * s + n and p * (v * s + n) of two entries, an instruction each (the roundings of the scalar forms)
+__device__ __forceinline__ uint64_t fma_pair(uint32_t v0, uint32_t v1, float s, float n0, float n1)
+{
+    uint64_t x, y, z;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(v0), "r"(v1));
+    asm("mov.b64 %0, {%1, %1};" : "=l"(y) : "f"(s));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(n0), "f"(n1));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(x) : "l"(x), "l"(y), "l"(z));
+    return x;
+}
+__device__ __forceinline__ void mul_pair(uint64_t x, uint32_t p0, uint32_t p1, float &d0, float &d1)
+{
+    uint64_t w;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(w) : "r"(p0), "r"(p1));
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(x) : "l"(x), "l"(w));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(x));
+}
+
 // What two fp32 values lose when they are packed as `hi` (pack_bf16), packed the same way: x = hi + lo up to 2^-17 |x|.
 __device__ __forceinline__ uint32_t pack_bf16_rest(float x, float y, uint32_t hi)
 {
