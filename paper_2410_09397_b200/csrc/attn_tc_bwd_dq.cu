@@ -14,7 +14,12 @@
 // the price of summing dQ in a fixed order: 7 products instead of 5 per tile pair.
 // Roles: warps 0-15 = four warpgroups, warpgroup g owning key columns 32 g .. 32 g + 31 of every
 // tile (no barrier couples them, so their exp, dS and tensor-memory phases interleave freely);
-// warp 16 lane 0 issues S and dP, warp 17 lane 0 issues dQ, warp 18 lane 0 runs TMA.  Tensor memory: S0 128, S1 128, dP 128, dQ d columns.
+// warp 16 lane 0 issues S and dP, warp 17 lane 0 issues dQ, warp 18 runs TMA and the schedule.  Tensor memory: S0 128, S1 128, dP 128,
+// dQ d columns.
+//
+// A CTA takes the query tiles of CTAs that have not started yet (cluster launch control): Q, dO and the first products of the next
+// one come while dQ of this one is written out.  24 heads, n = 3000, d = 64: 119 -> 113 us; 32 heads, n = 4096, d = 128, causal:
+// 207 -> 203; 16 heads, n = 2047, d = 128, causal (two terms): 57.6 -> 55.8.
 #include "attn_internal.h"
 #include "tc_common.cuh"
 
@@ -50,41 +55,24 @@ struct DqSmem {
     static constexpr uint32_t oK = odO + kTile;          // NSTK stages
     static constexpr uint32_t oV = oK + NSTK * kTile;    // NSTV stages
     static constexpr uint32_t oBar = oV + NSTV * kTile;
-    static constexpr uint32_t oMisc = oBar + 24 * 8;
-    static constexpr uint32_t kUsed = oMisc + 64;
+    static constexpr uint32_t oWork = oBar + 32 * 8;     // two slots of DqWork, the answer of the scheduler
+    static constexpr uint32_t oMisc = oWork + 2 * 32 + 16;
+    static constexpr uint32_t kUsed = oMisc + 16;
     static constexpr uint32_t kBytes = kUsed < 117 * 1024 ? 117 * 1024 : kUsed;   // one CTA per SM (512 TMEM columns)
     static_assert(kUsed <= 227 * 1024, "shared memory budget");
 };
 
-enum { DB_Q = 0, DB_KFULL = 1, DB_KEMPTY = 4, DB_VFULL = 7, DB_VEMPTY = 9, DB_S = 11, DB_DP = 13, DB_DPFREE = 14, DB_DS = 15,
-       DB_DQ = 17 };
+enum { DB_Q = 0, DB_KFULL = 1, DB_KEMPTY = 4, DB_VFULL = 7, DB_VEMPTY = 9, DB_S = 11, DB_DP = 13, DB_DQ = 14, DB_QEMPTY = 15,
+       DB_CLC = 16, DB_WF = 17, DB_DPFREE = 19, DB_DS = 20, DB_WE = 22, DB_COUNT = 24 };
 
-struct KeyIterD {
-    int kind, n, sub, raw, last_i;
-    const int *cols;
-    __device__ KeyIterD(const DqArgs &a, int it, long bh) : kind(a.mask_kind), n(a.n), sub(1), raw(0), cols(nullptr)
-    {
-        last_i = min(it * TQ + TQ, n) - 1;
-        const int ntk = (n + TKD - 1) / TKD;
-        if (kind == ATTN_MASK_NONE) raw = ntk;
-        else if (kind == ATTN_MASK_CAUSAL) raw = (min(it * TQ + TQ, n) - 1) / TKD + 1;
-        else {
-            sub = a.block / TKD;
-            const int I = it * TQ / a.block;
-            const long mh = a.mask_heads == 1 ? 0 : bh;
-            const int *rp = a.row_ptr + mh * 2 * a.nb + 2 * I;
-            cols = a.col_idx + mh * (long)a.nb * a.nb + rp[0];
-            raw = (rp[1] - rp[0]) * sub;
-        }
-    }
-    __device__ int tile(int idx) const
-    {
-        const int jt = mask_is_block(kind) ? cols[idx / sub] * sub + idx % sub : idx;
-        // block mask AND causal: a key tile that begins after the last query of the tile keeps nothing
-        if (kind == ATTN_MASK_BLOCK_SPARSE_CAUSAL && jt * TKD > last_i) return -1;
-        return jt * TKD < n ? jt : -1;
-    }
+// One unit of work: a query tile of one head and the key tiles that it visits
+struct DqWork {
+    int it, bh, count;   // it = -1: there is no more work
+    int pad;
+    const int *cols;     // key blocks of a mask with lists
+    int pad2[2];
 };
+static_assert(sizeof(DqWork) == 32, "two slots in shared memory");
 
 __device__ __forceinline__ float ex2_fast(float x)
 {
@@ -109,11 +97,14 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
     volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(smem + L::oMisc + 4);
     const Abort ab{abort_flag, a.status};
 
+    volatile DqWork *slots = reinterpret_cast<volatile DqWork *>(smem + L::oWork);
+    uint8_t *answer = smem + L::oWork + 2 * sizeof(DqWork);
+    constexpr int kWarps = kSoftmaxThreads / 32;
+
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-    const int nt = (a.n + TQ - 1) / TQ;
-    const int it = nt - 1 - (int)blockIdx.x;    // heaviest causal tiles first
-    const long bh = blockIdx.y;
-    const int i0 = it * TQ, n = a.n;
+    const int n = a.n;
+    const bool lists = mask_is_block(a.mask_kind), causal = mask_is_causal(a.mask_kind);
+    const int sub = lists ? a.block / TKD : 1;
 
     if ((smem_u32(smem) & 1023u) != 0) {
         chain_wait();
@@ -122,13 +113,8 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
     }
     if (tid == 0) {
         *abort_flag = 0;
-        mbar_init(&bars[DB_Q], 1);
-        for (int s = 0; s < NSTK; ++s) { mbar_init(&bars[DB_KFULL + s], 1); mbar_init(&bars[DB_KEMPTY + s], 1); }
-        for (int s = 0; s < NSTV; ++s) { mbar_init(&bars[DB_VFULL + s], 1); mbar_init(&bars[DB_VEMPTY + s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&bars[DB_S + b], 1); mbar_init(&bars[DB_DS + b], kSoftmaxThreads / 32); }   // one arrival per warp
-        mbar_init(&bars[DB_DP], 1);
-        mbar_init(&bars[DB_DPFREE], kSoftmaxThreads / 32);
-        mbar_init(&bars[DB_DQ], 1);
+        for (int b = 0; b < DB_COUNT; ++b)   // DPFREE, DS: one arrival per warp; WE: both issuers and the dS warps
+            mbar_init(&bars[b], b >= DB_WE ? 2 + kWarps : b >= DB_DPFREE ? kWarps : 1);
         fence_barrier_init();
         prefetch_tensormap(&mQ); prefetch_tensormap(&mK); prefetch_tensormap(&mV); prefetch_tensormap(&mdO);
     }
@@ -140,101 +126,146 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
     chain_release();
     const uint32_t tm = *tmem_base_s;
     const uint32_t T_dP = tm + 256, T_dQ = tm + 384;
-    const KeyIterD iter(a, it, bh);
-    int niter = 0;
-    for (int idx = 0; idx < iter.raw; ++idx) niter += iter.tile(idx) >= 0;
 
+    // the t-th unit of work of this CTA as the loading warp has published it (false: there is none)
+    auto work = [&](int t) { return mbar_wait(&bars[DB_WF + (t & 1)], (t >> 1) & 1, ab) && slots[t & 1].it >= 0; };
+    auto key_tile = [&](const int *cols, int e) { return !lists ? e : sub == 1 ? cols[e] : cols[e / sub] * sub + e % sub; };
+
+    // In every role k counts the key tiles of all units of work so far (a wait for what belongs to a tile before the first returns
+    // at once): the barriers run on, and the loads and first products of the next unit come while dQ of this one is written out.
     if (warp == 18) {
-        // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
-            mbar_expect_tx(&bars[DB_Q], 2 * L::kTile);
-#pragma unroll
-            for (uint32_t sl = 0; sl < L::kSlabs; ++sl) {
-                tma_load_3d(smem + L::oQ + sl * SLAB, &mQ, &bars[DB_Q], sl * 64, i0, (int)bh);
-                tma_load_3d(smem + L::odO + sl * SLAB, &mdO, &bars[DB_Q], sl * 64, i0, (int)bh);
+        // ------------------------------------------------------------ TMA producer, and the schedule
+        const int nt = (n + TQ - 1) / TQ;
+        int bx = blockIdx.x, by = blockIdx.y;
+        int k = 0, nq = 0;
+        bool more = true;
+        for (int t = 0; more; ++t) {
+            const int it = nt - 1 - bx, bh = by, i0 = it * TQ;    // heaviest causal tiles first
+            const int last_i = min(i0 + TQ, n) - 1;
+            const int *cols = nullptr;
+            int count;
+            if (lists) {
+                // the lists ascend: what lies beyond n or (block mask AND causal) begins after the last query is at their end
+                const long mh = a.mask_heads == 1 ? 0 : bh;
+                const int *rp = a.row_ptr + mh * 2 * a.nb + 2 * (i0 / a.block);
+                const int first = rp[0], raw = (rp[1] - first) * sub, limit = causal ? last_i : n - 1;
+                cols = a.col_idx + mh * (long)a.nb * a.nb + first;
+                count = 0;
+                for (int e = lane; e < raw; e += 32) count += key_tile(cols, e) * TKD <= limit;
+                count = __reduce_add_sync(0xffffffffu, count);
+            } else {
+                count = causal ? last_i / TKD + 1 : (n + TKD - 1) / TKD;
             }
-            int k = 0;
-            for (int idx = 0; idx < iter.raw; ++idx) {
-                const int jt = iter.tile(idx);
-                if (jt < 0) continue;
-                const int sk = k % NSTK, sv = k % NSTV;
-                if (k >= NSTK) mbar_wait(&bars[DB_KEMPTY + sk], ((k / NSTK) - 1) & 1, ab);
-                mbar_expect_tx(&bars[DB_KFULL + sk], L::kTile);
+            if (lane == 0) {
+                if (t >= 2) mbar_wait(&bars[DB_WE + (t & 1)], ((t >> 1) - 1) & 1, ab);
+                volatile DqWork &to = slots[t & 1];
+                to.it = it; to.bh = bh; to.count = count; to.cols = cols;
+                mbar_arrive(&bars[DB_WF + (t & 1)]);
+                if (count > 0) {
+                    mbar_wait(&bars[DB_QEMPTY], (nq - 1) & 1, ab);   // dP of the unit before
+                    ++nq;
+                    mbar_expect_tx(&bars[DB_Q], 2 * L::kTile);
 #pragma unroll
-                for (uint32_t sl = 0; sl < L::kSlabs; ++sl)
-                    tma_load_3d(smem + L::oK + sk * L::kTile + sl * SLAB, &mK, &bars[DB_KFULL + sk], sl * 64, jt * TKD, (int)bh);
-                if (k >= NSTV) mbar_wait(&bars[DB_VEMPTY + sv], ((k / NSTV) - 1) & 1, ab);
-                mbar_expect_tx(&bars[DB_VFULL + sv], L::kTile);
+                    for (uint32_t sl = 0; sl < L::kSlabs; ++sl) {
+                        tma_load_3d(smem + L::oQ + sl * SLAB, &mQ, &bars[DB_Q], sl * 64, i0, bh);
+                        tma_load_3d(smem + L::odO + sl * SLAB, &mdO, &bars[DB_Q], sl * 64, i0, bh);
+                    }
+                } else {
+                    clc_request(answer, &bars[DB_CLC]);
+                }
+                for (int e = 0; e < count; ++e, ++k) {
+                    const int jt = key_tile(cols, e), sk = k % NSTK, sv = k % NSTV;
+                    // the next unit of work, asked for early enough that the answer is there when the loads get to it
+                    if (e == max(count - 2, 0)) clc_request(answer, &bars[DB_CLC]);
+                    if (k >= NSTK) mbar_wait(&bars[DB_KEMPTY + sk], ((k / NSTK) - 1) & 1, ab);
+                    mbar_expect_tx(&bars[DB_KFULL + sk], L::kTile);
 #pragma unroll
-                for (uint32_t sl = 0; sl < L::kSlabs; ++sl)
-                    tma_load_3d(smem + L::oV + sv * L::kTile + sl * SLAB, &mV, &bars[DB_VFULL + sv], sl * 64, jt * TKD, (int)bh);
-                ++k;
+                    for (uint32_t sl = 0; sl < L::kSlabs; ++sl)
+                        tma_load_3d(smem + L::oK + sk * L::kTile + sl * SLAB, &mK, &bars[DB_KFULL + sk], sl * 64, jt * TKD, bh);
+                    if (k >= NSTV) mbar_wait(&bars[DB_VEMPTY + sv], ((k / NSTV) - 1) & 1, ab);
+                    mbar_expect_tx(&bars[DB_VFULL + sv], L::kTile);
+#pragma unroll
+                    for (uint32_t sl = 0; sl < L::kSlabs; ++sl)
+                        tma_load_3d(smem + L::oV + sv * L::kTile + sl * SLAB, &mV, &bars[DB_VFULL + sv], sl * 64, jt * TKD, bh);
+                }
+                more = mbar_wait(&bars[DB_CLC], t & 1, ab) && clc_answer(answer, bx, by);
+                if (!more) {
+                    if (t >= 1) mbar_wait(&bars[DB_WE + ((t + 1) & 1)], (((t + 1) >> 1) - 1) & 1, ab);
+                    slots[(t + 1) & 1].it = -1;
+                    mbar_arrive(&bars[DB_WF + ((t + 1) & 1)]);
+                }
             }
-            if (niter == 0) mbar_wait(&bars[DB_Q], 0, ab);   // let the Q / dO load land before exit
+            more = __shfl_sync(0xffffffffu, (int)more, 0) != 0;
+            bx = __shfl_sync(0xffffffffu, bx, 0);
+            by = __shfl_sync(0xffffffffu, by, 0);
         }
     } else if (warp == 16) {
         // ------------------------------------------------------------ MMA issuer A: the products the warps wait for, S and dP,
         // one tile ahead.  (Two issuing threads: a thread that waits on a barrier or commits cannot keep the short
         // queue of the tensor pipe filled; B's dQ products are ordered against A's through barriers only.)
-        if (lane == 0 && niter > 0) {
+        if (lane == 0) {
             constexpr uint32_t idesc_s = idesc_bf16(128, 128, 0, 0);
             constexpr uint32_t kSlab = SLAB >> 4;
             const uint32_t kQ = desc_lo_kmajor(smem_u32(smem + L::oQ)), kdO = desc_lo_kmajor(smem_u32(smem + L::odO));
-            auto issue_S = [&](int k) {
-                const int s = k % NSTK;
-                mbar_wait(&bars[DB_KFULL + s], (k / NSTK) & 1, ab);
-                // the buffer of S(k) held dS(k-2): the dQ product of tile k-2 (other thread) must have consumed it
-                if (k >= 2) mbar_wait(&bars[DB_KEMPTY + (k - 2) % NSTK], ((k - 2) / NSTK) & 1, ab);
-                tcgen05_fence_after();
-                const uint32_t kK = desc_lo_kmajor(smem_u32(smem + L::oK + s * L::kTile));
+            int k = 0, nq = 0;
+            for (int t = 0; work(t); ++t) {
+                const int end = k + slots[t & 1].count;
+                mbar_arrive(&bars[DB_WE + (t & 1)]);
+                if (k == end) continue;
+                mbar_wait(&bars[DB_Q], nq & 1, ab);
+                ++nq;
+                for (; k < end; ++k) {
+                    const int s = k % NSTK;
+                    mbar_wait(&bars[DB_KFULL + s], (k / NSTK) & 1, ab);
+                    // the buffer of S(k) held dS(k-2): the dQ product of tile k-2 (other thread) must have consumed it
+                    if (k >= 2) mbar_wait(&bars[DB_KEMPTY + (k - 2) % NSTK], ((k - 2) / NSTK) & 1, ab);
+                    tcgen05_fence_after();
+                    const uint32_t kK = desc_lo_kmajor(smem_u32(smem + L::oK + s * L::kTile));
 #pragma unroll
-                for (int kk = 0; kk < HD / 16; ++kk) {
-                    const uint32_t off = (kk / 4) * kSlab + (kk % 4) * 2;
-                    mma_ss_lo(tm + (k & 1) * 128, kQ + off, kK + off, idesc_s, kk > 0);
-                }
-                mma_commit(&bars[DB_S + (k & 1)]);
-            };
-            auto issue_dP = [&](int k) {
-                mbar_wait(&bars[DB_VFULL + k % NSTV], (k / NSTV) & 1, ab);
-                tcgen05_fence_after();
-                const uint32_t kV = desc_lo_kmajor(smem_u32(smem + L::oV + (k % NSTV) * L::kTile));
+                    for (int kk = 0; kk < HD / 16; ++kk) {
+                        const uint32_t off = (kk / 4) * kSlab + (kk % 4) * 2;
+                        mma_ss_lo(tm + (k & 1) * 128, kQ + off, kK + off, idesc_s, kk > 0);
+                    }
+                    mma_commit(&bars[DB_S + (k & 1)]);
+                    // dP(k) once every thread has read dP(k-1) out of tensor memory
+                    mbar_wait(&bars[DB_DPFREE], (k - 1) & 1, ab);
+                    mbar_wait(&bars[DB_VFULL + k % NSTV], (k / NSTV) & 1, ab);
+                    tcgen05_fence_after();
+                    const uint32_t kV = desc_lo_kmajor(smem_u32(smem + L::oV + (k % NSTV) * L::kTile));
 #pragma unroll
-                for (int kk = 0; kk < HD / 16; ++kk) {
-                    const uint32_t off = (kk / 4) * kSlab + (kk % 4) * 2;
-                    mma_ss_lo(T_dP, kdO + off, kV + off, idesc_s, kk > 0);
+                    for (int kk = 0; kk < HD / 16; ++kk) {
+                        const uint32_t off = (kk / 4) * kSlab + (kk % 4) * 2;
+                        mma_ss_lo(T_dP, kdO + off, kV + off, idesc_s, kk > 0);
+                    }
+                    mma_commit(&bars[DB_DP]);
+                    mma_commit(&bars[DB_VEMPTY + k % NSTV]);
                 }
-                mma_commit(&bars[DB_DP]);
-                mma_commit(&bars[DB_VEMPTY + k % NSTV]);
-            };
-            mbar_wait(&bars[DB_Q], 0, ab);
-            issue_S(0);
-            issue_dP(0);
-            for (int k = 0; k + 1 < niter; ++k) {
-                issue_S(k + 1);
-                // dP(k+1) once every thread has read dP(k) out of tensor memory
-                mbar_wait(&bars[DB_DPFREE], k & 1, ab);
-                tcgen05_fence_after();
-                issue_dP(k + 1);
+                mma_commit(&bars[DB_QEMPTY]);
             }
         }
     } else if (warp == 17) {
         // ------------------------------------------------------------ MMA issuer B: dQ_i += dS K_j
-        if (lane == 0 && niter > 0) {
+        if (lane == 0) {
             constexpr uint32_t idesc_dq = idesc_bf16(128, HD, 0, 1);
-            for (int k = 0; k < niter; ++k) {
-                const int s = k % NSTK, b = k & 1;
-                mbar_wait(&bars[DB_KFULL + s], (k / NSTK) & 1, ab);
-                mbar_wait(&bars[DB_DS + b], (k >> 1) & 1, ab);
-                tcgen05_fence_after();
-                const uint32_t mK_ = desc_lo_mnmajor(smem_u32(smem + L::oK + s * L::kTile), SLAB);
+            int k = 0;
+            for (int t = 0; work(t); ++t) {
+                const int begin = k, end = k + slots[t & 1].count;
+                mbar_arrive(&bars[DB_WE + (t & 1)]);
+                for (; k < end; ++k) {
+                    const int s = k % NSTK, b = k & 1;
+                    mbar_wait(&bars[DB_KFULL + s], (k / NSTK) & 1, ab);
+                    mbar_wait(&bars[DB_DS + b], (k >> 1) & 1, ab);   // of every warp: the first of a unit has been preceded by their reading dQ
+                    tcgen05_fence_after();
+                    const uint32_t mK_ = desc_lo_mnmajor(smem_u32(smem + L::oK + s * L::kTile), SLAB);
 #pragma unroll
-                for (int kk = 0; kk < TKD / 16; ++kk) {
-                    const uint32_t dS = tm + b * 128 + (kk / 2) * 32 + (kk % 2) * 8;
-                    mma_ts_lo(T_dQ, dS, mK_ + kk * 128, idesc_dq, (k > 0) || (kk > 0));
-                    if constexpr (SPLIT) mma_ts_lo(T_dQ, dS + 16, mK_ + kk * 128, idesc_dq, 1);
+                    for (int kk = 0; kk < TKD / 16; ++kk) {
+                        const uint32_t dS = tm + b * 128 + (kk / 2) * 32 + (kk % 2) * 8;
+                        mma_ts_lo(T_dQ, dS, mK_ + kk * 128, idesc_dq, (k > begin) || (kk > 0));
+                        if constexpr (SPLIT) mma_ts_lo(T_dQ, dS + 16, mK_ + kk * 128, idesc_dq, 1);
+                    }
+                    mma_commit(&bars[DB_KEMPTY + s]);
                 }
-                mma_commit(&bars[DB_KEMPTY + s]);
-                if (k == niter - 1) mma_commit(&bars[DB_DQ]);
+                if (end > begin) mma_commit(&bars[DB_DQ]);
             }
         }
     } else {
@@ -242,97 +273,92 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
         const int wg = warp / 4;
         const int row = (warp % 4) * 32 + lane;           // tensor-memory lane = query row of the tile
         const uint32_t lane_addr = (uint32_t)((warp % 4) * 32) << 16;
-        const int ig = i0 + row;
         const float sl2 = a.scale * 1.4426950408889634f;
-        const float nl = ig < n ? a.nLSE2[(size_t)bh * a.ns + ig] : -INFINITY;   // -inf: every probability of the row is 0
-        const float dsi = ig < n ? a.nDs[(size_t)bh * a.ns + ig] : 0.f;
-        int k = 0;
-        for (int idx = 0; idx < iter.raw; ++idx) {
-            const int jt = iter.tile(idx);
-            if (jt < 0) continue;
-            const int b = k & 1, j0 = jt * TKD + wg * 32;
-            const uint32_t T_S = tm + b * 128;
-            // a mask finer than the tile: the keep bits of this thread's query row and its 32 key columns
-            uint32_t kw = 0xffffffffu;
-            if (a.fine.mode) kw = (ig < n && j0 < n) ? fine_word(a.fine, a.mask_heads, bh, true, ig, j0) : 0u;
-            const bool masked = (mask_is_causal(a.mask_kind) && jt * TKD + TKD - 1 > i0) || jt * TKD + TKD > n || a.fine.mode != 0;
-            mbar_wait(&bars[DB_S + b], (k >> 1) & 1, ab);
-            tcgen05_fence_after();
-            float p[32];
-            {
-                uint32_t sv0[32];
-                tmem_ld32(T_S + lane_addr + wg * 32, sv0);
-                tmem_wait_ld();
+        const bool wide = ((uintptr_t)a.dQ & 31) == 0;
+        int k = 0, nq = 0;
+        for (int t = 0; work(t); ++t) {
+            const int i0 = slots[t & 1].it * TQ, bh = slots[t & 1].bh, count = slots[t & 1].count, begin = k;
+            const int *cols = slots[t & 1].cols;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars[DB_WE + (t & 1)]);
+            const int ig = i0 + row;
+            const float nl = ig < n ? a.nLSE2[(size_t)bh * a.ns + ig] : -INFINITY;   // -inf: every probability of the row is 0
+            const float dsi = ig < n ? a.nDs[(size_t)bh * a.ns + ig] : 0.f;
+            for (; k < begin + count; ++k) {
+                const int jt = key_tile(cols, k - begin);
+                const int b = k & 1, j0 = jt * TKD + wg * 32;
+                const uint32_t T_S = tm + b * 128;
+                // a mask finer than the tile: the keep bits of this thread's query row and its 32 key columns
+                uint32_t kw = 0xffffffffu;
+                if (a.fine.mode) kw = (ig < n && j0 < n) ? fine_word(a.fine, a.mask_heads, bh, true, ig, j0) : 0u;
+                const bool masked = (causal && jt * TKD + TKD - 1 > i0) || jt * TKD + TKD > n || a.fine.mode != 0;
+                mbar_wait(&bars[DB_S + b], (k >> 1) & 1, ab);
+                tcgen05_fence_after();
+                float p[32];
+                {
+                    uint32_t sv0[32];
+                    tmem_ld32(T_S + lane_addr + wg * 32, sv0);
+                    tmem_wait_ld();
 #pragma unroll
-                for (int e = 0; e < 32; e += 2) {
-                    asm("mov.b64 {%0, %1}, %2;" : "=f"(p[e]), "=f"(p[e + 1]) : "l"(fma_pair(sv0[e], sv0[e + 1], sl2, nl, nl)));
-                    p[e] = ex2_fast(p[e]);
-                    p[e + 1] = ex2_fast(p[e + 1]);
+                    for (int e = 0; e < 32; e += 2) {
+                        asm("mov.b64 {%0, %1}, %2;" : "=f"(p[e]), "=f"(p[e + 1]) : "l"(fma_pair(sv0[e], sv0[e + 1], sl2, nl, nl)));
+                        p[e] = ex2_fast(p[e]);
+                        p[e + 1] = ex2_fast(p[e + 1]);
+                    }
                 }
-            }
-            if (masked) {
-                const bool causal = mask_is_causal(a.mask_kind);
+                if (masked) {
 #pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    const int jg = j0 + e;
-                    if (jg >= n || (causal && jg > ig) || !((kw >> e) & 1u)) p[e] = 0.f;
+                    for (int e = 0; e < 32; ++e) {
+                        const int jg = j0 + e;
+                        if (jg >= n || (causal && jg > ig) || !((kw >> e) & 1u)) p[e] = 0.f;
+                    }
                 }
-            }
-            mbar_wait(&bars[DB_DP], k & 1, ab);
-            tcgen05_fence_after();
-            uint32_t dpack[16], drest[SPLIT ? 16 : 1];
-            {
-                uint32_t dv0[32];
-                tmem_ld32(T_dP + lane_addr + wg * 32, dv0);
-                tmem_wait_ld();
+                mbar_wait(&bars[DB_DP], k & 1, ab);
+                tcgen05_fence_after();
+                uint32_t dpack[16], drest[SPLIT ? 16 : 1];
+                {
+                    uint32_t dv0[32];
+                    tmem_ld32(T_dP + lane_addr + wg * 32, dv0);
+                    tmem_wait_ld();
+                    tcgen05_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bars[DB_DPFREE]);
+#pragma unroll
+                    for (int e = 0; e < 32; e += 2) {
+                        float d0, d1;
+                        mul_pair(fma_pair(dv0[e], dv0[e + 1], a.scale, dsi, dsi), __float_as_uint(p[e]), __float_as_uint(p[e + 1]), d0, d1);
+                        dpack[e / 2] = pack_bf16(d0, d1);
+                        if constexpr (SPLIT) drest[e / 2] = pack_bf16_rest(d0, d1, dpack[e / 2]);
+                    }
+                }
+                // dS (bf16 pairs) over the first 16 of the 32 S columns this thread has read itself
+                tmem_st16(T_S + lane_addr + wg * 32, dpack);
+                if constexpr (SPLIT) tmem_st16(T_S + lane_addr + wg * 32 + 16, drest);
+                tmem_wait_st();
                 tcgen05_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&bars[DB_DPFREE]);
-#pragma unroll
-                for (int e = 0; e < 32; e += 2) {
-                    float d0, d1;
-                    mul_pair(fma_pair(dv0[e], dv0[e + 1], a.scale, dsi, dsi), __float_as_uint(p[e]), __float_as_uint(p[e + 1]), d0, d1);
-                    dpack[e / 2] = pack_bf16(d0, d1);
-                    if constexpr (SPLIT) drest[e / 2] = pack_bf16_rest(d0, d1, dpack[e / 2]);
-                }
+                if (lane == 0) mbar_arrive(&bars[DB_DS + b]);
             }
-            // dS (bf16 pairs) over the first 16 of the 32 S columns this thread has read itself
-            tmem_st16(T_S + lane_addr + wg * 32, dpack);
-            if constexpr (SPLIT) tmem_st16(T_S + lane_addr + wg * 32 + 16, drest);
-            tmem_wait_st();
-            tcgen05_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&bars[DB_DS + b]);
-            ++k;
-        }
-        // ------------------------------------------------------------ epilogue: dQ_i (dS carried the scale)
-        if (k > 0) {
-            mbar_wait(&bars[DB_DQ], 0, ab);
-            tcgen05_fence_after();
-        }
-        constexpr int OW = HD / 4;   // dQ columns per warpgroup: 32 or 16
-        const int ic = ig < n ? ig : 0;
-        __nv_bfloat16 *pq = a.dQ + ((size_t)bh * n + ic) * HD + wg * OW;
-        {
-            constexpr int c = 0;
-            uint32_t v[32];
-            if (k > 0) {
-                if (OW == 32) tmem_ld32(T_dQ + lane_addr + wg * OW, v);
-                else tmem_ld16(T_dQ + lane_addr + wg * OW, *reinterpret_cast<uint32_t(*)[16]>(v));
+            // -------------------------------------------------------- epilogue: dQ_i (dS carried the scale)
+            if (count > 0) {
+                mbar_wait(&bars[DB_DQ], nq & 1, ab);
+                ++nq;
+                tcgen05_fence_after();
+            }
+            constexpr int OW = HD / 4;   // dQ columns per warpgroup: 32 or 16
+            const int ic = ig < n ? ig : 0;
+            __nv_bfloat16 *pq = a.dQ + ((size_t)bh * n + ic) * HD + wg * OW;
+#pragma unroll
+            for (int e0 = 0; e0 < OW; e0 += 16) {
+                uint32_t v[16], y[8];
+                tmem_ld16(T_dQ + lane_addr + wg * OW + e0, v);
                 tmem_wait_ld();
-            } else {
 #pragma unroll
-                for (int e = 0; e < 32; ++e) v[e] = 0u;
+                for (int u = 0; u < 8; ++u)   // without a key tile nothing has been accumulated
+                    y[u] = count > 0 ? pack_bf16(__uint_as_float(v[2 * u]), __uint_as_float(v[2 * u + 1])) : 0u;
+                if (ig < n) store32(pq + e0, y, wide);
             }
-            if (ig < n) {
-#pragma unroll
-                for (int e = 0; e < OW; e += 8)
-                    *reinterpret_cast<uint4 *>(pq + c + e) =
-                        make_uint4(pack_bf16(__uint_as_float(v[e]), __uint_as_float(v[e + 1])),
-                                   pack_bf16(__uint_as_float(v[e + 2]), __uint_as_float(v[e + 3])),
-                                   pack_bf16(__uint_as_float(v[e + 4]), __uint_as_float(v[e + 5])),
-                                   pack_bf16(__uint_as_float(v[e + 6]), __uint_as_float(v[e + 7])));
-            }
+            tcgen05_fence_before();
         }
     }
     tcgen05_fence_before();
