@@ -50,27 +50,25 @@ struct BwdSmem {
     static constexpr uint32_t oLSE = odS + NdS * 2 * SLAB;
     static constexpr uint32_t oD = oLSE + NS * 128 * 4;
     static constexpr uint32_t oBar = oD + NS * 128 * 4;    // mbarriers (8 bytes each)
-    static constexpr uint32_t oWork = oBar + 32 * 8;      // two slots of FusedWork, the answer of the scheduler
+    static constexpr uint32_t oWork = oBar + 32 * 8;      // two slots of KeyWork, the answer of the scheduler
     static constexpr uint32_t oTile = oWork + 2 * 32 + 16;// query tile of the last four loads
     static constexpr uint32_t oMisc = oTile + 16;         // tmem base, abort flag
     static constexpr uint32_t kBytes = oMisc + 16;
     static_assert(kBytes <= 227 * 1024, "shared memory budget");
 };
 
-using TileIter = TileIterT<TQ>;
-
 // barrier indices of the fused kernel; P exists once per 64-query half of a tile
 enum { V2_KF = 0, V2_KE = 1, V2_VF = 2, V2_VE = 3, V2_QFULL = 4, V2_QEMPTY = 7, V2_S = 10, V2_DP = 11, V2_DQ = 12, V2_CLC = 13, V2_WF = 14,
        V2_WE = 16, V2_SLD = 18, V2_DPLD = 19, V2_DS = 20, V2_P = 21, V2_DQDONE = 23, V2_DQREL = 24 };
 
-// One unit of work of the fused kernel: a key tile of one head and the query tiles that it visits
-struct FusedWork {
+// One unit of work: a key tile of one head and the query tiles that it visits
+struct KeyWork {
     int jt, bh, count;   // jt = -1: there is no more work
     int first;           // the first query tile, or its place in the list
     const int *rows;     // query blocks of a mask with lists
     int pad[2];
 };
-static_assert(sizeof(FusedWork) == 32, "two slots in shared memory");
+static_assert(sizeof(KeyWork) == 32, "two slots in shared memory");
 
 
 // ---------------------------------------------------------------------------------------
@@ -84,6 +82,10 @@ static_assert(sizeof(FusedWork) == 32, "two slots in shared memory");
 // dS^T(k-1)) and S^T(k+1) (once dP^T(k) has been copied out); B issues dV(k) and dK(k).  The 32 KB that
 // dS^T does not take in shared memory hold a third Q stage; Q, dO and the row statistics are released
 // separately (dO after dV, Q after dK, LSE / D after the dS phase).
+//
+// A CTA takes the key tiles of CTAs that have not started yet, as in the fused kernel.  32 heads, n = 4096, d = 128, causal: 293 ->
+// 267 us; 32 heads, n = 1024, d = 64, causal: 35.2 -> 33.1; 24 heads, n = 3000, d = 64, no mask: 205 -> 202; two terms, 16 heads,
+// n = 2047, d = 128, causal: 65.8 -> 63.9.
 //
 // SPLIT: P and dS enter their products as two bf16 terms each, x = hi + lo up to 2^-17, for calls whose P and dS must not be
 // rounded to one (bf16 storage whose length is no multiple of 8): six product units instead of four.  P^T then fills region B,
@@ -100,13 +102,41 @@ template <int HD> struct DkdvSmem {
     static constexpr uint32_t oLSE = odO + 2 * kTile;       // 2 stages x 128 floats
     static constexpr uint32_t oD = oLSE + 2 * 128 * 4;
     static constexpr uint32_t oBar = oD + 2 * 128 * 4;
-    static constexpr uint32_t oMisc = oBar + 24 * 8;
-    static constexpr uint32_t kBytes = oMisc + 64;
+    static constexpr uint32_t oWork = oBar + 40 * 8;        // two slots of KeyWork, the answer of the scheduler
+    static constexpr uint32_t oMisc = oWork + 2 * 32 + 16;
+    static constexpr uint32_t kBytes = oMisc + 16;
     static_assert(kBytes <= 227 * 1024, "shared memory budget");
 };
-enum { KD_KV = 0, KD_QFULL = 1, KD_QEMPTY = 4, KD_OFULL = 7, KD_OEMPTY = 9, KD_LFULL = 11, KD_LEMPTY = 13,
-       KD_S = 15, KD_DP = 16, KD_SLD = 17, KD_DPLD = 18, KD_P = 19, KD_DS = 21, KD_DONE = 22 };
+enum { KD_KV = 0, KD_QFULL = 1, KD_QEMPTY = 4, KD_OFULL = 7, KD_OEMPTY = 9, KD_LFULL = 11, KD_S = 13, KD_DP = 14, KD_DONE = 15,
+       KD_KVE = 16, KD_CLC = 17, KD_WF = 18, KD_LEMPTY = 20, KD_SLD = 22, KD_DPLD = 23, KD_DS = 24, KD_P = 25, KD_WE = 27, KD_COUNT = 29 };
 constexpr int kThreadsDkdv = 512 + 128;   // 16 exp/dS warps, issuer A, TMA producer, issuer B, one idle warp
+
+// The query tiles of a key tile: places first .. first + count - 1 of `rows` (a mask with lists) or the tiles themselves.  By a
+// whole warp.
+__device__ __forceinline__ void query_range(const BwdArgs &a, int jt, int bh, int lane, const int *&rows, int &first, int &count)
+{
+    const bool causal = mask_is_causal(a.mask_kind);
+    if (!mask_is_block(a.mask_kind)) {
+        first = causal ? jt : 0;
+        count = (a.n + TQ - 1) / TQ - first;
+        return;
+    }
+    // the lists ascend: what lies beyond n is at their end, and (block mask AND causal) what ends before the key tile begins at
+    // their start
+    const int sub = a.block / TQ, J = jt / (a.block / TK);
+    const long mh = a.mask_heads == 1 ? 0 : bh;
+    const int *cp = a.col_ptr + mh * 2 * a.nb + 2 * J;
+    const int start = cp[0], raw = (cp[1] - start) * sub;
+    rows = a.row_idx + mh * (long)a.nb * a.nb + start;
+    int before = 0, within = 0;
+    for (int e = lane; e < raw; e += 32) {
+        const int it = rows[e / sub] * sub + e % sub;
+        before += causal && it < jt;
+        within += it * TQ < a.n;
+    }
+    first = __reduce_add_sync(0xffffffffu, before);
+    count = max((int)__reduce_add_sync(0xffffffffu, within) - first, 0);
+}
 
 template <int HD, bool SPLIT>
 __global__ void __launch_bounds__(kThreadsDkdv, 1)
@@ -122,9 +152,11 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
     const Abort ab{abort_flag, a.status};
 
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-    const int jt = blockIdx.x / a.group;
-    const long bh = (long)blockIdx.y * a.group + blockIdx.x % a.group;
-    const int j0 = jt * TK, n = a.n;
+    const int n = a.n;
+    const bool lists = mask_is_block(a.mask_kind), causal = mask_is_causal(a.mask_kind);
+    const int sub = lists ? a.block / TQ : 1;
+    volatile KeyWork *slots = reinterpret_cast<volatile KeyWork *>(smem + L::oWork);
+    uint8_t *answer = smem + L::oWork + 2 * sizeof(KeyWork);
 
     if ((smem_u32(smem) & 1023u) != 0) {
         chain_wait();
@@ -133,21 +165,8 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
     }
     if (tid == 0) {
         *abort_flag = 0;
-        mbar_init(&bars[KD_KV], 1);
-        for (int s = 0; s < 3; ++s) { mbar_init(&bars[KD_QFULL + s], 1); mbar_init(&bars[KD_QEMPTY + s], 1); }
-        for (int s = 0; s < 2; ++s) {
-            mbar_init(&bars[KD_OFULL + s], 1);
-            mbar_init(&bars[KD_OEMPTY + s], 1);
-            mbar_init(&bars[KD_LFULL + s], 1);
-            mbar_init(&bars[KD_LEMPTY + s], kExpWarps);
-            mbar_init(&bars[KD_P + s], kHalfWarps);
-        }
-        mbar_init(&bars[KD_S], 1);
-        mbar_init(&bars[KD_DP], 1);
-        mbar_init(&bars[KD_SLD], kExpWarps);
-        mbar_init(&bars[KD_DPLD], kExpWarps);
-        mbar_init(&bars[KD_DS], kExpWarps);
-        mbar_init(&bars[KD_DONE], 1);
+        for (int b = 0; b < KD_COUNT; ++b)   // WE: both issuers and the exp / dS warps
+            mbar_init(&bars[b], b >= KD_WE ? 2 + kExpWarps : b >= KD_P ? kHalfWarps : b >= KD_LEMPTY ? kExpWarps : 1);
         fence_barrier_init();
         prefetch_tensormap(&mQ); prefetch_tensormap(&mK_); prefetch_tensormap(&mV); prefetch_tensormap(&mdO);
     }
@@ -163,42 +182,70 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
     const uint32_t T_dS = !SPLIT ? T_B + 32 : kShareB ? T_B : tm + 384;
     constexpr uint32_t HALF_ROWS = 64 * 128;   // byte offset of rows 64.. inside a [128][64] slab
 
-    const TileIter iter(a, jt, bh);
+    // the t-th unit of work of this CTA as the loading warp has published it (false: there is none)
+    auto work = [&](int t) { return mbar_wait(&bars[KD_WF + (t & 1)], (t >> 1) & 1, ab) && slots[t & 1].jt >= 0; };
+    auto query_tile = [&](const int *rows, int e) { return !lists ? e : sub == 1 ? rows[e] : rows[e / sub] * sub + e % sub; };
+
+    // In every role k counts the query tiles of all units of work so far (a wait for what belongs to a tile before the first
+    // returns at once); units follow one another as in the fused kernel.
 
     if (warp == 17) {
-        // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
-            mbar_expect_tx(&bars[KD_KV], 2 * L::kTile);
+        // ------------------------------------------------------------ TMA producer, and the schedule
+        int bx = blockIdx.x, by = blockIdx.y;
+        int k = 0, nkv = 0;
+        bool more = true;
+        for (int t = 0; more; ++t) {
+            const int jt = bx / a.group, bh = by * a.group + bx % a.group, j0 = jt * TK;
+            int count, first;
+            const int *rows = nullptr;
+            query_range(a, jt, bh, lane, rows, first, count);
+            if (lane == 0) {
+                if (t >= 2) mbar_wait(&bars[KD_WE + (t & 1)], ((t >> 1) - 1) & 1, ab);
+                volatile KeyWork &to = slots[t & 1];
+                to.jt = jt; to.bh = bh; to.count = count; to.first = first; to.rows = rows;
+                mbar_arrive(&bars[KD_WF + (t & 1)]);
+                if (count > 0) {
+                    mbar_wait(&bars[KD_KVE], (nkv - 1) & 1, ab);   // S^T and dP^T of the unit before
+                    ++nkv;
+                    mbar_expect_tx(&bars[KD_KV], 2 * L::kTile);
 #pragma unroll
-            for (uint32_t sl = 0; sl < L::kSlabs; ++sl) {
-                tma_load_3d(smem + L::oK + sl * SLAB, &mK_, &bars[KD_KV], sl * 64, j0, (int)bh);
-                tma_load_3d(smem + L::oV + sl * SLAB, &mV, &bars[KD_KV], sl * 64, j0, (int)bh);
+                    for (uint32_t sl = 0; sl < L::kSlabs; ++sl) {
+                        tma_load_3d(smem + L::oK + sl * SLAB, &mK_, &bars[KD_KV], sl * 64, j0, bh);
+                        tma_load_3d(smem + L::oV + sl * SLAB, &mV, &bars[KD_KV], sl * 64, j0, bh);
+                    }
+                } else {
+                    clc_request(answer, &bars[KD_CLC]);
+                }
+                for (int e = 0; e < count; ++e, ++k) {
+                    const int i0 = query_tile(rows, first + e) * TQ, sq = k % 3, s2 = k & 1;
+                    const uint32_t nrows = min(TQ, a.ns - i0);
+                    // the next unit of work, asked for early enough that the answer is there when the loads get to it
+                    if (e == max(count - 2, 0)) clc_request(answer, &bars[KD_CLC]);
+                    if (k >= 3) mbar_wait(&bars[KD_QEMPTY + sq], ((k / 3) - 1) & 1, ab);
+                    mbar_expect_tx(&bars[KD_QFULL + sq], L::kTile);
+#pragma unroll
+                    for (uint32_t sl = 0; sl < L::kSlabs; ++sl)
+                        tma_load_3d(smem + L::oQ + sq * L::kTile + sl * SLAB, &mQ, &bars[KD_QFULL + sq], sl * 64, i0, bh);
+                    if (k >= 2) mbar_wait(&bars[KD_LEMPTY + s2], ((k >> 1) - 1) & 1, ab);
+                    mbar_expect_tx(&bars[KD_LFULL + s2], 2 * nrows * 4);
+                    bulk_load_1d(smem + L::oLSE + s2 * 512, a.nLSE2 + (size_t)bh * a.ns + i0, nrows * 4, &bars[KD_LFULL + s2]);
+                    bulk_load_1d(smem + L::oD + s2 * 512, a.nDs + (size_t)bh * a.ns + i0, nrows * 4, &bars[KD_LFULL + s2]);
+                    if (k >= 2) mbar_wait(&bars[KD_OEMPTY + s2], ((k >> 1) - 1) & 1, ab);
+                    mbar_expect_tx(&bars[KD_OFULL + s2], L::kTile);
+#pragma unroll
+                    for (uint32_t sl = 0; sl < L::kSlabs; ++sl)
+                        tma_load_3d(smem + L::odO + s2 * L::kTile + sl * SLAB, &mdO, &bars[KD_OFULL + s2], sl * 64, i0, bh);
+                }
+                more = mbar_wait(&bars[KD_CLC], t & 1, ab) && clc_answer(answer, bx, by);
+                if (!more) {
+                    if (t >= 1) mbar_wait(&bars[KD_WE + ((t + 1) & 1)], (((t + 1) >> 1) - 1) & 1, ab);
+                    slots[(t + 1) & 1].jt = -1;
+                    mbar_arrive(&bars[KD_WF + ((t + 1) & 1)]);
+                }
             }
-            int k = 0;
-            for (int idx = 0; idx < iter.raw; ++idx) {
-                const int it = iter.tile(idx);
-                if (it < 0) continue;
-                const int i0 = it * TQ, sq = k % 3, s2 = k & 1;
-                const uint32_t rows = min(TQ, a.ns - i0);
-                if (k >= 3) mbar_wait(&bars[KD_QEMPTY + sq], ((k / 3) - 1) & 1, ab);
-                mbar_expect_tx(&bars[KD_QFULL + sq], L::kTile);
-#pragma unroll
-                for (uint32_t sl = 0; sl < L::kSlabs; ++sl)
-                    tma_load_3d(smem + L::oQ + sq * L::kTile + sl * SLAB, &mQ, &bars[KD_QFULL + sq], sl * 64, i0, (int)bh);
-                if (k >= 2) mbar_wait(&bars[KD_LEMPTY + s2], ((k >> 1) - 1) & 1, ab);
-                mbar_expect_tx(&bars[KD_LFULL + s2], 2 * rows * 4);
-                bulk_load_1d(smem + L::oLSE + s2 * 512, a.nLSE2 + bh * a.ns + i0, rows * 4, &bars[KD_LFULL + s2]);
-                bulk_load_1d(smem + L::oD + s2 * 512, a.nDs + bh * a.ns + i0, rows * 4, &bars[KD_LFULL + s2]);
-                if (k >= 2) mbar_wait(&bars[KD_OEMPTY + s2], ((k >> 1) - 1) & 1, ab);
-                mbar_expect_tx(&bars[KD_OFULL + s2], L::kTile);
-#pragma unroll
-                for (uint32_t sl = 0; sl < L::kSlabs; ++sl)
-                    tma_load_3d(smem + L::odO + s2 * L::kTile + sl * SLAB, &mdO, &bars[KD_OFULL + s2], sl * 64, i0, (int)bh);
-                ++k;
-            }
-            // a key tile without a single query tile (an empty block column): nobody else waits for K_j and V_j, and
-            // the CTA must not exit with their bulk loads still in flight into its shared memory
-            if (k == 0) mbar_wait(&bars[KD_KV], 0, ab);
+            more = __shfl_sync(0xffffffffu, (int)more, 0) != 0;
+            bx = __shfl_sync(0xffffffffu, bx, 0);
+            by = __shfl_sync(0xffffffffu, by, 0);
         }
     } else if (warp == 16) {
         // ------------------------------------------------------------ MMA issuer A: the products into region A
@@ -206,34 +253,31 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
             constexpr uint32_t idesc_s = idesc_bf16(128, 128, 0, 0);       // S^T, dP^T
             const uint32_t kK = desc_lo_kmajor(smem_u32(smem + L::oK)), kV = desc_lo_kmajor(smem_u32(smem + L::oV));
             constexpr uint32_t kSlab = SLAB >> 4;
-            auto issue_S = [&](int k) {
-                const uint32_t kQ = desc_lo_kmajor(smem_u32(smem + L::oQ + (k % 3) * L::kTile));
+            int k = 0, nkv = 0;
+            for (int t = 0; work(t); ++t) {
+                const int end = k + slots[t & 1].count;
+                mbar_arrive(&bars[KD_WE + (t & 1)]);
+                if (k == end) continue;
+                mbar_wait(&bars[KD_KV], nkv & 1, ab);
+                ++nkv;
+                for (; k < end; ++k) {
+                    // S^T(k) as soon as dP^T(k-1) has been copied out
+                    mbar_wait(&bars[KD_QFULL + k % 3], (k / 3) & 1, ab);
+                    mbar_wait(&bars[KD_DPLD], (k - 1) & 1, ab);
+                    tcgen05_fence_after();
+                    const uint32_t kQ = desc_lo_kmajor(smem_u32(smem + L::oQ + (k % 3) * L::kTile));
 #pragma unroll
-                for (int kk = 0; kk < HD / 16; ++kk) {
-                    const uint32_t off = (kk / 4) * kSlab + (kk % 4) * 2;
-                    mma_ss_lo(T_A, kK + off, kQ + off, idesc_s, kk > 0);
-                }
-                mma_commit(&bars[KD_S]);
-            };
-            int idx = 0, it = -1;
-            while (idx < iter.raw && (it = iter.tile(idx)) < 0) ++idx;
-            if (it >= 0) {
-                mbar_wait(&bars[KD_KV], 0, ab);
-                mbar_wait(&bars[KD_QFULL], 0, ab);
-                tcgen05_fence_after();
-                issue_S(0);
-            }
-            int k = 0;
-            while (idx < iter.raw) {
-                int nidx = idx + 1, nit = -1;
-                while (nidx < iter.raw && (nit = iter.tile(nidx)) < 0) ++nidx;
-                // dP^T(k) into region A: S^T(k) copied out, dO(k) landed, and -- because the exp / dS warps store
-                // dS^T(k) as soon as they have seen dP^T(k) -- the dK product of tile k-1 done with dS^T(k-1)
-                mbar_wait(&bars[KD_OFULL + (k & 1)], (k >> 1) & 1, ab);
-                if (k > 0) mbar_wait(&bars[KD_QEMPTY + (k - 1) % 3], ((k - 1) / 3) & 1, ab);
-                mbar_wait(&bars[KD_SLD], k & 1, ab);
-                tcgen05_fence_after();
-                {
+                    for (int kk = 0; kk < HD / 16; ++kk) {
+                        const uint32_t off = (kk / 4) * kSlab + (kk % 4) * 2;
+                        mma_ss_lo(T_A, kK + off, kQ + off, idesc_s, kk > 0);
+                    }
+                    mma_commit(&bars[KD_S]);
+                    // dP^T(k) into region A: S^T(k) copied out, dO(k) landed, and -- because the exp / dS warps store
+                    // dS^T(k) as soon as they have seen dP^T(k) -- the dK product of tile k-1 done with dS^T(k-1)
+                    mbar_wait(&bars[KD_OFULL + (k & 1)], (k >> 1) & 1, ab);
+                    if (k > 0) mbar_wait(&bars[KD_QEMPTY + (k - 1) % 3], ((k - 1) / 3) & 1, ab);
+                    mbar_wait(&bars[KD_SLD], k & 1, ab);
+                    tcgen05_fence_after();
                     const uint32_t kdO = desc_lo_kmajor(smem_u32(smem + L::odO + (k & 1) * L::kTile));
 #pragma unroll
                     for (int kk = 0; kk < HD / 16; ++kk) {
@@ -242,14 +286,7 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                     }
                     mma_commit(&bars[KD_DP]);
                 }
-                if (nit >= 0) {   // S^T(k+1) as soon as dP^T(k) has been copied out
-                    mbar_wait(&bars[KD_QFULL + (k + 1) % 3], ((k + 1) / 3) & 1, ab);
-                    mbar_wait(&bars[KD_DPLD], k & 1, ab);
-                    tcgen05_fence_after();
-                    issue_S(k + 1);
-                }
-                ++k;
-                idx = nidx;
+                mma_commit(&bars[KD_KVE]);
             }
         }
     } else if (warp == 18) {
@@ -258,18 +295,24 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
             constexpr uint32_t idesc_dv = idesc_bf16(128, HD, 0, 1);       // A in tensor memory, B MN-major
             constexpr uint32_t kHalf = HALF_ROWS >> 4;
             int k = 0;
-            for (int idx = 0; idx < iter.raw; ++idx) {
-                if (iter.tile(idx) < 0) continue;
+            for (int t = 0; work(t); ++t) {
+              const int begin = k, end = k + slots[t & 1].count;
+              mbar_arrive(&bars[KD_WE + (t & 1)]);
+              if (k == end) continue;
+              // the first dV of a unit overwrites the accumulator of the unit before: both halves' warps have read it
+              mbar_wait(&bars[KD_P + 1], k & 1, ab);
+              for (; k < end; ++k) {
                 const uint32_t mdO_ = desc_lo_mnmajor(smem_u32(smem + L::odO + (k & 1) * L::kTile), SLAB);
                 const uint32_t mQ_ = desc_lo_mnmajor(smem_u32(smem + L::oQ + (k % 3) * L::kTile), SLAB);
-                mbar_wait(&bars[KD_OFULL + (k & 1)], (k >> 1) & 1, ab);
+                // P^T of one term is handed over by warps that have seen dP^T(k), so dO(k) is there; dS^T(k) follows both loads
+                if constexpr (SPLIT) mbar_wait(&bars[KD_OFULL + (k & 1)], (k >> 1) & 1, ab);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     mbar_wait(&bars[KD_P + h], k & 1, ab);
                     tcgen05_fence_after();
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk)
-                        mma_ts_lo(T_dV, T_B + 64 * h + kk * 8, mdO_ + h * kHalf + kk * 128, idesc_dv, (k > 0) || (h > 0) || (kk > 0));
+                        mma_ts_lo(T_dV, T_B + 64 * h + kk * 8, mdO_ + h * kHalf + kk * 128, idesc_dv, (k > begin) || (h > 0) || (kk > 0));
                     if constexpr (SPLIT) {
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk)
@@ -277,14 +320,13 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                     }
                 }
                 mma_commit(&bars[KD_OEMPTY + (k & 1)]);
-                mbar_wait(&bars[KD_QFULL + k % 3], (k / 3) & 1, ab);
                 mbar_wait(&bars[KD_DS], k & 1, ab);
                 tcgen05_fence_after();
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk)
-                        mma_ts_lo(T_dK, T_dS + 64 * h + kk * 8, mQ_ + h * kHalf + kk * 128, idesc_dv, (k > 0) || (h > 0) || (kk > 0));
+                        mma_ts_lo(T_dK, T_dS + 64 * h + kk * 8, mQ_ + h * kHalf + kk * 128, idesc_dv, (k > begin) || (h > 0) || (kk > 0));
                     if constexpr (SPLIT) {
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk)
@@ -292,27 +334,32 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                     }
                 }
                 mma_commit(&bars[KD_QEMPTY + k % 3]);
-                ++k;
+              }
+              mma_commit(&bars[KD_DONE]);
             }
-            mma_commit(&bars[KD_DONE]);
         }
     } else if (warp < 16) {
         // ------------------------------------------------------------ warpgroup 2h + qq owns queries 64 h + 32 qq .. + 31
         const int h = warp / 8, qq = (warp / 4) & 1;
         const int row = (warp % 4) * 32 + lane;        // tensor-memory lane = key row inside the tile
         const uint32_t lane_addr = (uint32_t)((warp % 4) * 32) << 16;
-        const int jg = j0 + row;
         const float sl2 = a.scale * 1.4426950408889634f;
+        const bool wide = (((uintptr_t)a.dK | (uintptr_t)a.dV) & 31) == 0;
         const uint32_t c0 = h * 64 + qq * 32;          // this thread's first column of S^T / dP^T in region A
         const uint32_t cP = h * 64 + qq * 16;          // of its bf16 pairs of P^T in region B; dS^T 32 columns further
-        int k = 0;
-        for (int idx = 0; idx < iter.raw; ++idx) {
-            const int it = iter.tile(idx);
-            if (it < 0) continue;
+        int k = 0, done = 0;
+        for (int t = 0; work(t); ++t) {
+          const int jt = slots[t & 1].jt, bh = slots[t & 1].bh, count = slots[t & 1].count, begin = k - slots[t & 1].first, end = k + count;
+          const int *rows = slots[t & 1].rows;
+          int it0 = slots[t & 1].first;
+          warp_arrive(&bars[KD_WE + (t & 1)], lane);
+          const int j0 = jt * TK, jg = j0 + row;
+          for (; k < end; ++k) {
+            const int it = !lists ? it0++ : query_tile(rows, k - begin);
             const int s2 = k & 1, i0 = it * TQ;
             const float4 *sNL = reinterpret_cast<const float4 *>(smem + L::oLSE + s2 * 512 + h * 256 + qq * 128);
             const float4 *sDs = reinterpret_cast<const float4 *>(smem + L::oD + s2 * 512 + h * 256 + qq * 128);
-            const bool diag = mask_is_causal(a.mask_kind) && it == jt;
+            const bool diag = causal && it == jt;
             const int ig0 = i0 + h * 64 + qq * 32;
             // a mask finer than the tile: the keep bits of this thread's key row and its 32 query columns
             uint32_t kw = 0xffffffffu;
@@ -428,6 +475,12 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                         ppack[q * 2 + 1] = pack_bf16(p[2], p[3]);
                     }
                 }
+                // P^T(k) over P^T(k-1): the dV product of the previous tile must have consumed it.  Stored ahead of the wait for dP^T
+                if (k > 0) {
+                    mbar_wait(&bars[KD_OEMPTY + ((k - 1) & 1)], ((k - 1) >> 1) & 1, ab);
+                    tcgen05_fence_after();
+                }
+                tmem_st16(T_B + lane_addr + cP, ppack);
                 mbar_wait(&bars[KD_DP], k & 1, ab);
                 tcgen05_fence_after();
                 uint32_t dv[32];
@@ -435,12 +488,6 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                 tmem_wait_ld();
                 tcgen05_fence_before();
                 warp_arrive(&bars[KD_DPLD], lane);   // region A may take the next S^T
-                // P^T(k) over P^T(k-1): the dV product of the previous tile must have consumed it
-                if (k > 0) {
-                    mbar_wait(&bars[KD_OEMPTY + ((k - 1) & 1)], ((k - 1) >> 1) & 1, ab);
-                    tcgen05_fence_after();
-                }
-                tmem_st16(T_B + lane_addr + cP, ppack);
                 tmem_wait_st();
                 tcgen05_fence_before();
                 warp_arrive(&bars[KD_P + h], lane);
@@ -469,39 +516,32 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
             tcgen05_fence_before();
             warp_arrive(&bars[KD_DS], lane);
             warp_arrive(&bars[KD_LEMPTY + s2], lane);
-            ++k;
-        }
-        // ------------------------------------------------------------ epilogue: dV_j, dK_j (32 columns per warpgroup)
-        if (k > 0) {
-            mbar_wait(&bars[KD_DONE], 0, ab);
-            tcgen05_fence_after();
-        }
-        {
-            const int cq = (warp / 4) * 32;       // d = 64: the upper two warpgroups have no columns
-            const int jc = jg < n ? jg : 0;
-            if (cq < HD) {
+          }
+          // ---------------------------------------------------------- epilogue: dV_j, dK_j (32 columns per warpgroup)
+          if (count > 0) {
+              mbar_wait(&bars[KD_DONE], done & 1, ab);
+              ++done;
+              tcgen05_fence_after();
+          }
+          const int cq = (warp / 4) * 32;       // d = 64: the upper two warpgroups have no columns
+          if (cq < HD) {
+              const int jc = jg < n ? jg : 0;
 #pragma unroll
-                for (int which = 0; which < 2; ++which) {
-                    __nv_bfloat16 *po = (which == 0 ? a.dV : a.dK) + ((size_t)bh * n + jc) * HD + cq;
-                    uint32_t v[32];
-                    if (k > 0) {
-                        tmem_ld32((which == 0 ? T_dV : T_dK) + lane_addr + cq, v);
-                        tmem_wait_ld();
-                    } else {
+              for (int which = 0; which < 2; ++which) {
+                  __nv_bfloat16 *po = (which == 0 ? a.dV : a.dK) + ((size_t)bh * n + jc) * HD + cq;
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) v[e] = 0u;
-                    }
-                    if (jg < n) {
+                  for (int e0 = 0; e0 < 32; e0 += 16) {
+                      uint32_t v[16], y[8];
+                      tmem_ld16((which == 0 ? T_dV : T_dK) + lane_addr + cq + e0, v);
+                      tmem_wait_ld();
 #pragma unroll
-                        for (int e = 0; e < 32; e += 8)
-                            *reinterpret_cast<uint4 *>(po + e) =
-                                make_uint4(pack_bf16(__uint_as_float(v[e]), __uint_as_float(v[e + 1])),
-                                           pack_bf16(__uint_as_float(v[e + 2]), __uint_as_float(v[e + 3])),
-                                           pack_bf16(__uint_as_float(v[e + 4]), __uint_as_float(v[e + 5])),
-                                           pack_bf16(__uint_as_float(v[e + 6]), __uint_as_float(v[e + 7])));
-                    }
-                }
-            }
+                      for (int u = 0; u < 8; ++u)   // without a query tile nothing has been accumulated
+                          y[u] = count > 0 ? pack_bf16(__uint_as_float(v[2 * u]), __uint_as_float(v[2 * u + 1])) : 0u;
+                      if (jg < n) store32(po + e0, y, wide);
+                  }
+              }
+              tcgen05_fence_before();
+          }
         }
     }
     tcgen05_fence_before();
@@ -566,8 +606,8 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constan
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L::oBar);
     uint32_t *tmem_base_s = reinterpret_cast<uint32_t *>(smem + L::oMisc);
     volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(smem + L::oMisc + 4);
-    volatile FusedWork *slots = reinterpret_cast<volatile FusedWork *>(smem + L::oWork);
-    uint8_t *answer = smem + L::oWork + 2 * sizeof(FusedWork);
+    volatile KeyWork *slots = reinterpret_cast<volatile KeyWork *>(smem + L::oWork);
+    uint8_t *answer = smem + L::oWork + 2 * sizeof(KeyWork);
     const Abort ab{abort_flag, a.status};
 
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
@@ -632,32 +672,12 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constan
             bool more = true;
             for (int t = 0; more; ++t) {
                 const int jt = bx / a.group, bh = by * a.group + bx % a.group, j0 = jt * TK;
-                int count, first = 0;
+                int count, first;
                 const int *rows = nullptr;
-                if (lists) {
-                    // the lists ascend: what lies beyond n is at their end, and (block mask AND causal) what ends before the key
-                    // tile begins at their start
-                    const int J = jt / (a.block / TK);
-                    const long mh = a.mask_heads == 1 ? 0 : bh;
-                    const int *cp = a.col_ptr + mh * 2 * a.nb + 2 * J;
-                    const int start = cp[0], raw = (cp[1] - start) * sub;
-                    rows = a.row_idx + mh * (long)a.nb * a.nb + start;
-                    int before = 0, within = 0;
-                    for (int e = lane; e < raw; e += 32) {
-                        const int it = rows[e / sub] * sub + e % sub;
-                        before += causal && it < jt;
-                        within += it * TQ < n;
-                    }
-                    first = __reduce_add_sync(0xffffffffu, before);
-                    count = __reduce_add_sync(0xffffffffu, within) - first;
-                    if (count < 0) count = 0;
-                } else {
-                    first = causal ? jt : 0;
-                    count = (n + TQ - 1) / TQ - first;
-                }
+                query_range(a, jt, bh, lane, rows, first, count);
                 if (lane == 0) {
                     if (t >= 2) mbar_wait(&bars[V2_WE + (t & 1)], ((t >> 1) - 1) & 1, ab);
-                    volatile FusedWork &to = slots[t & 1];
+                    volatile KeyWork &to = slots[t & 1];
                     int it = count > 0 ? query_tile(rows, first) : 0;
                     to.jt = jt; to.bh = bh; to.count = count; to.first = first; to.rows = rows;
                     mbar_arrive(&bars[V2_WF + (t & 1)]);
