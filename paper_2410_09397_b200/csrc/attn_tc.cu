@@ -38,8 +38,8 @@ size_t tc_cfg_onchip_bytes(int d, const attn_cfg &c, int backward)
         return bwd64_smem_bytes(d) + (size_t)(256 + 128 + (d == 256 ? 128 : 0)) * 128 * 4;
     // regions A and B, dK_j and dV_j; d = 64: a second region for dP^T in the columns that would otherwise stay free
     if (backward) return bwd_smem_bytes(d) + (size_t)(256 + 2 * d + (d == 64 ? 128 : 0)) * 128 * 4;
-    // two S buffers, and two partial accumulators of O or (d = 256) one
-    return fwd_smem_bytes(d) + (size_t)(256 + (d == 256 ? d : 2 * d)) * 128 * 4;
+    // all of tensor memory: S (d = 64: two buffers), P and O of each warpgroup; d = 256: two S buffers and one O
+    return fwd_smem_bytes(d) + (size_t)512 * 128 * 4;
 }
 
 }  // namespace attn
