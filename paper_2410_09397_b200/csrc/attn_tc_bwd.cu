@@ -655,7 +655,8 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constan
     // both issuers, the exp / dS warps and the reducers have arrived on WE
     auto work = [&](int t) { return mbar_wait(&bars[V2_WF + (t & 1)], (t >> 1) & 1, ab) && slots[t & 1].jt >= 0; };
     auto query_tile = [&](const int *rows, int e) { return !lists ? e : sub == 1 ? rows[e] : rows[e / sub] * sub + e % sub; };
-    // query tile of the kt-th load; the fourth load after it needs dP^T of tile kt + 2, and so dQ^T(kt) read by the reducers
+    // query tile of the kt-th load, for the exp / dS warps; the fourth load after it follows dK(kt + 1) at the latest, by when they
+    // are past it
     volatile int *tiles = reinterpret_cast<volatile int *>(smem + L::oTile);
 
     // In every role kt counts the query tiles of all units of work so far (a wait for what belongs to tile -1 returns at once: a

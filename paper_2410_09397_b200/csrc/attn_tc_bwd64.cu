@@ -24,6 +24,10 @@
 // Roles: warps 0-7 exp / dS (lane quarter = warp % 4, 32 query columns each), warps 8-11 reducers
 // (dQ^T tile -> registers -> fp32 accumulator), warp 12 lane 0 issues S^T and dP^T, warp 14 lane 0 dV, dQ^T and dK, warp 13
 // lane 0 every TMA load.  All waits are bounded (tc_common.cuh).
+//
+// Bound by the chain through RD: dP^T copied out -> dS -> dQ^T -> read by the reducers -> next dP^T, each link a barrier and a
+// product.  With one issuing thread S^T of the next tile (768 cycles) went ahead of dK and dQ^T, and dK ahead of dQ^T.  8 heads,
+// n = 4096, d = 256: 592 -> 570 us; n = 8192, causal: 1041 -> 998.
 #include "tc_bwd_common.cuh"
 
 namespace attn {
