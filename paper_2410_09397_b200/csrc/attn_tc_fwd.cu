@@ -70,7 +70,11 @@ struct FwdCfg {                                                // d = 256
     static constexpr uint32_t kBytes = kUsed < 117 * 1024 ? 117 * 1024 : kUsed;
 };
 
-enum { FB_Q = 0, FB_KVFULL = 1, FB_KVEMPTY = 4, FB_S = 7, FB_P = 9, FB_O = 11, FB_OLAST = 12 };
+// FB_KVEMPTY: O += P V of the tile that this stage held has completed; the loading thread takes it as the release of the stage, a
+// softmax thread as the news that O holds the product.  When it asks, the completion before is known from S of its own tile, whose
+// K came after that one, and the next one needs its P.  A barrier that completes with every tile's product could be two
+// completions behind: of the product of tile k - 2 nothing but the release of its stage is known from S(k).
+enum { FB_Q = 0, FB_KVFULL = 1, FB_KVEMPTY = 3, FB_S = 5, FB_P = 7 };
 
 template <int TKF>
 struct KeyIter {
@@ -192,8 +196,6 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CU
         mbar_init(&bars[FB_Q], 1);
         for (int s = 0; s < NST; ++s) { mbar_init(&bars[FB_KVFULL + s], 1); mbar_init(&bars[FB_KVEMPTY + s], 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(&bars[FB_S + b], 1); mbar_init(&bars[FB_P + b], kSoftmaxThreads / 32); }
-        mbar_init(&bars[FB_O], 1);
-        mbar_init(&bars[FB_OLAST], 1);
         fence_barrier_init();
         prefetch_tensormap(&mQ); prefetch_tensormap(&mK); prefetch_tensormap(&mV);
     }
@@ -269,8 +271,6 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CU
                 for (int kk = 0; kk < TKF / 16; ++kk)
                     mma_ts_lo(T_O, tm + b * 128 + kk * 8, mV_ + kk * 128, idesc_o, (k > 0) || (kk > 0));
                 mma_commit(&bars[FB_KVEMPTY + s]);
-                mma_commit(&bars[FB_O]);
-                if (k + 1 == niter) mma_commit(&bars[FB_OLAST]);
             }
         }
     } else {
@@ -325,7 +325,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CU
                 const float m_new = need ? fmaxf(m_ref, m_tile) : m_ref;
                 const float alpha = (need && m_ref != -INFINITY) ? ex2_fast_f(m_ref - m_new) : 1.f;
                 if (k > 0) {
-                    mbar_wait(&bars[FB_O], (k - 1) & 1, ab);   // O += P V of the previous tile has landed
+                    mbar_wait(&bars[FB_KVEMPTY + (k - 1) % NST], ((k - 1) / NST) & 1, ab);   // O += P V of the previous tile has landed
                     tcgen05_fence_after();
 #pragma unroll
                     for (int c = 0; c < HD / 2; c += 32) {
@@ -364,10 +364,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CU
         named_bar_sync_f(1, kSoftmaxThreads);
         const float l_tot = xsum[row] + xsum[128 + row];
         if (k > 0) {
-            // FB_O completes once per tile and a parity wait tells two phases apart, not three: the last completion
-            // this thread knows of is S(k-1), queued before O += P V of tile k-2, so FB_O may be two completions
-            // behind the one needed here and a wait on it could pass at once.  The last product has a barrier of its own.
-            mbar_wait(&bars[FB_OLAST], 0, ab);
+            mbar_wait(&bars[FB_KVEMPTY + (k - 1) % NST], ((k - 1) / NST) & 1, ab);   // the last product
             tcgen05_fence_after();
         }
         const float inv = l_tot > 0.f ? 1.f / l_tot : 0.f;
