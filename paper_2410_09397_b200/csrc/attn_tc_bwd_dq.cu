@@ -67,7 +67,7 @@ enum { DB_Q = 0, DB_KFULL = 1, DB_KEMPTY = 4, DB_VFULL = 7, DB_VEMPTY = 9, DB_S 
 
 // One unit of work: a query tile of one head and the key tiles that it visits
 struct DqWork {
-    int it, bh, count;   // it = -1: there is no more work
+    int tile, bh, count; // tile = -1: there is no more work
     int pad;
     const int *cols;     // key blocks of a mask with lists
     int pad2[2];
@@ -98,7 +98,6 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
     const Abort ab{abort_flag, a.status};
 
     volatile DqWork *slots = reinterpret_cast<volatile DqWork *>(smem + L::oWork);
-    uint8_t *answer = smem + L::oWork + 2 * sizeof(DqWork);
     constexpr int kWarps = kSoftmaxThreads / 32;
 
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
@@ -127,8 +126,8 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
     const uint32_t tm = *tmem_base_s;
     const uint32_t T_dP = tm + 256, T_dQ = tm + 384;
 
-    // the t-th unit of work of this CTA as the loading warp has published it (false: there is none)
-    auto work = [&](int t) { return mbar_wait(&bars[DB_WF + (t & 1)], (t >> 1) & 1, ab) && slots[t & 1].it >= 0; };
+    // the units of work of this CTA as the loading warp publishes them
+    const UnitQueue<DqWork, UnitIo> units{slots, &bars[DB_WF], &bars[DB_WE], &bars[DB_CLC], smem + L::oWork + 2 * sizeof(DqWork), {ab}};
     auto key_tile = [&](const int *cols, int e) { return !lists ? e : sub == 1 ? cols[e] : cols[e / sub] * sub + e % sub; };
 
     // In every role k counts the key tiles of all units of work so far (a wait for what belongs to a tile before the first returns
@@ -156,13 +155,13 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
             } else {
                 count = causal ? last_i / TKD + 1 : (n + TKD - 1) / TKD;
             }
-            if (lane == 0) {
-                if (t >= 2) mbar_wait(&bars[DB_WE + (t & 1)], ((t >> 1) - 1) & 1, ab);
-                volatile DqWork &to = slots[t & 1];
-                to.it = it; to.bh = bh; to.count = count; to.cols = cols;
-                mbar_arrive(&bars[DB_WF + (t & 1)]);
+            auto load_unit = [&]() -> bool {   // false: there is no further unit, or the kernel is giving up
+                volatile DqWork *to = units.claim(t);
+                if (!to) return false;
+                to->tile = it; to->bh = bh; to->count = count; to->cols = cols;
+                units.publish(t);
                 if (count > 0) {
-                    mbar_wait(&bars[DB_QEMPTY], (nq - 1) & 1, ab);   // dP of the unit before
+                    if (!mbar_wait(&bars[DB_QEMPTY], (nq - 1) & 1, ab)) return false;   // dP of the unit before
                     ++nq;
                     mbar_expect_tx(&bars[DB_Q], 2 * L::kTile);
 #pragma unroll
@@ -171,30 +170,25 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
                         tma_load_3d(smem + L::odO + sl * SLAB, &mdO, &bars[DB_Q], sl * 64, i0, bh);
                     }
                 } else {
-                    clc_request(answer, &bars[DB_CLC]);
+                    units.ask();
                 }
                 for (int e = 0; e < count; ++e, ++k) {
                     const int jt = key_tile(cols, e), sk = k % NSTK, sv = k % NSTV;
-                    // the next unit of work, asked for early enough that the answer is there when the loads get to it
-                    if (e == max(count - 2, 0)) clc_request(answer, &bars[DB_CLC]);
-                    if (k >= NSTK) mbar_wait(&bars[DB_KEMPTY + sk], ((k / NSTK) - 1) & 1, ab);
+                    if (e == max(count - 2, 0)) units.ask();
+                    if (k >= NSTK && !mbar_wait(&bars[DB_KEMPTY + sk], ((k / NSTK) - 1) & 1, ab)) return false;
                     mbar_expect_tx(&bars[DB_KFULL + sk], L::kTile);
 #pragma unroll
                     for (uint32_t sl = 0; sl < L::kSlabs; ++sl)
                         tma_load_3d(smem + L::oK + sk * L::kTile + sl * SLAB, &mK, &bars[DB_KFULL + sk], sl * 64, jt * TKD, bh);
-                    if (k >= NSTV) mbar_wait(&bars[DB_VEMPTY + sv], ((k / NSTV) - 1) & 1, ab);
+                    if (k >= NSTV && !mbar_wait(&bars[DB_VEMPTY + sv], ((k / NSTV) - 1) & 1, ab)) return false;
                     mbar_expect_tx(&bars[DB_VFULL + sv], L::kTile);
 #pragma unroll
                     for (uint32_t sl = 0; sl < L::kSlabs; ++sl)
                         tma_load_3d(smem + L::oV + sv * L::kTile + sl * SLAB, &mV, &bars[DB_VFULL + sv], sl * 64, jt * TKD, bh);
                 }
-                more = mbar_wait(&bars[DB_CLC], t & 1, ab) && clc_answer(answer, bx, by);
-                if (!more) {
-                    if (t >= 1) mbar_wait(&bars[DB_WE + ((t + 1) & 1)], (((t + 1) >> 1) - 1) & 1, ab);
-                    slots[(t + 1) & 1].it = -1;
-                    mbar_arrive(&bars[DB_WF + ((t + 1) & 1)]);
-                }
-            }
+                return units.next(t, bx, by);
+            };
+            if (lane == 0) more = load_unit();
             more = __shfl_sync(0xffffffffu, (int)more, 0) != 0;
             bx = __shfl_sync(0xffffffffu, bx, 0);
             by = __shfl_sync(0xffffffffu, by, 0);
@@ -208,11 +202,11 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
             constexpr uint32_t kSlab = SLAB >> 4;
             const uint32_t kQ = desc_lo_kmajor(smem_u32(smem + L::oQ)), kdO = desc_lo_kmajor(smem_u32(smem + L::odO));
             int k = 0, nq = 0;
-            for (int t = 0; work(t); ++t) {
+            for (int t = 0; units.take_alone(t); ++t) {
                 const int end = k + slots[t & 1].count;
                 mbar_arrive(&bars[DB_WE + (t & 1)]);
                 if (k == end) continue;
-                mbar_wait(&bars[DB_Q], nq & 1, ab);
+                if (!mbar_wait(&bars[DB_Q], nq & 1, ab)) break;
                 ++nq;
                 for (; k < end; ++k) {
                     const int s = k % NSTK;
@@ -229,7 +223,7 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
                     mma_commit(&bars[DB_S + (k & 1)]);
                     // dP(k) once every thread has read dP(k-1) out of tensor memory
                     mbar_wait(&bars[DB_DPFREE], (k - 1) & 1, ab);
-                    mbar_wait(&bars[DB_VFULL + k % NSTV], (k / NSTV) & 1, ab);
+                    if (!mbar_wait(&bars[DB_VFULL + k % NSTV], (k / NSTV) & 1, ab)) break;
                     tcgen05_fence_after();
                     const uint32_t kV = desc_lo_kmajor(smem_u32(smem + L::oV + (k % NSTV) * L::kTile));
 #pragma unroll
@@ -248,12 +242,12 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
         if (lane == 0) {
             constexpr uint32_t idesc_dq = idesc_bf16(128, HD, 0, 1);
             int k = 0;
-            for (int t = 0; work(t); ++t) {
+            for (int t = 0; units.take_alone(t); ++t) {
                 const int begin = k, end = k + slots[t & 1].count;
                 mbar_arrive(&bars[DB_WE + (t & 1)]);
                 for (; k < end; ++k) {
                     const int s = k % NSTK, b = k & 1;
-                    mbar_wait(&bars[DB_KFULL + s], (k / NSTK) & 1, ab);
+                    if (!mbar_wait(&bars[DB_KFULL + s], (k / NSTK) & 1, ab)) break;
                     mbar_wait(&bars[DB_DS + b], (k >> 1) & 1, ab);   // of every warp: the first of a unit has been preceded by their reading dQ
                     tcgen05_fence_after();
                     const uint32_t mK_ = desc_lo_mnmajor(smem_u32(smem + L::oK + s * L::kTile), SLAB);
@@ -276,8 +270,8 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
         const float sl2 = a.scale * 1.4426950408889634f;
         const bool wide = ((uintptr_t)a.dQ & 31) == 0;
         int k = 0, nq = 0;
-        for (int t = 0; work(t); ++t) {
-            const int i0 = slots[t & 1].it * TQ, bh = slots[t & 1].bh, count = slots[t & 1].count, begin = k;
+        for (int t = 0; units.take(t); ++t) {
+            const int i0 = slots[t & 1].tile * TQ, bh = slots[t & 1].bh, count = slots[t & 1].count, begin = k;
             const int *cols = slots[t & 1].cols;
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars[DB_WE + (t & 1)]);

@@ -1030,7 +1030,7 @@ enum { F4_QF = 0, F4_QE = 2, F4_KF = 4, F4_KE = 7, F4_VF = 10, F4_VE = 13, F4_S 
 
 // One unit of work: a query tile (or two) of one head
 struct FlowWork {
-    int i0, bh;        // first query; -1: there is no more work
+    int tile, bh;      // query tile (or two) of that many rows; -1: there is no more work
     int n0, n1;        // items of the warpgroups
     const int *cols;   // key blocks of a mask with lists
     int pad[2];
@@ -1127,12 +1127,11 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
         __device__ bool begins(int i) const { return !PAIR || i >= 2 * both || (i & 1) == 0; }  // the first item of its key tile
         __device__ bool ends(int i) const { return !PAIR || i >= 2 * both || (i & 1) != 0; }    // the last one
     };
-    // the t-th unit of work of this CTA as the loading warp has published it (false: there is none)
-    auto work = [&](int t, FlowWork &f) {
-        if (!mbar_wait(&bars[F4_WF + (t & 1)], (t >> 1) & 1, ab)) return false;
+    // the t-th unit of work of this CTA as the loading warp has published it
+    const UnitQueue<FlowWork, UnitIo> units{slots, &bars[F4_WF], &bars[F4_WE], &bars[F4_CLC], smem + C::oWork + 2 * sizeof(FlowWork), {ab}};
+    auto unit = [&](int t) {
         const volatile FlowWork &v = slots[t & 1];
-        f.i0 = v.i0; f.bh = v.bh; f.n0 = v.n0; f.n1 = v.n1; f.cols = v.cols;
-        return f.i0 >= 0;
+        return FlowWork{v.tile, v.bh, v.n0, v.n1, v.cols, {}};
     };
 
     if (warp >= 8) {
@@ -1149,7 +1148,7 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
         int nq0 = 0, nq1 = 0;      // loads of each Q buffer so far
         bool more = true;
         for (int t = 0; more; ++t) {
-            const int i0 = ((n + QROWS - 1) / QROWS - 1 - bx / a.group) * QROWS;   // heaviest causal tiles first
+            const int tile = (n + QROWS - 1) / QROWS - 1 - bx / a.group, i0 = tile * QROWS;   // heaviest causal tiles first
             const int bh = by * a.group + bx % a.group;
             int n0, n1;
             const int *cols = nullptr;
@@ -1177,13 +1176,13 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                 n0 = (kept + 1) / 2, n1 = kept / 2;
             }
             const Order o(n0, n1);
-            if (lane == 0) {
-                if (t >= 2) mbar_wait(&bars[F4_WE + (t & 1)], ((t >> 1) - 1) & 1, ab);
-                volatile FlowWork &f = slots[t & 1];
-                f.i0 = i0; f.bh = bh; f.n0 = n0; f.n1 = n1; f.cols = cols;
-                mbar_arrive(&bars[F4_WF + (t & 1)]);
+            auto load_unit = [&]() -> bool {   // false: there is no further unit, or the kernel is giving up
+                volatile FlowWork *f = units.claim(t);
+                if (!f) return false;
+                f->tile = tile; f->bh = bh; f->n0 = n0; f->n1 = n1; f->cols = cols;
+                units.publish(t);
                 if (o.items > 0) {
-                    if (nq0 > 0) mbar_wait(&bars[F4_QE], (nq0 - 1) & 1, ab);
+                    if (nq0 > 0 && !mbar_wait(&bars[F4_QE], (nq0 - 1) & 1, ab)) return false;
                     load(C::oQ, &mQ, &bars[F4_QF], i0, bh);
                     ++nq0;
                 }
@@ -1192,26 +1191,21 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                     const int sk = kt % NK, sv = kt % NV;
                     const int here = jt;
                     if (k + 1 < o.tiles) jt = lists ? cols[(k + 1) / sub] * sub + (k + 1) % sub : k + 1;
-                    // the next unit of work, asked for early enough that the answer is there when the loads get to it
-                    if (k == max(o.tiles - 2, 0)) clc_request(smem + C::oWork + 2 * sizeof(FlowWork), &bars[F4_CLC]);
-                    if (kt >= NK) mbar_wait(&bars[F4_KE + sk], (kt / NK - 1) & 1, ab);
+                    if (k == max(o.tiles - 2, 0)) units.ask();
+                    if (kt >= NK && !mbar_wait(&bars[F4_KE + sk], (kt / NK - 1) & 1, ab)) return false;
                     load(C::oK + sk * C::kTile, &mK, &bars[F4_KF + sk], here * TKF, bh);
                     if (PAIR && k == 0 && n1 > 0) {
-                        if (nq1 > 0) mbar_wait(&bars[F4_QE + 1], (nq1 - 1) & 1, ab);
+                        if (nq1 > 0 && !mbar_wait(&bars[F4_QE + 1], (nq1 - 1) & 1, ab)) return false;
                         load(C::oQ + C::kTile, &mQ, &bars[F4_QF + 1], i0 + TQ, bh);
                         ++nq1;
                     }
-                    if (kt >= NV) mbar_wait(&bars[F4_VE + sv], (kt / NV - 1) & 1, ab);
+                    if (kt >= NV && !mbar_wait(&bars[F4_VE + sv], (kt / NV - 1) & 1, ab)) return false;
                     load(C::oV + sv * C::kTile, &mV, &bars[F4_VF + sv], here * TKF, bh);
                 }
-                if (o.tiles == 0) clc_request(smem + C::oWork + 2 * sizeof(FlowWork), &bars[F4_CLC]);
-                more = mbar_wait(&bars[F4_CLC], t & 1, ab) && clc_answer(smem + C::oWork + 2 * sizeof(FlowWork), bx, by);
-                if (!more) {
-                    if (t >= 1) mbar_wait(&bars[F4_WE + ((t + 1) & 1)], (((t + 1) >> 1) - 1) & 1, ab);
-                    slots[(t + 1) & 1].i0 = -1;
-                    mbar_arrive(&bars[F4_WF + ((t + 1) & 1)]);
-                }
-            }
+                if (o.tiles == 0) units.ask();
+                return units.next(t, bx, by);
+            };
+            if (lane == 0) more = load_unit();
             more = __shfl_sync(0xffffffffu, (int)more, 0) != 0;
             bx = __shfl_sync(0xffffffffu, bx, 0);
             by = __shfl_sync(0xffffffffu, by, 0);
@@ -1221,20 +1215,20 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
         if (lane == 0) {
             constexpr uint32_t idesc_s = idesc_bf16(128, TKF, 0, 0);
             const uint32_t kQ = desc_lo_kmajor(smem_u32(smem + C::oQ));
-            FlowWork f;
             int g = 0, kt0 = 0, last_w = -1;   // items and key tiles before this unit of work; warpgroup of the item before
             int nq0 = 0, nq1 = 0;
-            for (int t = 0; work(t, f); ++t) {
+            for (int t = 0; units.take_alone(t); ++t) {
+                const FlowWork f = unit(t);
                 mbar_arrive(&bars[F4_WE + (t & 1)]);
                 const Order o(f.n0, f.n1);
                 for (int i = 0; i < o.items; ++i, ++g) {
                     const int w = o.group(i), k = kt0 + o.tile(i), x = g % NX;
                     const int q = PAIR ? w : 0;
                     if (i == 0 || (PAIR && i == 1 && w == 1)) {
-                        mbar_wait(&bars[F4_QF + q], (q == 0 ? nq0 : nq1) & 1, ab);
+                        if (!mbar_wait(&bars[F4_QF + q], (q == 0 ? nq0 : nq1) & 1, ab)) break;
                         if (q == 0) ++nq0; else ++nq1;
                     }
-                    if (o.begins(i)) mbar_wait(&bars[F4_KF + k % NK], (k / NK) & 1, ab);
+                    if (o.begins(i) && !mbar_wait(&bars[F4_KF + k % NK], (k / NK) & 1, ab)) break;
                     if (g >= NX) mbar_wait(&bars[F4_XF + x], (g / NX - 1) & 1, ab);
                     // two items of one warpgroup in a row: the barrier of its S may not complete a second time before it has seen the first
                     if (NX > 1 && w == last_w) mbar_wait(&bars[F4_XF + (g - 1) % NX], ((g - 1) / NX) & 1, ab);
@@ -1258,9 +1252,9 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
         // ------------------------------------------------------------ MMA issuer B: O += P V
         if (lane == 0) {
             constexpr uint32_t idesc_o = idesc_bf16(128, HD, 0, 1);
-            FlowWork f;
             int kt0 = 0, c0 = 0, c1 = 0;   // key tiles and items of each warpgroup before this unit of work
-            for (int t = 0; work(t, f); ++t) {
+            for (int t = 0; units.take_alone(t); ++t) {
+                const FlowWork f = unit(t);
                 mbar_arrive(&bars[F4_WE + (t & 1)]);
                 const Order o(f.n0, f.n1);
                 for (int i = 0; i < o.items; ++i) {
@@ -1268,7 +1262,7 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                     const uint32_t parity = (c + (w == 0 ? c0 : c1)) & 1;
                     const uint32_t mV_ = desc_lo_mnmajor(smem_u32(smem + C::oV + (k % NV) * C::kTile), C::kSlab);
                     const uint32_t tO = tm + C::tO + w * HD, tP = tm + C::tP + w * 64;
-                    if (o.begins(i)) mbar_wait(&bars[F4_VF + k % NV], (k / NV) & 1, ab);
+                    if (o.begins(i) && !mbar_wait(&bars[F4_VF + k % NV], (k / NV) & 1, ab)) break;
                     mbar_wait(&bars[F4_PE + w], parity, ab);   // the first 96 keys, then the rest
                     tcgen05_fence_after();
 #pragma unroll
@@ -1297,12 +1291,12 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
         const float sl2 = a.scale * kLog2e;
         const uint32_t T_P = tm + C::tP + w * 64 + lane_addr, T_O = tm + C::tO + w * HD + lane_addr;
         const bool wide = ((uintptr_t)a.O & 31) == 0;
-        FlowWork f;
         int g0 = 0, c0 = 0;   // items of both warpgroups and of this one before this unit of work
-        for (int t = 0; work(t, f); ++t) {
+        for (int t = 0; units.take(t); ++t) {
+            const FlowWork f = unit(t);
             warp_arrive_f(&bars[F4_WE + (t & 1)], lane);
             const Order o(f.n0, f.n1);
-            const int iw = f.i0 + (PAIR ? w * TQ : 0), ig = iw + row, mine = w == 0 ? f.n0 : f.n1;
+            const int iw = f.tile * QROWS + (PAIR ? w * TQ : 0), ig = iw + row, mine = w == 0 ? f.n0 : f.n1;
             const long bh = f.bh;
             float m_ref = -INFINITY, l_run = 0.f;
             // key tiles of this warpgroup's next two items and the keep bits of the next one are fetched ahead

@@ -6,12 +6,16 @@
 // raises the CTA's abort flag and the global status word and returns false.  After an
 // abort all later waits of the CTA return at once, the kernel runs to its normal end
 // (its results are then meaningless, and the caller sees ATTN_ERR_DEVICE_TIMEOUT), TMEM
-// is freed and the CTA exits.
+// is freed and the CTA exits.  Nothing is in order between the roles by then: a thread that
+// loads stops at its first wait that fails, and a stage is released only by a thread that has
+// seen its load land, since a barrier must not be armed twice in one phase.
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include "tc_units.cuh"
 
 namespace attn {
 namespace tc {
@@ -83,6 +87,24 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, const 
         }
     }
     return true;
+}
+
+// For a loading thread: the stage has been released and the load before, for which `full` was armed, has landed, which a release that
+// comes early because the CTA is giving up does not tell.  (Only where the role that releases the stage does not itself wait for the
+// load.)  Both in one go: a wait of the loading thread takes long while the products stream their operands.
+__device__ __forceinline__ bool mbar_reload(uint64_t *full, uint64_t *empty, uint32_t parity, const Abort &ab)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %3;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 q, [%2], %3;\n\t"
+        "and.pred p, p, q;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(full)), "r"(smem_u32(empty)), "r"(parity)
+        : "memory");
+    return ok != 0 || (mbar_wait(full, parity, ab) && mbar_wait(empty, parity, ab));
 }
 
 // ------------------------------------------------------------------ fences
@@ -342,6 +364,16 @@ __device__ __forceinline__ bool clc_answer(const void *answer, int &bx, int &by)
     fence_proxy_async_smem();   // read before the next answer is written
     return ok != 0;
 }
+
+struct UnitIo {   // UnitQueue on the hardware
+    Abort ab;
+    __device__ __forceinline__ bool wait(uint64_t *bar, uint32_t parity) const { return mbar_wait(bar, parity, ab); }
+    __device__ __forceinline__ bool late() const { return *ab.flag != 0; }
+    __device__ __forceinline__ bool all(bool x) const { return __all_sync(0xffffffffu, x); }
+    __device__ __forceinline__ void arrive(uint64_t *bar) const { mbar_arrive(bar); }
+    __device__ __forceinline__ void request(void *answer, uint64_t *bar) const { clc_request(answer, bar); }
+    __device__ __forceinline__ bool answer(const void *from, int &bx, int &by) const { return clc_answer(from, bx, by); }
+};
 
 // 32 bytes to global memory (a whole sector); `wide`: the address is a multiple of 32, else of 16
 __device__ __forceinline__ void store32(void *to, const uint32_t (&v)[8], bool wide)
