@@ -182,7 +182,7 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
     constexpr uint32_t HALF_ROWS = 64 * 128;   // byte offset of rows 64.. inside a [128][64] slab
 
     // the units of work of this CTA as the loading warp publishes them
-    const UnitQueue<KeyWork, UnitIo> units{slots, &bars[KD_WF], &bars[KD_WE], &bars[KD_CLC], smem + L::oWork + 2 * sizeof(KeyWork), {ab}};
+    const UnitQueue<KeyWork, UnitIo<>> units{slots, &bars[KD_WF], &bars[KD_WE], &bars[KD_CLC], smem + L::oWork + 2 * sizeof(KeyWork), {ab}};
     auto query_tile = [&](const int *rows, int e) { return !lists ? e : sub == 1 ? rows[e] : rows[e / sub] * sub + e % sub; };
 
     // In every role k counts the query tiles of all units of work so far (a wait for what belongs to a tile before the first
@@ -649,7 +649,7 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constan
 
     // the units of work of this CTA as the loading warp publishes them; one stays in its slot until both issuers, the exp / dS warps
     // and the reducers have arrived on WE
-    const UnitQueue<KeyWork, UnitIo> units{slots, &bars[V2_WF], &bars[V2_WE], &bars[V2_CLC], smem + L::oWork + 2 * sizeof(KeyWork), {ab}};
+    const UnitQueue<KeyWork, UnitIo<>> units{slots, &bars[V2_WF], &bars[V2_WE], &bars[V2_CLC], smem + L::oWork + 2 * sizeof(KeyWork), {ab}};
     auto query_tile = [&](const int *rows, int e) { return !lists ? e : sub == 1 ? rows[e] : rows[e / sub] * sub + e % sub; };
     // query tile of the kt-th load, for the exp / dS warps; the fourth load after it follows dK(kt + 1) at the latest, by when they
     // are past it

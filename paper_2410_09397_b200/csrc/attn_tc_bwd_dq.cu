@@ -127,7 +127,7 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
     const uint32_t T_dP = tm + 256, T_dQ = tm + 384;
 
     // the units of work of this CTA as the loading warp publishes them
-    const UnitQueue<DqWork, UnitIo> units{slots, &bars[DB_WF], &bars[DB_WE], &bars[DB_CLC], smem + L::oWork + 2 * sizeof(DqWork), {ab}};
+    const UnitQueue<DqWork, UnitIo<>> units{slots, &bars[DB_WF], &bars[DB_WE], &bars[DB_CLC], smem + L::oWork + 2 * sizeof(DqWork), {ab}};
     auto key_tile = [&](const int *cols, int e) { return !lists ? e : sub == 1 ? cols[e] : cols[e / sub] * sub + e % sub; };
 
     // In every role k counts the key tiles of all units of work so far (a wait for what belongs to a tile before the first returns
@@ -189,6 +189,7 @@ tc_bwd_dq_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__
                 return units.next(t, bx, by);
             };
             if (lane == 0) more = load_unit();
+            __syncwarp();
             more = __shfl_sync(0xffffffffu, (int)more, 0) != 0;
             bx = __shfl_sync(0xffffffffu, bx, 0);
             by = __shfl_sync(0xffffffffu, by, 0);

@@ -1128,7 +1128,7 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
         __device__ bool ends(int i) const { return !PAIR || i >= 2 * both || (i & 1) != 0; }    // the last one
     };
     // the t-th unit of work of this CTA as the loading warp has published it
-    const UnitQueue<FlowWork, UnitIo> units{slots, &bars[F4_WF], &bars[F4_WE], &bars[F4_CLC], smem + C::oWork + 2 * sizeof(FlowWork), {ab}};
+    const UnitQueue<FlowWork, UnitIo<kSoftmaxThreads>> units{slots, &bars[F4_WF], &bars[F4_WE], &bars[F4_CLC], smem + C::oWork + 2 * sizeof(FlowWork), {ab}};
     auto unit = [&](int t) {
         const volatile FlowWork &v = slots[t & 1];
         return FlowWork{v.tile, v.bh, v.n0, v.n1, v.cols, {}};
@@ -1206,6 +1206,7 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                 return units.next(t, bx, by);
             };
             if (lane == 0) more = load_unit();
+            __syncwarp();
             more = __shfl_sync(0xffffffffu, (int)more, 0) != 0;
             bx = __shfl_sync(0xffffffffu, bx, 0);
             by = __shfl_sync(0xffffffffu, by, 0);
@@ -1292,7 +1293,9 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
         const uint32_t T_P = tm + C::tP + w * 64 + lane_addr, T_O = tm + C::tO + w * HD + lane_addr;
         const bool wide = ((uintptr_t)a.O & 31) == 0;
         int g0 = 0, c0 = 0;   // items of both warpgroups and of this one before this unit of work
-        for (int t = 0; units.take(t); ++t) {
+        // one query tile: the warpgroups meet at a named barrier for the merge, so all their warps take a unit or none does
+        bool more = PAIR ? units.take(0) : units.take_together(0);
+        for (int t = 0; more; ++t) {
             const FlowWork f = unit(t);
             warp_arrive_f(&bars[F4_WE + (t & 1)], lane);
             const Order o(f.n0, f.n1);
@@ -1419,6 +1422,7 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                     }
                     if (ig < n) a.LSE[(size_t)bh * n + ig] = row_lse(m_ref, l_run);
                 }
+                more = units.take(t + 1);
             } else {
                 // merge the two partial softmaxes
                 xm[w * 128 + row] = m_ref;
@@ -1459,7 +1463,7 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                 if (w == 0 && ig < n) a.LSE[(size_t)bh * n + ig] = row_lse(m_all, l_tot);
                 // both accumulators and the exchange buffers have been read: P of the next unit of work may be handed over
                 tcgen05_fence_before();
-                named_bar_sync_f(1, kSoftmaxThreads);
+                more = units.take_together(t + 1);
             }
         }
     }

@@ -365,11 +365,19 @@ __device__ __forceinline__ bool clc_answer(const void *answer, int &bx, int &by)
     return ok != 0;
 }
 
+template <int kGroup = 0>   // threads that take units together (named barrier 1)
 struct UnitIo {   // UnitQueue on the hardware
     Abort ab;
     __device__ __forceinline__ bool wait(uint64_t *bar, uint32_t parity) const { return mbar_wait(bar, parity, ab); }
     __device__ __forceinline__ bool late() const { return *ab.flag != 0; }
     __device__ __forceinline__ bool all(bool x) const { return __all_sync(0xffffffffu, x); }
+    __device__ __forceinline__ bool all_warps(bool x) const
+    {
+        uint32_t y;
+        asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                     : "=r"(y) : "r"((uint32_t)x), "n"(kGroup) : "memory");
+        return y != 0;
+    }
     __device__ __forceinline__ void arrive(uint64_t *bar) const { mbar_arrive(bar); }
     __device__ __forceinline__ void request(void *answer, uint64_t *bar) const { clc_request(answer, bar); }
     __device__ __forceinline__ bool answer(const void *from, int &bx, int &by) const { return clc_answer(from, bx, by); }

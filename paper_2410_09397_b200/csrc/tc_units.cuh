@@ -51,9 +51,11 @@ struct UnitQueue {
         return false;
     }
 
-    // -- the other roles: whether there is a t-th unit, for a single thread and for a whole warp
+    // -- the other roles: whether there is a t-th unit, for a single thread, a whole warp, and a group of warps that wait for one
+    // another without a limit while they work on it: either all of them take it or none (io.all_warps is such a wait itself)
     ATTN_UNITS_FN bool take_alone(int t) const { return io.wait(&full[t & 1], (t >> 1) & 1) && slots[t & 1].tile >= 0; }
     ATTN_UNITS_FN bool take(int t) const { return io.all(io.wait(&full[t & 1], (t >> 1) & 1)) && slots[t & 1].tile >= 0; }
+    ATTN_UNITS_FN bool take_together(int t) const { return io.all_warps(io.wait(&full[t & 1], (t >> 1) & 1)) && slots[t & 1].tile >= 0; }
 };
 
 }  // namespace tc
