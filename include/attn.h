@@ -290,8 +290,9 @@ int attn_timing_collect(float *ms /* host */, const char **names /* host */, int
  * one warp that waits, for at most `limit_us` microseconds (1 .. 100000), on a barrier
  * nothing arrives at; afterwards attn_workspace_status(workspace) is
  * ATTN_ERR_DEVICE_TIMEOUT and the context is as usable as before.  workspace: device,
- * at least 256 bytes; its first two words are overwritten (word 1: bit 0 / bit 1 set if
- * the first / second wait wrongly reported success). */
+ * at least 256 bytes; its first three words are overwritten (word 1: bit 0 / bit 1 set if
+ * the first / second wait wrongly reported success; word 2: microseconds for which tensor
+ * memory was held afterwards, so that loads and products in flight could land). */
 attn_status attn_selftest_wait_timeout(void *workspace, size_t workspace_bytes, unsigned limit_us,
                                        void *cuda_stream);
 

@@ -267,9 +267,7 @@ mat_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ 
         }
         if (tid == 0) tma_store_wait_all();
     }
-    tcgen05_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, kTmemCols);
+    tmem_leave(tm, kTmemCols, warp, ab);
 }
 
 // phase 3: dS = P o (scale dP - scale D), 8 elements per thread per step

@@ -539,9 +539,7 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
           }
         }
     }
-    tcgen05_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, 512);
+    tmem_leave(tm, 512, warp, ab);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1025,9 +1023,7 @@ tc_bwd_fused_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constan
             }
         }
     }
-    tcgen05_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, 512);
+    tmem_leave(tm, 512, warp, ab);
 }
 
 // fp32 accumulator -> bf16 dQ

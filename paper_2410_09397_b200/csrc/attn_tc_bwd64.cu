@@ -398,9 +398,7 @@ tc_bwd_fused64_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_const
             }
         }
     }
-    tcgen05_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, 512);
+    tmem_leave(tm, 512, warp, ab);
 }
 
 template <int HD>

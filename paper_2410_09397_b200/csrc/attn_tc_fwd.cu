@@ -394,9 +394,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CU
         }
         if (wg == 0 && ig < n) a.LSE[(size_t)bh * n + ig] = row_lse(m_ref, l_tot);
     }
-    tcgen05_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, 512);
+    tmem_leave(tm, 512, warp, ab);
 }
 
 // The work of a softmax thread on its row of 128 scores.  While one warpgroup waits for its products the other one's warps are
@@ -736,9 +734,7 @@ tc_fwd_rows_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
         }
         if (w == 0 && ig < n) a.LSE[(size_t)bh * n + ig] = row_lse(m_all, l_tot);
     }
-    tcgen05_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, 512);
+    tmem_leave(tm, 512, warp, ab);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -969,9 +965,7 @@ tc_fwd_pair_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
             if (ig < n) a.LSE[(size_t)bh * n + ig] = row_lse(m_ref, l_run);
         }
     }
-    tcgen05_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, 512);
+    tmem_leave(tm, 512, warp, ab);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1467,9 +1461,7 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
             }
         }
     }
-    tcgen05_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, 512);
+    tmem_leave(tm, 512, warp, ab);
 }
 
 // Heads that are launched together.  Under a causal mask the query tiles of a group start longest first; head after head the

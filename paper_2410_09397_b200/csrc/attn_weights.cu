@@ -133,9 +133,7 @@ wproj_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUt
                     pack_bf16(__uint_as_float(v[e + 6]), __uint_as_float(v[e + 7])));
         }
     }
-    tcgen05_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, kTmemCols);
+    tmem_leave(tm, kTmemCols, warp, ab);
 }
 
 // ===================================================================== out = A W, persistent (d = 64, 128)
@@ -315,9 +313,7 @@ wproj_persistent_kernel(const __grid_constant__ CUtensorMap mA, const __grid_con
         }
         if (tid == 0) tma_store_wait_all();
     }
-    tcgen05_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, kTmemCols);
+    tmem_leave(tm, kTmemCols, warp, ab);
 }
 
 // ===================================================================== g += A^T G (bf16 in, fp32 out)
@@ -483,9 +479,7 @@ wgrad_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUt
             ++flushes;
         }
     }
-    tcgen05_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, kTmemCols);
+    tmem_leave(tm, kTmemCols, warp, ab);
 }
 
 // ===================================================================== g += A^T G with G in fp32
@@ -674,9 +668,7 @@ wgrad_acc_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__
             ++flushes;
         }
     }
-    tcgen05_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, kTmemCols);
+    tmem_leave(tm, kTmemCols, warp, ab);
 }
 
 // ===================================================================== fp32 FMA kernels (any dtype, d % 8 == 0)

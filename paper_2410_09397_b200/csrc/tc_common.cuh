@@ -5,8 +5,8 @@
 // Waiting never blocks for ever: every wait polls for at most Abort::limit_ns (kWaitNs) nanoseconds, then
 // raises the CTA's abort flag and the global status word and returns false.  After an
 // abort all later waits of the CTA return at once, the kernel runs to its normal end
-// (its results are then meaningless, and the caller sees ATTN_ERR_DEVICE_TIMEOUT), TMEM
-// is freed and the CTA exits.  Nothing is in order between the roles by then: a thread that
+// (its results are then meaningless, and the caller sees ATTN_ERR_DEVICE_TIMEOUT), what is
+// in flight is given time to land, TMEM is freed and the CTA exits.  Nothing is in order between the roles by then: a thread that
 // loads stops at its first wait that fails, and a stage is released only by a thread that has
 // seen its load land, since a barrier must not be armed twice in one phase.
 #pragma once
@@ -168,6 +168,24 @@ __device__ __forceinline__ void tmem_alloc(uint32_t *dst_smem, uint32_t cols)
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols)
 {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
+}
+
+// The end of a kernel that holds tensor memory.  In the usual course every load and product has been waited for by now.  A CTA that
+// gives up may have some in flight, which must not land in the shared or tensor memory of its successor: it holds both for kSettleNs
+// more.  The longest queue of products and the slowest load take some ten microseconds.
+constexpr unsigned long long kSettleNs = 1000000ull;
+__device__ __forceinline__ void tmem_leave(uint32_t taddr, uint32_t cols, int warp, const Abort &ab)
+{
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+        if (__any_sync(0xffffffffu, *ab.flag != 0)) {
+            const unsigned long long t0 = globaltimer();
+            while (globaltimer() - t0 < kSettleNs) __nanosleep(1000);
+            __syncwarp();
+        }
+        tmem_dealloc(taddr, cols);
+    }
 }
 
 // 32 lanes x 32 consecutive 32-bit columns: thread t of the warp gets lane (base lane + t),

@@ -79,21 +79,30 @@ bool make_tmap_bf16_2d(CUtensorMap *out, const void *base, uint64_t cols, uint64
 }
 
 // One warp waits, under `limit_ns`, on a barrier that nothing ever arrives at: the wait runs out, the status
-// word is set and the kernel returns normally.  Exercises the bounded-wait path of the tensor-core kernels.
-__global__ void wait_timeout_selftest_kernel(uint32_t *status, unsigned long long limit_ns, uint32_t *waited_ok)
+// word is set and the kernel returns normally, after the time that it gives to what is in flight (out[1], in us).  Exercises
+// the bounded-wait path of the tensor-core kernels.
+__global__ void wait_timeout_selftest_kernel(uint32_t *status, unsigned long long limit_ns, uint32_t *out)
 {
     __shared__ uint64_t bar;
-    __shared__ uint32_t flag;
+    __shared__ uint32_t flag, taddr;
     if (threadIdx.x == 0) {
         flag = 0;
         tc::mbar_init(&bar, 1);
         tc::fence_barrier_init();
     }
+    tc::tmem_alloc(&taddr, 32);
+    tc::tcgen05_fence_before();
     __syncthreads();
+    tc::tcgen05_fence_after();
     const tc::Abort ab{&flag, status, limit_ns};
     const bool done = tc::mbar_wait(&bar, 0, ab);        // phase 0 never completes
     const bool again = tc::mbar_wait(&bar, 0, ab);       // after an abort, later waits return at once
-    if (threadIdx.x == 0) *waited_ok = (done ? 1u : 0u) | (again ? 2u : 0u);
+    const unsigned long long t0 = tc::globaltimer();
+    tc::tmem_leave(taddr, 32, 0, ab);
+    if (threadIdx.x == 0) {
+        out[0] = (done ? 1u : 0u) | (again ? 2u : 0u);
+        out[1] = (uint32_t)((tc::globaltimer() - t0) / 1000);
+    }
 }
 
 }  // namespace attn
@@ -105,7 +114,7 @@ extern "C" attn_status attn_selftest_wait_timeout(void *workspace, size_t worksp
     if (workspace_bytes < 256 || limit_us == 0 || limit_us > 100000) return ATTN_ERR_WORKSPACE;
     uint32_t *w = static_cast<uint32_t *>(workspace);
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    if (cudaMemsetAsync(w, 0, 8, s) != cudaSuccess) return ATTN_ERR_LAUNCH;
+    if (cudaMemsetAsync(w, 0, 12, s) != cudaSuccess) return ATTN_ERR_LAUNCH;
     attn::launch_begin("selftest_wait_timeout", s);
     attn::wait_timeout_selftest_kernel<<<1, 32, 0, s>>>(w, (unsigned long long)limit_us * 1000ull, w + 1);
     attn::launch_end(s);

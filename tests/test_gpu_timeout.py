@@ -30,6 +30,14 @@ def test_wait_that_runs_out_sets_the_status_and_leaves_the_context_usable():
     H.assert_within(errs, "bf16")
 
 
+def test_tensor_memory_is_held_until_what_is_in_flight_has_landed():
+    import torch
+    import paper_2410_09397_b200 as attn
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    attn.attn_selftest_wait_timeout(ws, limit_us=1000)
+    assert ws.view(torch.int32)[2].item() >= 999    # us
+
+
 def test_selftest_rejects_bad_arguments_before_any_launch():
     import torch
     import paper_2410_09397_b200 as attn
