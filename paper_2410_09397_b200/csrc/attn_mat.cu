@@ -128,13 +128,14 @@ mat_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ 
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {
             int kc = 0;   // chunks loaded so far, over all tiles
-            for (long t = blockIdx.x; t < total; t += gridDim.x) {
+            bool go = true;
+            for (long t = blockIdx.x; t < total && go; t += gridDim.x) {
                 const int head = (int)(t / ((long)tiles_n * tiles_m));
                 const int m0 = (int)(t / tiles_n % tiles_m) * TM, n0 = (int)(t % tiles_n) * BN;
                 if (skipped(m0, n0)) continue;
                 for (int kt = 0; kt < nk; ++kt, ++kc) {
                     const int s = kc % kStages;
-                    if (kc >= kStages) mbar_wait(&empty[s], ((kc / kStages) - 1) & 1, ab);
+                    if (kc >= kStages && !(go = mbar_wait(&empty[s], ((kc / kStages) - 1) & 1, ab))) break;
                     uint8_t *sA = smem + s * L::kStage, *sB = sA + L::kA;
                     mbar_expect_tx(&full[s], L::kStage);
                     if (A_MN) {
@@ -158,7 +159,8 @@ mat_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ 
         if (lane == 0) {
             constexpr uint32_t idesc = idesc_bf16(128, BN, A_MN ? 1 : 0, B_MN ? 1 : 0);
             int kc = 0, ai = 0;   // chunks consumed; accumulator sets filled
-            for (long t = blockIdx.x; t < total; t += gridDim.x) {
+            bool go = true;
+            for (long t = blockIdx.x; t < total && go; t += gridDim.x) {
                 const int m0 = (int)(t / tiles_n % tiles_m) * TM, n0 = (int)(t % tiles_n) * BN;
                 if (skipped(m0, n0)) continue;
                 const int b = ai % NBUF;
@@ -168,7 +170,7 @@ mat_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ 
                 }
                 for (int kt = 0; kt < nk; ++kt, ++kc) {
                     const int s = kc % kStages;
-                    mbar_wait(&full[s], (kc / kStages) & 1, ab);
+                    if (!(go = mbar_wait(&full[s], (kc / kStages) & 1, ab))) break;
                     tcgen05_fence_after();
                     const uint32_t sA = smem_u32(smem + s * L::kStage), sB = sA + L::kA;
                     const uint32_t db = B_MN ? desc_lo_mnmajor(sB, 8192) : desc_lo_kmajor(sB);

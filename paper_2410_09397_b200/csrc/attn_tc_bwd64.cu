@@ -132,14 +132,14 @@ tc_bwd_fused64_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_const
                 tma_load_3d(smem + (L::kVinTmem ? L::oQ : L::oV) + sl * SLAB, &mV, &bars[B_KV], sl * 64, j0, (int)bh);
             }
             // V_j was staged where the Q stages are: they are free once the exp / dS warps have moved it
-            if (L::kVinTmem && T > 0) mbar_wait(&bars[B_VDONE], 0, ab);
+            const bool staged = !L::kVinTmem || T == 0 || mbar_wait(&bars[B_VDONE], 0, ab);
             int t = 0;
-            for (int idx = 0; idx < iter.raw; ++idx) {
+            for (int idx = 0; idx < iter.raw && staged; ++idx) {
                 const int it = iter.tile(idx);
                 if (it < 0) continue;
                 const int s = t % NS, i0 = it * TQ64;
                 const uint32_t rows = min(TQ64, n - i0);
-                if (t >= NS) mbar_wait(&bars[B_QEMPTY + s], ((t / NS) - 1) & 1, ab);
+                if (t >= NS && !mbar_reload(&bars[B_QFULL + s], &bars[B_QEMPTY + s], ((t / NS) - 1) & 1, ab)) break;
                 uint64_t *bar = &bars[B_QFULL + s];
                 mbar_expect_tx(bar, 2 * L::kQTile + 2 * rows * 4);
 #pragma unroll

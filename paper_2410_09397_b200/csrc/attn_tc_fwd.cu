@@ -226,7 +226,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CU
                 const int jt = iter.tile(idx);
                 if (jt < 0) continue;
                 const int s = k % NST;
-                if (k >= NST) mbar_wait(&bars[FB_KVEMPTY + s], ((k / NST) - 1) & 1, ab);
+                if (k >= NST && !mbar_reload(&bars[FB_KVFULL + s], &bars[FB_KVEMPTY + s], ((k / NST) - 1) & 1, ab)) break;
                 uint64_t *bar = &bars[FB_KVFULL + s];
                 mbar_expect_tx(bar, 2 * C::kKTile);
 #pragma unroll
@@ -549,6 +549,7 @@ tc_fwd_rows_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
             mbar_expect_tx(&bars[F2_Q], (niter > 0 ? 2 : 1) * C::kTile);
             load(C::oQ, &mQ, &bars[F2_Q], i0);
             int k = 0;
+            bool go = true;
             for (int idx = 0; idx < iter.raw; ++idx) {
                 const int jt = iter.tile(idx);
                 if (jt < 0) continue;
@@ -557,7 +558,7 @@ tc_fwd_rows_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                 if (k == 1) mbar_expect_tx(bar_k, C::kTile);
                 if (k >= 2) {
                     // S(k-2) is the newest completion its barrier can have here (S(k) needs the loads below)
-                    mbar_wait(&bars[F2_S + (k & 1)], ((k - 2) >> 1) & 1, ab);
+                    if (!(go = mbar_wait(&bars[F2_S + (k & 1)], ((k - 2) >> 1) & 1, ab))) break;
                     bar_k = bar_v = &bars[F2_P + (k & 1)];
                     mbar_expect_tx(bar_k, 2 * C::kTile);
                 }
@@ -566,9 +567,9 @@ tc_fwd_rows_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                 ++k;
             }
             // the last two tiles have nothing to load behind them
-            for (int q = max(niter - 2, 0); q < niter; ++q) {
-                mbar_wait(&bars[F2_S + (q & 1)], (q >> 1) & 1, ab);
-                mbar_arrive(&bars[F2_P + (q & 1)]);
+            for (int q = max(niter - 2, 0); q < niter && go; ++q) {
+                go = mbar_wait(&bars[F2_S + (q & 1)], (q >> 1) & 1, ab);
+                if (go) mbar_arrive(&bars[F2_P + (q & 1)]);
             }
         }
       } else if (warp == 8) {
@@ -602,10 +603,11 @@ tc_fwd_rows_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                 const uint32_t tO = tm + 256 + b * HD, tP = tm + b * 128;
                 mbar_wait(&bars[F2_PE + b], (k >> 1) & 1, ab);   // the first 96 keys, then the rest (and K, V of tile k + 2)
                 tcgen05_fence_after();
+                bool landed = true;
 #pragma unroll
                 for (int kk = 0; kk < TKF / 16; ++kk) {
                     if (kk == 6) {
-                        mbar_wait(&bars[F2_P + b], (k >> 1) & 1, ab);
+                        landed = mbar_wait(&bars[F2_P + b], (k >> 1) & 1, ab);
                         tcgen05_fence_after();
                     }
                     mma_ts_lo(tO, tP + kk * 8, mV_ + kk * 128, idesc_o, (k > 1) || (kk > 0));
@@ -613,6 +615,7 @@ tc_fwd_rows_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                 }
                 // the products execute in issue order: S(k+2) overwrites buffer b after P(k) has been consumed, and
                 // its completion tells warpgroup b that O_b holds the product of tile k as well
+                if (!landed) break;
                 if (k + 2 < niter) issue_S(k + 2);
                 else mma_commit(&bars[F2_O + b]);   // the last product of each warpgroup, for the epilogue
             }
@@ -643,7 +646,7 @@ tc_fwd_rows_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                 for (int q = 0; q < TKF / 32; ++q)
                     kws[q] = (ig < n && j0 + q * 32 < n) ? fine_word(a.fine, a.mask_heads, bh, true, ig, j0 + q * 32) : 0u;
             }
-            mbar_wait(&bars[F2_S + w], cnt & 1, ab);
+            const bool here = mbar_wait(&bars[F2_S + w], cnt & 1, ab);
             tcgen05_fence_after();
             // the whole row of raw scores in registers: four loads in flight, one wait
             uint32_t v[TKF];
@@ -692,7 +695,7 @@ tc_fwd_rows_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
             const float noff = m_ref == -INFINITY ? 0.f : -m_ref;
             // P = exp2(S * scale * log2e - m_ref) as bf16 pairs over the first 64 columns of S (every thread
             // overwrites only its own lane, whose scores it already holds)
-            l_run += exp_row_split(v, sl2, noff, T_S + lane_addr, &bars[F2_PE + w], &bars[F2_P + w], lane);
+            l_run += exp_row_split(v, sl2, noff, T_S + lane_addr, &bars[F2_PE + w], &bars[F2_P + w], here ? lane : -1);
             ++cnt;
         }
         // ------------------------------------------------------------ epilogue: merge the two partial softmaxes
@@ -834,7 +837,8 @@ tc_fwd_pair_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
             mbar_expect_tx(&bars[F3_V0], C::kTile);
             load(C::oV, &mV, &bars[F3_V0], 0);
             for (int k = 0; k < n0; ++k) {
-                mbar_wait(&bars[F3_S], k & 1, ab);
+                // the loads before have landed (P_0(k-1), known from S_0(k) unless the CTA is giving up)
+                if (!mbar_wait(&bars[F3_P], (k - 1) & 1, ab) || !mbar_wait(&bars[F3_S], k & 1, ab)) break;
                 if (k + 1 < most) {
                     mbar_expect_tx(&bars[F3_P], 2 * C::kTile);
                     load(C::oK + (k + 1) % NK * C::kTile, &mK, &bars[F3_P], (k + 1) * TKF);
@@ -905,7 +909,7 @@ tc_fwd_pair_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
         float m_ref = -INFINITY, l_run = 0.f;
         for (int k = 0; k < mine; ++k) {
             const int j0 = k * TKF;
-            mbar_wait(&bars[F3_S + w], k & 1, ab);
+            const bool here = mbar_wait(&bars[F3_S + w], k & 1, ab);
             tcgen05_fence_after();
             uint32_t v[TKF];   // the whole row of raw scores in registers: four loads in flight, one wait
 #pragma unroll
@@ -937,7 +941,7 @@ tc_fwd_pair_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
                 m_ref = m_new;
             }
             const float noff = m_ref == -INFINITY ? 0.f : -m_ref;
-            l_run += exp_row_split(v, sl2, noff, T_S + lane_addr, &bars[F3_PE + w], &bars[F3_P + w], lane);
+            l_run += exp_row_split(v, sl2, noff, T_S + lane_addr, &bars[F3_PE + w], &bars[F3_P + w], here ? lane : -1);
         }
         // ------------------------------------------------------------ epilogue
         if (mine > 0) {

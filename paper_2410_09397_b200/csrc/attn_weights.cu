@@ -239,12 +239,12 @@ wproj_persistent_kernel(const __grid_constant__ CUtensorMap mA, const __grid_con
             for (long t = t0 + early; t < t1; ++t, ++kt) {
                 const long wi = (t / g.tiles_per_unit) % g.weight_units;
                 if (wi != wprev) {
-                    mbar_wait(wfree, (wloads - 1) & 1, ab);   // products with the old W are done
+                    if (!mbar_wait(wfree, (wloads - 1) & 1, ab)) break;   // products with the old W are done
                     load_W(wi);
                     ++wloads;
                     wprev = wi;
                 }
-                if (kt >= kStages) mbar_wait(&aempty[kt % kStages], ((kt / kStages) - 1) & 1, ab);
+                if (kt >= kStages && !mbar_wait(&aempty[kt % kStages], ((kt / kStages) - 1) & 1, ab)) break;
                 load_A(kt, t);
             }
         }
@@ -257,13 +257,13 @@ wproj_persistent_kernel(const __grid_constant__ CUtensorMap mA, const __grid_con
             for (long t = t0; t < t1; ++t, ++kt) {
                 const long wi = (t / g.tiles_per_unit) % g.weight_units;
                 if (wi != wprev) {
-                    mbar_wait(wfull, wloads & 1, ab);
+                    if (!mbar_wait(wfull, wloads & 1, ab)) break;
                     ++wloads;
                     wprev = wi;
                 }
                 const int s = kt % kStages, b = kt & 1;
                 if (kt >= 2) mbar_wait(&accempty[b], ((kt / 2) - 1) & 1, ab);
-                mbar_wait(&afull[s], (kt / kStages) & 1, ab);
+                if (!mbar_wait(&afull[s], (kt / kStages) & 1, ab)) break;
                 tcgen05_fence_after();
                 const uint32_t sA = smem_u32(smem + L::oA + s * L::kATile);
 #pragma unroll
@@ -409,7 +409,7 @@ wgrad_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUt
         if (lane == 0) {
             int kt = early;
             for (long t = t0 + early; t < t1; ++t, ++kt) {
-                mbar_wait(&empty[kt % kStages], ((kt / kStages) - 1) & 1, ab);
+                if (!mbar_wait(&empty[kt % kStages], ((kt / kStages) - 1) & 1, ab)) break;
                 load_stage(kt, t);
             }
         }
@@ -424,7 +424,7 @@ wgrad_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUt
                     mbar_wait(tfree, (flushes - 1) & 1, ab);
                     tcgen05_fence_after();
                 }
-                mbar_wait(&full[s], (kt / kStages) & 1, ab);
+                if (!mbar_wait(&full[s], (kt / kStages) & 1, ab)) break;
                 tcgen05_fence_after();
                 const uint32_t sA = smem_u32(smem + s * L::kStage), sG = sA + L::kTile;
                 const uint32_t lboA = HD == 64 ? smem_u32(smem + L::oZero) - sA : L::kSlab;
@@ -466,7 +466,7 @@ wgrad_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUt
                         uint32_t v[32];
                         tmem_ld32(tm + lane_addr + half * 256 + c, v);
                         tmem_wait_ld();
-                        if (*abort_flag) continue;
+                        if (__any_sync(0xffffffffu, *abort_flag != 0)) continue;
 #pragma unroll
                         for (int e = 0; e < 32; e += 4)
                             red_add_v4(grow + c + e, __uint_as_float(v[e]), __uint_as_float(v[e + 1]),
@@ -572,7 +572,7 @@ wgrad_acc_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__
         if (lane == 0) {
             int kt = early;
             for (long t = t0 + early; t < t1; ++t, ++kt) {
-                mbar_wait(&empty[kt % kStages], ((kt / kStages) - 1) & 1, ab);
+                if (!mbar_wait(&empty[kt % kStages], ((kt / kStages) - 1) & 1, ab)) break;
                 load_stage(kt, t);
             }
         }
@@ -587,7 +587,7 @@ wgrad_acc_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__
                     mbar_wait(tfree, (flushes - 1) & 1, ab);
                     tcgen05_fence_after();
                 }
-                mbar_wait(&full[s], (kt / kStages) & 1, ab);
+                if (!mbar_wait(&full[s], (kt / kStages) & 1, ab)) break;
                 mbar_wait(&gbfull[cb], (kt >> 1) & 1, ab);
                 tcgen05_fence_after();
                 const uint32_t sA = smem_u32(smem + s * L::kStage), sG = smem_u32(smem + L::oGb + cb * L::kATile);
@@ -655,7 +655,7 @@ wgrad_acc_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__
                         uint32_t v[32];
                         tmem_ld32(tm + lane_addr + half * 256 + c, v);
                         tmem_wait_ld();
-                        if (*abort_flag) continue;
+                        if (__any_sync(0xffffffffu, *abort_flag != 0)) continue;
 #pragma unroll
                         for (int e = 0; e < 32; e += 4)
                             red_add_v4(grow_p + c + e, __uint_as_float(v[e]), __uint_as_float(v[e + 1]),

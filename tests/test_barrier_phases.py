@@ -93,3 +93,55 @@ def test_a_barrier_committed_behind_the_release_is_met_two_phases_late():
     with pytest.raises(AssertionError, match="meets a barrier"):
         for seed in range(2000):
             run(12, random.Random(seed), o_barrier=True)
+
+
+def give_up(rng, loader_stops, issuer_stops, tiles=12, stages=2):
+    """A ring of stages in which some wait runs out although nothing is wrong (the CTA was not scheduled for a while): from then on
+    every wait that is not fulfilled fails at once.  Asserts that no barrier is armed while a load for it is on its way."""
+    full, empty = [0] * stages, [0] * stages      # completed phases
+    on_their_way, late, steps = [], [False], 0
+
+    def wait(bars, s, phase):
+        while bars[s] <= phase and not late[0]:
+            yield
+        return bars[s] > phase
+
+    def loader():
+        for k in range(tiles):
+            if k >= stages and not (yield from wait(empty, k % stages, k // stages - 1)) and loader_stops:
+                return
+            assert k % stages not in on_their_way, "armed twice in one phase"
+            on_their_way.append(k % stages)
+            yield
+
+    def issuer():
+        for k in range(tiles):
+            if not (yield from wait(full, k % stages, k // stages)) and issuer_stops:
+                return
+            empty[k % stages] += 1
+            yield
+
+    roles = [loader(), issuer()]
+    while roles:
+        steps += 1
+        late[0] = late[0] or rng.random() < 0.03
+        if on_their_way and rng.random() < 0.2:
+            full[on_their_way.pop(rng.randrange(len(on_their_way)))] += 1
+        role = rng.choice(roles)
+        try:
+            next(role)
+        except StopIteration:
+            roles.remove(role)
+    assert steps < 2000
+
+
+def test_a_loading_and_an_issuing_thread_that_stop_arm_no_barrier_twice():
+    for seed in range(2000):
+        give_up(random.Random(seed), True, True)
+
+
+@pytest.mark.parametrize("loader_stops,issuer_stops", [(False, False), (True, False), (False, True)])
+def test_one_that_goes_on_arms_a_barrier_twice(loader_stops, issuer_stops):
+    with pytest.raises(AssertionError, match="armed twice"):
+        for seed in range(2000):
+            give_up(random.Random(seed), loader_stops, issuer_stops)
