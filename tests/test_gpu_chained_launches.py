@@ -1,8 +1,10 @@
 """Calls back to back without a synchronisation, sharing workspaces and outputs, on one stream and on two, directly and from a
-captured graph: a kernel that starts while its predecessor runs must not read or overwrite anything early."""
+captured graph: a kernel that starts while its predecessor runs must not read or overwrite anything early.  With four heads every
+CTA has one tile of work; with 130 there are more tiles than SMs, and CTAs take those of others that have not started yet."""
 import pytest
 
 pytestmark = pytest.mark.gpu
+HEADS = [4, 130]
 
 
 def _state(seed, dtype, n, d, h=4):
@@ -19,18 +21,19 @@ def _step(attn, x, out, ws, mask, cfg):
 
 @pytest.mark.parametrize("dtype,n,d,det", [("f32", 100, 64, 0), ("bf16", 320, 64, 1), ("bf16", 320, 128, 1), ("bf16", 331, 64, 1)])
 @pytest.mark.parametrize("how", ["stream", "two_streams", "graph"])
-def test_back_to_back_steps_equal_separate_ones(dtype, n, d, det, how):
+@pytest.mark.parametrize("heads", HEADS)
+def test_back_to_back_steps_equal_separate_ones(dtype, n, d, det, how, heads):
     import torch
     import paper_2410_09397_b200 as attn
     dt = torch.float32 if dtype == "f32" else torch.bfloat16
     cfg, mask = attn.Cfg(deterministic=det), attn.Mask(kind=attn.ATTN_MASK_CAUSAL)      # repeatable: compared bit for bit
     code = attn.ATTN_F32 if dtype == "f32" else attn.ATTN_BF16
-    size = attn.attn_bwd_workspace_bytes(n, d, 4, 1, mask, code, cfg)
-    xs = [_state(90 + i, dt, n, d) for i in range(2)]
+    size = attn.attn_bwd_workspace_bytes(n, d, heads, 1, mask, code, cfg)
+    xs = [_state(90 + i, dt, n, d, heads) for i in range(2)]
 
     def buffers():
         like = xs[0][0]
-        return ([torch.zeros_like(like), torch.zeros(1, 4, n, device="cuda")] + [torch.zeros_like(like) for _ in range(3)],
+        return ([torch.zeros_like(like), torch.zeros(1, heads, n, device="cuda")] + [torch.zeros_like(like) for _ in range(3)],
                 torch.full((size,), 255, dtype=torch.uint8, device="cuda"))     # garbage: the status word too
     want = []
     for x in xs:
@@ -108,7 +111,8 @@ ROUTES = [("fused", 320, 64, "causal", {}), ("fused", 320, 128, "causal", {}), (
 
 @pytest.mark.parametrize("name,n,d,kind,options", ROUTES)
 @pytest.mark.parametrize("how", ["stream", "two_streams", "graph"])
-def test_default_routes_back_to_back_equal_separate_calls(name, n, d, kind, options, how):
+@pytest.mark.parametrize("heads", HEADS)
+def test_default_routes_back_to_back_equal_separate_calls(name, n, d, kind, options, how, heads):
     """Two problems in turn on the same outputs and workspace.  O, LSE, dK and dV have a fixed order of summation and are compared
     bit for bit, dQ within its atomics (exactly where there are none)."""
     import torch
@@ -120,13 +124,13 @@ def test_default_routes_back_to_back_equal_separate_calls(name, n, d, kind, opti
     else:
         cfg = attn.Cfg()
     mask = _mask(attn, kind, n)
-    size = max(attn.attn_fwd_workspace_bytes(n, d, 4, 1, mask, attn.ATTN_BF16, cfg),
-               attn.attn_bwd_workspace_bytes(n, d, 4, 1, mask, attn.ATTN_BF16, cfg))
-    xs = [_state(90 + i, torch.bfloat16, n, d) for i in range(2)]
+    size = max(attn.attn_fwd_workspace_bytes(n, d, heads, 1, mask, attn.ATTN_BF16, cfg),
+               attn.attn_bwd_workspace_bytes(n, d, heads, 1, mask, attn.ATTN_BF16, cfg))
+    xs = [_state(90 + i, torch.bfloat16, n, d, heads) for i in range(2)]
 
     def buffers():
         like = xs[0][0]
-        return ([torch.zeros_like(like), torch.zeros(1, 4, n, device="cuda")] + [torch.zeros_like(like) for _ in range(3)],
+        return ([torch.zeros_like(like), torch.zeros(1, heads, n, device="cuda")] + [torch.zeros_like(like) for _ in range(3)],
                 torch.full((size,), 255, dtype=torch.uint8, device="cuda"))
     want = []
     for x in xs:
@@ -168,14 +172,15 @@ def test_default_routes_back_to_back_equal_separate_calls(name, n, d, kind, opti
 
 @pytest.mark.parametrize("d", [64, 256])
 @pytest.mark.parametrize("how", ["stream", "two_streams", "graph"])
-def test_weights_steps_back_to_back_equal_separate_ones(d, how):
+@pytest.mark.parametrize("h", HEADS)
+def test_weights_steps_back_to_back_equal_separate_ones(d, how, h):
     """Projections, forward and weight gradients of two problems in turn; gX and gY hold garbage before every call."""
     import torch
     import paper_2410_09397_b200 as attn
-    n, h, mask, cfg = 328, 4, attn.Mask(kind=attn.ATTN_MASK_CAUSAL), attn.Cfg()
+    n, mask, cfg = 328, attn.Mask(kind=attn.ATTN_MASK_CAUSAL), attn.Cfg()
     size = max(256, attn.attn_fwd_workspace_bytes(n, d, h, 1, mask, attn.ATTN_BF16, cfg),
                attn.attn_weights_bwd_workspace_bytes(n, d, h, 1, mask, attn.ATTN_BF16, cfg))
-    xs = [_state(190 + i, torch.bfloat16, n, d) for i in range(2)]
+    xs = [_state(190 + i, torch.bfloat16, n, d, h) for i in range(2)]
     g = torch.Generator("cuda").manual_seed(192)
     X, Y = ((torch.randn(h, d, d, device="cuda", generator=g) / d ** 0.5).bfloat16() for _ in range(2))
 

@@ -43,7 +43,7 @@ def test_lists_with_empty_rows_and_columns(block, mask_kind, d, det):
 @pytest.mark.parametrize("n", [8, 136, 1000, 1160, 4104])
 @pytest.mark.parametrize("mask_heads", [1, 2])
 def test_row_lists_of_element_masks(n, mask_heads):
-    """Tiles with a single entry, in their first and last row and column, and rows of tiles without any."""
+    """At most one tile of work a CTA.  Tiles with a single entry, in their first and last row and column, and rows of tiles without any."""
     keep = np.zeros((mask_heads, n, n), dtype=np.uint8)
     for h in range(mask_heads):
         keep[h, 0, n - 1] = keep[h, n - 1, h] = keep[h, n // 2, n // 2] = 1
@@ -52,6 +52,30 @@ def test_row_lists_of_element_masks(n, mask_heads):
             keep[h, n - 8, ::300] = 1
     errs = H.run_case(1, 2, n, 64, "bf16", inputs.MASK_ELEMENT, seed=75, bmask=keep, check_bwd_only=False)
     H.assert_within({name: errs[name] for name in ("O", "LSE", "dV")}, "bf16")     # a row with one key has a dS of zero: nothing to relate an error to
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("mask_kind", [inputs.MASK_BLOCK_SPARSE, inputs.MASK_BLOCK_SPARSE_CAUSAL])
+def test_lists_at_a_length_with_two_terms(block, mask_kind, d):
+    n = 901
+    errs = H.run_case(1, 60, n, d, "bf16", mask_kind, seed=76, block=block, bmask=_holes((n + block - 1) // block), check_bwd_only=False)
+    H.assert_within(errs, "bf16")
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("det", [0, 1])
+@pytest.mark.parametrize("heads,n,mask_heads", [(200, 392, 1), (90, 1160, 1), (90, 392, 90)])
+def test_element_masks(heads, n, mask_heads, d, det):
+    """Several tiles of a CTA whose lists and keep words differ: few keys a row but at least two, tiles that keep none at all."""
+    from paper_2410_09397_b200 import binding as B
+    rng = np.random.default_rng(77)
+    keep = (rng.random((mask_heads, n, n)) < 8 / n).astype(np.uint8)
+    keep[:, :, 128:256] = 0
+    rows = np.arange(n)
+    keep[:, rows, rows % 100] = keep[:, rows, n - 1 - rows % 70] = 1
+    errs = H.run_case(1, heads, n, d, "bf16", inputs.MASK_ELEMENT, seed=77, bmask=keep, cfg=B.Cfg(deterministic=det), check_bwd_only=False)
+    H.assert_within(errs, "bf16")
 
 
 @pytest.mark.parametrize("heads,n,mask_kind", [(300, 72, inputs.MASK_NONE), (90, 328, inputs.MASK_CAUSAL)])
