@@ -272,7 +272,7 @@ mat_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ 
     tmem_leave(tm, kTmemCols, warp, ab);
 }
 
-// phase 3: dS = P o (scale dP - scale D), 8 elements per thread per step
+// phase 3: dS = P o (scale dP - scale D), 8 elements per thread per step; nDs holds -scale D
 __global__ void __launch_bounds__(256) mat_ds_kernel(const uint4 *__restrict__ P, const uint4 *__restrict__ dP,
                                                      uint4 *__restrict__ dS, const float *__restrict__ nDs, size_t nvec,
                                                      int n, float scale)
@@ -420,7 +420,7 @@ size_t mat_onchip_bytes(int, const attn_cfg &c)
 attn_status mat_bwd(const Problem &p)
 {
     if (mask_is_block(p.mask_kind)) return ATTN_ERR_MASK;
-    if (bwd_preprocess_launch(p, false) != ATTN_OK) return ATTN_ERR_LAUNCH;   // Ds = scale D, -LSE log2e
+    if (bwd_preprocess_launch(p, false) != ATTN_OK) return ATTN_ERR_LAUNCH;   // -scale D, -LSE log2e
     for (size_t h0 = 0; h0 < (size_t)p.BH; h0 += p.mat_heads) {
         const int mh = (int)((size_t)p.BH - h0 < (size_t)p.mat_heads ? (size_t)p.BH - h0 : (size_t)p.mat_heads);
         const attn_status st = run_chunk(p, h0, mh);

@@ -19,9 +19,8 @@
 //
 // dQ partial tiles are added into an fp32 accumulator in the workspace with
 // red.global.add (the one place where summation order is not fixed); a small kernel
-// converts it to bf16 at the end.  Tensor memory (512 columns): 128 shared by S^T and
-// dP^T (fused kernel; S^T / P^T in the dK/dV kernel), 128 by P^T and dQ^T (dP^T / dS^T
-// in the dK/dV kernel), dV d, dK d.
+// converts it to bf16 at the end.  Tensor memory (512 columns): 128 take S^T and dP^T in turn (fused kernel, d = 64: S^T
+// alone, dP^T has 128 of its own), 128 take P^T and dQ^T (dK/dV kernel: P^T and dS^T), dV d, dK d.
 //
 // Two kernels: tc_bwd_fused_kernel (all five products, the default) and tc_bwd_dkdv_kernel
 // (without the dQ product; `deterministic = 1`, and lengths that are no multiple of 8, pair it with the
@@ -338,7 +337,7 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
         const int h = warp / 8, qq = (warp / 4) & 1;
         const int row = (warp % 4) * 32 + lane;        // tensor-memory lane = key row inside the tile
         const uint32_t lane_addr = (uint32_t)((warp % 4) * 32) << 16;
-        const float sl2 = a.scale * 1.4426950408889634f;
+        const float sl2 = a.sl2;
         const bool wide = (((uintptr_t)a.dK | (uintptr_t)a.dV) & 31) == 0;
         const uint32_t c0 = h * 64 + qq * 32;          // this thread's first column of S^T / dP^T in region A
         const uint32_t cP = h * 64 + qq * 16;          // of its bf16 pairs of P^T in region B; dS^T 32 columns further
@@ -543,8 +542,8 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
 }
 
 // ---------------------------------------------------------------------------------------
-// The fused kernel.  Every 128-query tile is handled as two halves of 64 queries (every barrier exists
-// once per half).  Warps 0-15: exp / dS (warpgroups 2h and 2h+1 own the two 32-query quarters of half
+// The fused kernel.  The exp / dS warps handle a 128-query tile as two halves of 64 queries (P^T is handed
+// over per half, everything else per tile).  Warps 0-15: exp / dS (warpgroups 2h and 2h+1 own the two 32-query quarters of half
 // h, so each scheduler has four such warps to hide tensor-memory and MUFU latency); warps 16-23:
 // reducers, which do nothing but move finished dQ^T tiles from tensor memory into the fp32
 // accumulator, so that the red.global.add queue stalls them and not the warps on the tile loop;
@@ -558,7 +557,8 @@ tc_bwd_dkdv_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
 //
 //   issuer A:  dP^T(k) -> A  (once S^T(k) has been copied out)  |  S^T(k+1) -> A  (once dP^T(k) has been)
 //   issuer B:  dV += P^T(k) dO  (P^T(k) written in B)  |  dK += dS^T(k) Q, dQ^T(k) -> B  (dS^T(k) in shared
-//              memory, the reducers done with dQ^T(k-1)); dK goes first because it releases the Q / dO stage
+//              memory, the reducers done with dQ^T(k-1)); dK goes first at d = 128, where it releases one of two
+//              Q / dO stages, dQ^T at d = 64
 //
 // The exp / dS warps keep P only as the bf16 pairs they hand to the dV product, and form dS from
 // those, two entries an instruction (fma.rn.f32x2: the roundings of the scalar forms; -scale D comes from the pre-pass).

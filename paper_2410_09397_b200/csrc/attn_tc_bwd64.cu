@@ -262,7 +262,7 @@ tc_bwd_fused64_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_const
         const int row = (warp % 4) * 32 + lane;        // tensor-memory lane = key row inside the tile
         const uint32_t lane_addr = (uint32_t)((warp % 4) * 32) << 16;
         const int jg = j0 + row;
-        const float sl2 = a.scale * 1.4426950408889634f;
+        const float sl2 = a.sl2;
         const uint32_t c0 = g * 32;                    // this thread's columns of S^T / dP^T; its P^T pairs go to c0 .. c0 + 15
         if (L::kVinTmem && T > 0) {
             // V_j -> tensor memory, once: row `row`, bf16 pairs of head-dimension columns 128 g .. 128 g + 127
@@ -416,7 +416,7 @@ attn_status launch_bwd64(const Problem &p)
     a.n = p.n; a.BH = (int)p.BH; a.ns = p.stat_stride;
     a.mask_kind = p.mask_kind; a.block = p.block; a.nb = p.nb; a.mask_heads = p.mask_heads; a.fine = p.fine;
     a.col_ptr = p.col_ptr; a.row_idx = p.row_idx;
-    a.scale = p.scale;
+    a.scale = p.scale; a.sl2 = p.scale * 1.4426950408889634f;
     a.status = p.status;
     a.group = bwd_head_group(p);
     if (bwd_preprocess_launch(p, true) != ATTN_OK) return ATTN_ERR_LAUNCH;

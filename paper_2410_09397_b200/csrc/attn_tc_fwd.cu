@@ -9,7 +9,7 @@
 //   m, l running row maximum / row sum in the exp2 domain; the reference maximum is
 //       only moved (and O rescaled in tensor memory) when the tile maximum exceeds it
 //       by more than 2^8 -- the final LSE does not depend on which reference was used
-//   P   = exp2(S * scale*log2e - m)  -> bf16, written over S in tensor memory
+//   P   = exp2(S * scale*log2e - m)  -> bf16, in tensor memory (columns of its own; d = 256 and the two-term kernels: over S)
 //   O  += P V_j                      A = P from tensor memory, B = V_j MN-major
 //
 // Four kernels.  tc_fwd_flow_kernel (d = 64, 128): a thread holds a whole row of scores, S has buffers of its own that
@@ -1469,8 +1469,8 @@ tc_fwd_flow_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant
 }
 
 // Heads that are launched together.  Under a causal mask the query tiles of a group start longest first; head after head the
-// last head's longest tile started when the grid was nearly done, and SMs were busy 85 % of the launch (32 heads, n = 8192,
-// d = 128: 551 us so, 489 us in groups).  The group's K and V should stay in L2 while its tiles run.
+// last head's longest tile starts when the grid is nearly done (d = 128, 32 heads, n = 8192 461 us so, 426 us in groups; 16 heads,
+// n = 4096 95 and 66).  The group's K and V should stay in L2 while its tiles run.
 int fwd_head_group(const Problem &p)
 {
     constexpr size_t kBudget = 40u << 20;
@@ -1480,14 +1480,20 @@ int fwd_head_group(const Problem &p)
     return 1;
 }
 
-// 256 queries per CTA or 128.  A pair of query tiles takes 0.87 of the time of two CTAs one after the other, and half as many
-// CTAs pay for set-up and drain, but one CTA alone walks a row of key tiles 1.75 times as slowly: it pays as soon as the pairs
-// occupy half of the SMs (their halves would take more than one wave), under a causal mask when the SMs' average share of
-// tiles exceeds the longest row that much, BH (T + 1) / 2 / 148 >= 1.7 for T tiles.  Measured, pairs / single tiles in us:
-// causal d = 128, 32 heads, n = 4096 148 / 171; 16 heads, n = 2048 (BH (T + 1) = 272) 42 / 33; d = 64, 32 heads, n = 1000 (288)
-// 23.9 / 23.7; 8 heads, n = 8192 (520) 119 / 122; no mask, 8 heads, n = 4096 72 / 82; 16 heads, n = 1269 40 / 44.
+// 256 queries per CTA or 128.  A pair of query tiles shares its key tiles, but takes 1.7 (d = 128) to 1.9 times (d = 64, two
+// terms) as long as one of them: it pays where the SMs have several units each, not where the halves of the pairs would fill a
+// last wave that the pairs leave half empty.  The line: pairs that occupy half of the SMs, under a causal mask an average share
+// of the SMs that exceeds the longest row 1.7 times, BH (T + 1) / 2 / 148 >= 1.7 for T tiles.  It was drawn with kernels of a CTA
+// per unit; the kernels as they are, pairs / single tiles in us (calls back to back):
+//   chosen for pairs    causal d = 128: 32 heads, n = 8192 439 / 536; 32 heads, n = 4096 122 / 136; 12 heads, n = 8192 211 / 186
+//                       causal d = 64: 64 heads, n = 8192 760 / 831; 24 heads, n = 3000 67 / 59
+//                       no mask: d = 128, 32 heads, n = 4096 231 / 238; d = 64, 64 heads, n = 2048 115 / 117; 6 heads, n = 8192 223 / 174
+//                       two terms, d = 128: 32 heads, n = 8191, causal 776 / 822; 12 heads, n = 4095, no mask 207 / 159
+//   chosen for single   causal d = 128: 16 heads, n = 2048 35 / 26; 40 heads, n = 1000 23 / 28; no mask, 16 heads, n = 1000 22 / 16
+// Over 1,361 such points (d = 64 and 128, both masks, 1 to 128 heads, n = 512 to 16384) the choice is 1.5 to 2.5 % slower than the
+// better one on average, 2.0 to 4.4 % with two terms, and at most 41 %.
 // Not where results have to be repeatable: the two shapes differ in the last bits, and a head's result must not depend on how
-// many others are in the call (24 heads, n = 3000, d = 64, no mask, whole step: 422 us, 434 so).
+// many others are in the call (24 heads, n = 3000, d = 64, no mask: 91 us, 97 so).
 bool pair_pays(const Problem &p)
 {
     if (p.cfg.deterministic) return false;
